@@ -300,3 +300,56 @@ def tolerance(case):
     if case["kind"] in ("decode", "assign"):
         return "exact"
     return {"rel": 1.3e-3, "max": 5e-3}
+
+
+def _weights64(fmt, idx, cb, scale, r0, r1, norm=None):
+    """Rows r0..r1-1 of the weight matrix in binary64, unrounded: entry, times the block's or row group's scale,
+    times the sub-row's scale under normalisation."""
+    n, k, d, b, br, bc = fmt.n_rows, fmt.k_cols, fmt.vq_dim, fmt.index_bits, fmt.block_rows, fmt.block_cols
+    dev = idx.device
+    bit = torch.arange(k // d, device=dev) * b   # index j: bits j*b .. j*b + b - 1, least significant first
+    rows = torch.nn.functional.pad(idx[r0:r1], (0, 1)).short()
+    e = ((rows[:, bit // 8] | (rows[:, bit // 8 + 1] << 8)).int() & 0xFFFF) >> (bit % 8).int() & ((1 << b) - 1)
+    blk = torch.arange(r0, r1, device=dev)[:, None] // br * (k // bc) + (torch.arange(k // d, device=dev) * d // bc)[None, :]
+    if fmt.cb_type == INT4:
+        raw = cb.reshape(-1)
+        nib = torch.stack((raw & 15, raw >> 4), 1).reshape(-1).double()
+        entries = torch.where(nib >= 8, nib - 16, nib)
+    else:
+        entries = cb.reshape(-1).double()
+    w = entries.reshape(-1, d)[blk * (1 << b) + e]   # [rows, K/d, d]
+    if fmt.cb_type == INT8:
+        w = w * scale.double()[blk][..., None]
+    w = w.reshape(r1 - r0, k)
+    if fmt.cb_type == INT4:
+        w = w * scale[r0:r1].double().repeat_interleave(128, 1)
+    if norm:
+        codes, lut, cols = norm
+        codes = codes.reshape(n, -1)[r0:r1]
+        code = torch.stack((codes & 15, codes >> 4), 2).reshape(r1 - r0, -1)[:, : k // cols].long()
+        block = torch.arange(r0, r1, device=dev)[:, None] // br * (k // bc) + (torch.arange(k // cols, device=dev) * cols // bc)[None, :]
+        w = w * lut.double()[block * 16 + code].repeat_interleave(cols, 1)
+    return w
+
+
+def _product64(fmt, idx, cb, scale, x, norm=None):
+    x = x.cuda().double()
+    step = max(1, (1 << 24) // fmt.k_cols)
+    return torch.cat([x @ _weights64(fmt, idx, cb, scale, r, min(r + step, fmt.n_rows), norm).T for r in range(0, fmt.n_rows, step)], 1)
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, in binary64 from the stored bytes (index streams have no such value)."""
+    kind = case["kind"]
+    if kind == "assign":
+        return None
+    s = prepare({**case, "graph": False}, seed)
+    if kind in ("layers", "host"):
+        return [_product64(_fmt(case, n, k), idx, cb, scale, x)
+                for (k, _), (_, members, x, _) in zip(_calls(case), s["calls"]) for idx, cb, scale, _, n in members]
+    norm = (s["codes"], s["lut"], s["norm"]) if s["norm"] else None
+    if kind == "linear":
+        return _product64(s["fmt"], s["idx"], s["cb"], s["scale"], s["x"], norm)
+    step = max(1, (1 << 24) // s["fmt"].k_cols)
+    return torch.cat([_weights64(s["fmt"], s["idx"], s["cb"], s["scale"], r, min(r + step, s["fmt"].n_rows), norm)
+                      for r in range(0, s["fmt"].n_rows, step)], 0)
