@@ -1309,9 +1309,12 @@ vq_status launch(const StreamCall& call, int chunks_per_block, cudaStream_t s, i
   const size_t ticket_bytes = stream_ticket_bytes(rows_total);
   if (static_cast<size_t>(slabs) * sizeof(int) > ticket_bytes) return VQ_ERR_UNSUPPORTED;
   const size_t part_ws = static_cast<size_t>(Pn) * 2 * slab_rows * batch * sizeof(float);
-  if (!call.ws || call.ws_bytes < ticket_bytes + part_ws) return VQ_ERR_WORKSPACE;
+  // ... and they lie at the end of what this call may use: right behind its counters a call with few rows wrote sums
+  // where a call with more rows on the same workspace keeps its counters
+  const size_t total_ws = stream_workspace_bytes(rows_total, batch);
+  if (!call.ws || call.ws_bytes < total_ws || ticket_bytes + part_ws > total_ws) return VQ_ERR_WORKSPACE;
   a.ws_ticket = static_cast<int*>(call.ws);
-  a.ws_part = reinterpret_cast<float*>(static_cast<char*>(call.ws) + ticket_bytes);
+  a.ws_part = reinterpret_cast<float*>(static_cast<char*>(call.ws) + (total_ws - part_ws));
 
   // ---- tensor maps ----
   Maps maps;
