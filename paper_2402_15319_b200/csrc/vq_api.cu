@@ -195,6 +195,7 @@ static int group_family(const Geometry& g, int) {
 int vq_grouped_kernel_launches(const vq_format* fmt, int n_members, int batch) {
   Geometry g;
   if (make_geometry(fmt, &g) != VQ_OK || n_members < 1 || n_members > VQ_MAX_GROUP || batch < 1 || batch > 16) return 0;
+  if (n_members > 1 && tile_preferred(g, &g.N, 1, batch)) return 1;   // (g.N: the members' rows together)
   if (n_members > 1 && blockcb_covers(g) && group_family(g, batch) == 2) return 1;
   if (n_members > 1 && group_family(g, batch) == 3) return 1;
   return (n_members > 1 && group_family(g, batch) == 1 && stream_covers(g)) ? 1 : n_members;
@@ -238,6 +239,8 @@ vq_status vq_gemm_small_batch_grouped(const vq_format* fmt, const vq_group_membe
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   vq_status st = VQ_ERR_UNSUPPORTED;
   if (n_members > 1) {
+    if (tile_preferred(call.g, call.N, n_members, batch)) st = launch_gemm_tile(call, s);
+    if (st != VQ_ERR_UNSUPPORTED) return st;
     int fam = group_family(call.g, batch);
 #ifdef VQ_TUNING
     if (getenv("VQ_GROUP_FAMILY")) fam = atoi(getenv("VQ_GROUP_FAMILY"));

@@ -66,6 +66,11 @@ vq_status launch_gemm_stream(const StreamCall& call, cudaStream_t s);
 bool stream_covers(const Geometry& g);
 vq_status launch_int4g128_stream(int N, int K, const uint8_t* q, const __half* scale, const __half* X, __half* Y, int batch,
                                  void* ws, size_t ws_bytes, cudaStream_t s);
+// tcgen05 kernel (vq_tile.cu): rows per layer in call.N; needs the workspace.  covers: the formats it takes;
+// preferred: the calls it serves.
+vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s);
+bool tile_covers(const Geometry& g);
+bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch);
 vq_status launch_gemm_blockcb(const Geometry& g, const LayerPtrs& p, const __half* X, __half* Y, int batch,
                               cudaStream_t s);
 // The same kernels over several layers of one format and K in one launch (rows per layer in call.N;
@@ -112,7 +117,7 @@ vq_status encode_index_map(CUtensorMap* tm, const uint8_t* idx, long long stride
                            bool swizzle128 = false);
 
 // General tiled tensor map (loads with it always target the issuing CTA alone): elements of 1 or 2 bytes, rank <= 5,
-// dims / box in elements, strides of dimensions 1.. in bytes; swizzle 0 none, 1 64-byte, 2 128-byte.
+// dims / box in elements, strides of dimensions 1.. in bytes; swizzle 0 none, 1 64-byte, 2 128-byte, 3 32-byte.
 vq_status encode_tensor_map(CUtensorMap* tm, const void* base, int elem_bytes, int rank, const uint64_t* dims,
                             const uint64_t* strides, const uint32_t* box, int swizzle);
 

@@ -1,0 +1,982 @@
+// Skinny GEMM on the 5th-generation tensor cores: decoded weights go to tensor memory as the A operand of
+// tcgen05.mma (M = 128 weight rows, N = 16 batch rows), so one pass over the weights serves 1 to 16
+// sequences (paper Sec. 3.2: packed indices -> look-up table -> product).
+//
+// What bounds it.  Every pair of weights costs one 32-bit shared-memory gather, 32 of them a clock and SM: 64
+// weights / clk / SM at most.  So everything else is kept off the shared-memory port and out of the gathering warps:
+// activations are never loaded by a warp (the tensor core reads them from shared memory as the B operand), the
+// decoded tile goes from registers to tensor memory by tcgen05.st, which has its own path (gathers alone ran at
+// 63.0 weights / clk / SM in a probe on resident data, with the stores 60.7, with the products 48.4), and the
+// accumulators live in tensor memory, which leaves registers for 16 gathering warps per SM.
+//
+// Work.  The rows of a call's layers ("segments") are cut into tiles of 128 rows, a tile's columns into units of
+// UC.  The grid is persistent, four CTAs per SM at most; every CTA takes q whole tiles, and the units
+// of the tiles left over form one sequence that is cut into equal contiguous pieces, one per CTA.  A CTA walks its
+// piece first, so that shared tiles are summed while everyone still computes whole ones.
+//
+// Roles (192 threads).  Warps 0..3 decode: thread = weight row = lane of tensor memory.  A thread reads its row's
+// indices of a unit from the stage the producer filled, looks up 32 pairs (64 columns) and stores them as
+// 32 columns of tensor memory; three such stages are in flight.  Warp 4 (one thread) produces: index and
+// activation boxes by TMA; index boxes run ahead of the programmatic-dependency wait, activations come after it.
+// Warp 5 issues the products (one elected lane, warp-uniform control flow: with a divergent branch in place of
+// elect.sync an issue took five times as long) and owns the tensor memory.
+//
+// Tables.  One 32-bit word per entry and lane, bank = lane: no conflicts whatever the indices.  Three kinds:
+//   row  : 16 entries of the lane's own row, two tables per warp (256-byte entry pitch), so that the index byte
+//          enters the address by one byte permute and the next block's table is written beside the current one;
+//   warp : blocks of 4, 8, 16 or a multiple of 32 rows, every warp replicates its own rows' codebooks;
+//   CTA  : blocks of a multiple of 128 rows, one table for the four warps.
+// 8-bit codebooks with row tables keep the entries as exact integers in fp16 and multiply the fp32 sums of a block by its
+// scale; the other tables hold fp16(scale * c), the value vq_decode_weights writes.  4-bit codebooks multiply
+// the looked-up pair by the scale of the row and its group of 128 columns, the same value again.
+//
+// Sums.  A tile whose units all belong to one CTA is rounded to fp16 and stored.  A shared tile's parts go to the
+// workspace; the CTA that draws the tile's last ticket adds them in CTA order (results do not depend on
+// timing) and resets the counter.
+//
+// Every wait is bounded; a wait that runs out increments a device counter, the role stops waiting for anything
+// else and still arrives on every barrier it owes, so that the kernel ends.
+#include <cstdio>
+#include <cstdlib>
+#include <type_traits>
+#include <utility>
+
+#include "vq_common.cuh"
+#include "vq_device.cuh"
+
+namespace vq {
+namespace {
+
+using namespace dev;
+
+constexpr int kTileRows = 128;
+constexpr int kStageCols = 64;        // columns a thread decodes between two hand-overs to the tensor core
+constexpr int kStageTmem = 32;        // ... and the tensor-memory columns they take
+constexpr int kAStages = 3;           // decoded stages in tensor memory
+constexpr int kTmemCols = 128;        // 2 x 16 accumulator columns, 3 x 32 weight columns
+constexpr int kAOff = 32;
+constexpr int kDecodeWarps = 4, kThreads = 192;
+constexpr int kMaxDepth = 6;          // unit stages at most
+constexpr int kWaitTries = 1 << 18;
+constexpr int kPolls = 1 << 20;       // polls without progress before the producer gives up
+constexpr unsigned kPollSleep = 500;  // ns between polls of the producer
+constexpr uint32_t kMagic = 0x64646464u;   // high byte of fp16 1024.0
+constexpr uint32_t kBias2 = 0x64806480u;   // fp16 pair (1152, 1152)
+// tcgen05.mma kind::f16: D fp32, A and B fp16, both K-major, N = 16, M = 128
+constexpr uint32_t kIdesc = (1u << 4) | ((16u / 8) << 17) | ((128u / 16) << 24);
+
+enum TableKind { kRow = 0, kWarp = 1, kCta = 2 };
+
+struct Segment {
+  const void* cb;
+  const __half* scale;
+  __half* Y;
+  int N;
+  int tile0;   // first tile of the segment in the call's tile sequence
+};
+
+struct TileArgs {
+  Segment seg[kMaxSegments];
+  int n_seg;
+  float* ws_part;     // [CTA][2][batch][128] partial sums
+  int* ws_ticket;     // [tile], zero between calls
+  int* error_flag;
+  int K, batch;
+  int S;              // units per tile
+  int q;              // whole tiles per CTA
+  int tail_units, tail_ctas;   // units of the left-over tiles and the CTAs that share them
+  int blocks_per_row, Br, Bc, cb_int8;
+  int D;              // unit stages
+  int x_bytes, x_row_bytes;    // activation stage; bytes of one 64-column group of it
+  int idx_off, bar_off, front_bytes;   // dynamic shared memory: x stages, index stages, barriers, | tables
+};
+
+struct TileMaps {
+  CUtensorMap idx[kMaxSegments];
+  CUtensorMap x;
+};
+
+// Format policy: D columns per entry, B index bits; BR: rows that share a table word inside a warp (kWarp).
+template <int D_, int B_, int TK_, int BR_, bool I4_>
+struct Fmt {
+  static constexpr int D = D_, B = B_, TK = TK_, BR = BR_;
+  static constexpr bool I4 = I4_;
+  static constexpr int E = 1 << B;
+  // Columns of a unit: 256 where a row of 128 is no whole number of 16-byte pieces (5 bits) and for row tables (half as
+  // many unit changes: 69.5 against 73.6 us on 57344 x 8192 at batch 16), else 128 (more stages in flight).
+  static constexpr int UC = TK == kRow || (128 * B / (8 * D)) % 16 != 0 ? 256 : 128;
+  static constexpr int RB = UC * B / (8 * D);       // bytes of a row of a unit
+  static constexpr int IDX_BYTES = kTileRows * RB;
+  static constexpr int STAGES = UC / kStageCols;
+  static constexpr int WPS = 2 * B / D;              // index words per stage
+  static constexpr int TABLE = TK == kRow ? 4096 : E * 128;              // bytes of a warp's (CTA's) table
+  static constexpr int BUFS = TK == kCta && D == 2 ? 2 : 1;
+  static constexpr int TABLES = TK == kCta ? BUFS * TABLE : kDecodeWarps * TABLE;
+  // OR-merged addresses need tables on multiples of their size; 4-D look-ups add (one per four weights)
+  static constexpr int ALIGN = D == 4 ? 1024 : TABLE;
+  static constexpr int SWIZZLE = RB == 32 ? 3 : RB == 64 ? 1 : RB == 128 ? 2 : 0;
+  static_assert(RB % 16 == 0 && (TK != kRow || (B == 4 && D == 2)));
+};
+
+// ---- small device helpers ------------------------------------------------------------------------------------
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {   // has phase `parity` completed?
+  uint32_t done;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+  return done != 0;
+}
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {   // the same, blocking for a short time
+  uint32_t done;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+  return done != 0;
+}
+// Bounded wait for phase `parity`; `tries` is the role's budget: 0 once a wait has run out, so that later ones return at once.
+__device__ __forceinline__ void wait_phase(uint32_t bar, uint32_t parity, int& tries, int* error_flag) {
+  if (mbar_try(bar, parity)) return;
+#pragma unroll 1
+  for (int i = 0; !mbar_try(bar, parity);) {
+    if (++i >= tries) {
+      if (tries && (threadIdx.x & 31) == 0) atomicAdd(error_flag, 1);
+      tries = 0;
+      break;
+    }
+  }
+}
+__device__ __forceinline__ void decode_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }   // the four decoding warps
+__device__ __forceinline__ void tma_box_3d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, uint32_t bar) {
+  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+               ::"r"(dst), "l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* tm) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// D[128 x 16] (+)= A[128 x 16] (tensor memory) * B[16 x 16] (shared memory)
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a, uint64_t b_desc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+               ::"r"(d), "r"(a), "l"(b_desc), "r"(kIdesc), "r"(accumulate) : "memory");
+}
+// B operand, K-major rows of 128 bytes with the 128-byte swizzle, 8 rows (batch) per 1024-byte group
+__device__ __forceinline__ uint64_t b_descriptor(uint32_t addr) {
+  return (static_cast<uint64_t>(addr >> 4) & 0x3FFF) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+}
+__device__ __forceinline__ void tc_store32(uint32_t addr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,"
+      "%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
+      ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
+        "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]),
+        "r"(r[30]), "r"(r[31])
+      : "memory");
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+template <int NB>   // NB accumulator columns of the thread's row
+__device__ __forceinline__ void tc_load(uint32_t addr, float (&v)[NB]) {
+  uint32_t r[NB];
+  if constexpr (NB == 8) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr) : "memory");
+  } else {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                   "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(addr) : "memory");
+  }
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < NB; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t mul_f16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t int8_pair(uint32_t biased, uint32_t sel) {   // (u, u') - 128 as fp16, exact
+  uint32_t r;
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(prmt(biased, kMagic, sel)), "r"(kBias2));
+  return r;
+}
+__device__ __forceinline__ uint32_t scaled_pair(float s, uint32_t two) {   // fp16(s * c0), fp16(s * c1): exact products, one rounding
+  const __half2 h = __floats2half2_rn(s * static_cast<float>(static_cast<int8_t>(two & 0xffu)),
+                                      s * static_cast<float>(static_cast<int8_t>((two >> 8) & 0xffu)));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ uint32_t nibble_pair(uint32_t byte) {   // two signed 4-bit integers as fp16, exact
+  const __half2 h = __floats2half2_rn(static_cast<float>(static_cast<int>(byte << 28) >> 28), static_cast<float>(static_cast<int>(byte << 24) >> 28));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// A CTA's walk over its units: its piece of the left-over tiles first, then its q whole tiles.
+struct Walk {
+  int n, n_tail, t0, t1, slab, s, k, whole0, tail_tile0;
+
+  __device__ __forceinline__ void init(const TileArgs& a, int c, int ctas) {
+    t0 = t1 = 0;
+    if (c < a.tail_ctas) {   // (the host keeps tail_units * tail_ctas below 2^31)
+      t0 = static_cast<int>(static_cast<unsigned>(a.tail_units) * static_cast<unsigned>(c) / static_cast<unsigned>(a.tail_ctas));
+      t1 = static_cast<int>(static_cast<unsigned>(a.tail_units) * static_cast<unsigned>(c + 1) / static_cast<unsigned>(a.tail_ctas));
+    }
+    n_tail = t1 - t0;
+    n = n_tail + a.q * a.S;
+    whole0 = c * a.q;
+    tail_tile0 = a.q * ctas;
+    k = 0;
+    slab = whole0;
+    s = 0;
+    if (n_tail > 0) {
+      slab = tail_tile0 + t0 / a.S;
+      s = t0 % a.S;
+    }
+  }
+  __device__ __forceinline__ void next(const TileArgs& a) {
+    ++k;
+    if (k == n_tail) {
+      slab = whole0;
+      s = 0;
+    } else if (++s == a.S) {
+      s = 0;
+      ++slab;
+    }
+  }
+  __device__ __forceinline__ bool slab_end(const TileArgs& a) const { return s == a.S - 1 || k == n_tail - 1; }
+  __device__ __forceinline__ int fragment_units(const TileArgs& a) const {   // of the current tile, from here on
+    return k < n_tail ? min(n_tail - k, a.S - s) : a.S - s;
+  }
+  __device__ __forceinline__ bool complete(const TileArgs& a) const {   // does this CTA hold every unit of the tile?
+    if (k >= n_tail) return true;
+    const int first = (slab - tail_tile0) * a.S;
+    return first >= t0 && first + a.S <= t1;
+  }
+};
+
+__device__ __forceinline__ int segment_of(const TileArgs& a, int slab) {
+  int g = 0;
+#pragma unroll
+  for (int i = 1; i < kMaxSegments; ++i)
+    if (i < a.n_seg && slab >= a.seg[i].tile0) g = i;
+  return g;
+}
+
+// ---- look-up tables: request a block's entries (registers), write them as table words --------------------------
+template <class F>
+struct Tables {
+  // entries one lane requests: the whole codebook of its row (row), E / BR of one of the warp's codebooks (warp), or
+  // its share of the CTA's codebook: one entry of a 2-D one (two or four threads each), 2 of a 4-D one
+  static constexpr int EPL = F::TK == kRow ? 16 : F::TK == kWarp ? (F::E / F::BR) : (F::D == 4 ? 2 : 1);
+  static constexpr int VALS = EPL * F::D;                 // values requested
+  static constexpr int RAW = F::I4 ? (VALS + 7) / 8 : (VALS + 1) / 2;   // registers (fp16; 8-bit entries use half of them)
+  uint32_t raw[RAW];
+  uint32_t sc;                 // the block's scale (8-bit codebooks)
+  const uint8_t* src;          // this lane's share in block column 0 of the current fragment's block row
+  const unsigned short* ssrc;
+
+  __device__ __forceinline__ void open(const TileArgs& a, const Segment& sg, int row0, int tid) {   // a fragment's rows
+    const int lane = tid & 31, warp = tid >> 5;
+    int brow, part;
+    if constexpr (F::TK == kRow) {
+      brow = min(row0 + tid, sg.N - 1) / a.Br;
+      part = 0;
+    } else if constexpr (F::TK == kWarp) {
+      const int r = row0 + 32 * warp + (F::BR < 32 ? (lane % (32 / F::BR)) * F::BR : 0);
+      brow = min(r, sg.N - 1) / a.Br;
+      part = lane / (32 / F::BR) * EPL;
+    } else {
+      brow = row0 / a.Br;
+      part = F::D == 4 ? 2 * tid : tid % F::E;
+    }
+    const long long blk = static_cast<long long>(brow) * a.blocks_per_row;
+    const int bits = F::I4 ? 4 : a.cb_int8 ? 8 : 16;
+    src = static_cast<const uint8_t*>(sg.cb) + (blk * F::E + part) * F::D * bits / 8;
+    ssrc = reinterpret_cast<const unsigned short*>(sg.scale) + blk;
+  }
+  __device__ __forceinline__ void request(const TileArgs& a, int bcol) {
+    const int bits = F::I4 ? 4 : a.cb_int8 ? 8 : 16;
+    const uint8_t* p = src + static_cast<long long>(bcol) * (F::E * F::D * bits / 8);
+    if constexpr (F::I4) {
+      load<VALS / 2>(p);
+    } else if (a.cb_int8) {
+      load<VALS>(p);
+      sc = __ldg(ssrc + bcol);
+    } else {
+      load<VALS * 2>(p);
+    }
+  }
+  template <int BYTES>
+  __device__ __forceinline__ void load(const uint8_t* p) {
+    if constexpr (BYTES == 1) raw[0] = __ldg(p);
+    else if constexpr (BYTES == 2) raw[0] = __ldg(reinterpret_cast<const unsigned short*>(p));
+    else if constexpr (BYTES == 4) raw[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+    else if constexpr (BYTES == 8) {
+      const uint2 v = ldg64_nc(p);
+      raw[0] = v.x; raw[1] = v.y;
+    } else {
+#pragma unroll
+      for (int i = 0; i < BYTES / 16; ++i) {
+        const uint4 v = ldg128_nc(p + 16 * i);
+        raw[4 * i] = v.x; raw[4 * i + 1] = v.y; raw[4 * i + 2] = v.z; raw[4 * i + 3] = v.w;
+      }
+    }
+  }
+  __device__ __forceinline__ float scale() const { return __half2float(__ushort_as_half(static_cast<unsigned short>(sc))); }
+  // 2-D: pair i of the requested ones as a table word
+  template <bool EXACT>
+  __device__ __forceinline__ uint32_t word(const TileArgs& a, int i, float s) const {
+    if constexpr (F::I4) return nibble_pair((raw[i >> 2] >> (8 * (i & 3))) & 0xffu);
+    else if (!a.cb_int8) return raw[i];
+    else if constexpr (EXACT) return int8_pair(raw[i >> 1] ^ 0x80808080u, (i & 1) ? 0x4342u : 0x4140u);
+    else return scaled_pair(s, raw[i >> 1] >> (16 * (i & 1)));
+  }
+  // tbl: shared address of the warp's (CTA's) table, row kind: + the half
+  __device__ __forceinline__ void write(const TileArgs& a, uint32_t tbl, int tid) const {
+    const int lane = tid & 31;
+    const float s = !F::I4 && a.cb_int8 ? scale() : 1.f;
+    if constexpr (F::TK == kRow) {
+#pragma unroll
+      for (int i = 0; i < EPL; ++i) sts32(tbl + i * 256 + lane * 4, word<true>(a, i, s));
+    } else if constexpr (F::TK == kWarp) {
+      // replicated over the rows of the block by 128-bit stores; the order of the 16-byte groups is rotated so that a
+      // quarter warp writes 8 different ones
+      constexpr int G = F::BR / 4, NCB = 32 / F::BR;   // 16-byte groups per codebook, codebooks of the warp
+      const int c = lane % NCB, part = lane / NCB;
+#pragma unroll
+      for (int i = 0; i < EPL; ++i) {
+        const uint32_t w = word<false>(a, i, s);
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+          sts128(tbl + (part * EPL + i) * 128 + (c * G + ((u + part) & (G - 1))) * 16, make_uint4(w, w, w, w));
+      }
+    } else if constexpr (F::D == 2) {
+      constexpr int SHARE = 8 * F::E / 128;   // 16-byte groups per thread
+      const uint32_t w = word<false>(a, 0, s);
+      const int e = tid % F::E, h = tid / F::E;
+#pragma unroll
+      for (int i = 0; i < SHARE; ++i) sts128(tbl + e * 128 + ((lane + i + SHARE * h) & 7) * 16, make_uint4(w, w, w, w));
+    } else {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const uint32_t w0 = word<false>(a, 2 * i, s), w1 = word<false>(a, 2 * i + 1, s);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) sts128(tbl + (2 * tid + i) * 128 + ((lane + u) & 7) * 16, make_uint4(w0, w1, w0, w1));
+      }
+    }
+  }
+};
+
+// (index I of the stage's words) << 7, for tables of 128-byte entries
+template <int B, int I, int NW>
+__device__ __forceinline__ uint32_t entry_off(const uint32_t (&w)[NW]) {
+  constexpr uint32_t MASK = ((1u << B) - 1u) << 7;
+  constexpr int p = B * I, wi = p >> 5, s = p & 31;
+  if constexpr (s + B > 32) return __funnelshift_r(w[wi], w[wi + 1], s - 7) & MASK;   // (s >= 25 here)
+  else if constexpr (s < 7) return (w[wi] << (7 - s)) & MASK;
+  else return (w[wi] >> (s - 7)) & MASK;
+}
+
+// 64 columns of the thread's row, stage J of a unit's words -> 32 fp16 pairs
+template <class F, int J>
+__device__ __forceinline__ void gather(uint32_t (&r)[32], const uint32_t (&w)[F::RB / 4], uint32_t tbl, uint32_t pat) {
+  if constexpr (F::TK == kRow) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t even = (w[4 * J + j] & 0x0F0F0F0Fu) | pat, odd = ((w[4 * J + j] >> 4) & 0x0F0F0F0Fu) | pat;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        r[8 * j + 2 * i] = lds32(prmt(tbl, even, 0x3200u | ((4u + i) << 4)));
+        r[8 * j + 2 * i + 1] = lds32(prmt(tbl, odd, 0x3200u | ((4u + i) << 4)));
+      }
+    }
+  } else if constexpr (F::D == 2) {
+    [&]<int... I>(std::integer_sequence<int, I...>) {
+      ((r[I] = lds32(entry_off<F::B, 32 * J + I>(w) | tbl)), ...);
+    }(std::make_integer_sequence<int, 32>{});
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t e = prmt(w[4 * J + (i >> 2)], 0u, 0x4440u | (i & 3));
+      const uint2 v = lds64(e * 128u + tbl);
+      r[2 * i] = v.x;
+      r[2 * i + 1] = v.y;
+    }
+  }
+}
+
+template <class F, int NB>
+__global__ void __launch_bounds__(kThreads, 4) tile_kernel(const __grid_constant__ TileMaps maps, const TileArgs a) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  const uint32_t tables = (base + a.front_bytes + F::ALIGN - 1) & ~static_cast<uint32_t>(F::ALIGN - 1);
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  {   // the host planned for dynamic shared memory that starts 1024 bytes into the CTA's window
+    uint32_t dyn;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+    if (tables + F::TABLES - raw > dyn) {   // (the same for every thread)
+      if (tid == 0) atomicAdd(a.error_flag, 1);
+      return;
+    }
+  }
+  const int D = a.D;
+  const uint32_t idx_full = base + a.bar_off, idx_empty = idx_full + 8 * kMaxDepth, x_full = idx_empty + 8 * kMaxDepth,
+                 x_empty = x_full + 8 * kMaxDepth, a_full = x_empty + 8 * kMaxDepth, a_empty = a_full + 8 * kAStages,
+                 d_full = a_empty + 8 * kAStages, tmem_slot = d_full + 16, last_slot = tmem_slot + 4;
+  if (warp == 4 && lane == 0) {
+    for (int i = 0; i < D; ++i) {
+      mbar_init(idx_full + 8 * i, 1);
+      mbar_init(idx_empty + 8 * i, kDecodeWarps);
+      mbar_init(x_full + 8 * i, 1);
+      mbar_init(x_empty + 8 * i, 1);
+    }
+    for (int i = 0; i < kAStages; ++i) {
+      mbar_init(a_full + 8 * i, kDecodeWarps);
+      mbar_init(a_empty + 8 * i, 1);
+    }
+    mbar_init(d_full, 1);
+    mbar_init(d_full + 8, 1);
+    mbar_init_fence();
+  }
+  if (warp == 5) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "n"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  uint32_t tmem;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(tmem_slot) : "memory");
+  // (after the allocation: a CTA that waits for tensor memory only ever waits for CTAs that have theirs)
+  pdl_launch_dependents();
+
+  const int c = blockIdx.x;
+  Walk wk;
+  wk.init(a, c, gridDim.x);
+  constexpr bool kExact = F::TK == kRow && !F::I4;   // 8-bit row tables hold unscaled entries: sums are scaled per block
+  const bool by_block = kExact && a.cb_int8;
+  const int block_units = by_block ? a.Bc / F::UC : 1;
+
+  if (warp == 4) {
+    // ---- producer ------------------------------------------------------------------------------------------
+    if (lane == 0) {
+      prefetch_tensormap(&maps.x);
+      for (int i = 0; i < a.n_seg; ++i) prefetch_tensormap(&maps.idx[i]);
+      // Index and activation boxes in two independent sequences, each as far ahead as its own stages allow: one
+      // thread polls both (in one sequence the activations of a unit were requested only when the unit before it had been
+      // read, and their latency showed in every unit).
+      Walk wi = wk;
+      int slot_i = 0, slot_x = 0, idle = 0;
+      uint32_t ph_i = 1, ph_x = 1;   // parity of the empty barriers: the first D polls succeed at once
+      bool started = false;
+      while (wk.k < wk.n && idle < kPolls) {
+        if (++idle > 1) __nanosleep(kPollSleep);   // (polls without a pause take issue slots from the decoding warps)
+        if (wi.k < wi.n && mbar_test(idx_empty + 8 * slot_i, ph_i)) {
+          const int g = segment_of(a, wi.slab);
+          mbar_arrive_expect_tx(idx_full + 8 * slot_i, F::IDX_BYTES);
+          tma_box_2d(base + a.idx_off + slot_i * F::IDX_BYTES, &maps.idx[g], wi.s * F::RB, (wi.slab - a.seg[g].tile0) * kTileRows,
+                     idx_full + 8 * slot_i);
+          if (++slot_i == D) { slot_i = 0; ph_i ^= 1u; }
+          wi.next(a);
+          idle = 0;
+        }
+        if (!started && wi.k < min(D, wi.n)) continue;   // weights first: they do not depend on the previous kernel
+        if (!started) {
+          pdl_wait();   // the activations belong to the previous kernel of the stream until here
+          started = true;
+        }
+        if (mbar_test(x_empty + 8 * slot_x, ph_x)) {
+          mbar_arrive_expect_tx(x_full + 8 * slot_x, a.x_bytes);
+          tma_box_3d(base + slot_x * a.x_bytes, &maps.x, 0, 0, wk.s * F::STAGES, x_full + 8 * slot_x);
+          if (++slot_x == D) { slot_x = 0; ph_x ^= 1u; }
+          wk.next(a);
+          idle = 0;
+        }
+      }
+      if (wk.k < wk.n) {   // gave up: let this CTA's own copies land before its shared memory goes away
+        atomicAdd(a.error_flag, 1);
+        __nanosleep(1000000);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 5) {
+    // ---- products ------------------------------------------------------------------------------------------
+    int tries = kWaitTries;
+    int ab = 0, xs = 0, seg = 0;
+    uint32_t ph_a = 0, ph_x = 0;
+    uint32_t fresh = 1;   // the next product starts a sum
+    int block_left = by_block ? block_units - wk.s % block_units : 0;   // units left in the codebook block
+    for (; wk.k < wk.n; wk.next(a)) {
+      wait_phase(x_full + 8 * xs, ph_x, tries, a.error_flag);
+      for (int j = 0; j < F::STAGES; ++j) {
+        wait_phase(a_full + 8 * ab, ph_a, tries, a.error_flag);
+        __syncwarp();
+        tc_fence_after();
+        const uint64_t xd = b_descriptor(base + xs * a.x_bytes + j * a.x_row_bytes);   // (+ 2 q: 32-byte steps of K)
+        const uint32_t at = tmem + kAOff + ab * kStageTmem, dt = tmem + (seg & 1) * 16;
+        if (elect_one()) {   // (also after a wait that ran out: the operands are in bounds whatever they hold)
+          tc_mma(dt, at, xd, fresh ^ 1u);
+#pragma unroll
+          for (int q = 1; q < 4; ++q) tc_mma(dt, at + 8 * q, xd + 2 * q, 1u);
+          tc_commit(a_empty + 8 * ab);
+        }
+        __syncwarp();
+        fresh = 0;
+        if (++ab == kAStages) { ab = 0; ph_a ^= 1u; }
+      }
+      const bool frag_end = wk.slab_end(a);
+      const bool seg_end = frag_end || (by_block && block_left == 1);
+      if (elect_one()) {
+        tc_commit(x_empty + 8 * xs);
+        if (seg_end) tc_commit(d_full + 8 * (seg & 1));
+      }
+      __syncwarp();
+      if (seg_end) {
+        ++seg;
+        fresh = 1;
+      }
+      block_left = seg_end ? block_units : block_left - 1;   // (after a fragment's end the next one starts at column 0)
+      if (++xs == D) { xs = 0; ph_x ^= 1u; }
+    }
+  } else {
+    // ---- decode ----------------------------------------------------------------------------------------------
+    // One loop over units; what is not done in every unit stands in one place each (a codebook block, a running sum
+    // and a fragment are whole units).  With the sums read in three places the kernel had 110 to 195 KB of code and ran four
+    // times slower; with all of it checked in every stage a stage took 220 instructions a warp instead of 110.
+    int tries = kWaitTries;
+    Tables<F> tb;
+    const uint32_t my_table = tables + (F::TK == kCta ? 0 : warp * F::TABLE);
+    const uint32_t lane_off = F::D == 4 ? (lane & 15) * 8 : lane * 4;
+    const uint32_t pat = ((my_table >> 12) & 0xFu) * 0x10101010u;
+    const uint32_t swz = F::RB == 32 ? ((tid >> 2) & 1) << 4 : F::RB == 64 ? ((tid >> 1) & 3) << 4 : F::RB == 128 ? (tid & 7) << 4 : 0;
+    const uint32_t tmem_a = tmem + (static_cast<uint32_t>(warp * 32) << 16) + kAOff;
+    uint32_t tbl = my_table + lane_off;
+    int half = 0;
+    int ab = 0, islot = 0;
+    uint32_t ph_a = 1, ph_i = 0;
+
+    // The walk by fragments (the CTA's units of one tile): first column of the current unit, end column.
+    int col = wk.s * F::UC, frag_end = 0, next_k = 0;
+    int block_left = 0, seg_left = 0;   // units left in the codebook block, the running sum
+    int bcol = 0;
+    // The sum that is complete but not yet read (`pend_*`): it is read a unit or two later, when the tensor core has caught up.
+    int st = 0, fin_at = -1, seg = 0;
+    int pend_slab = 0;
+    bool pend_last = false, pend_complete = false, done = wk.n == 0, waited = false;
+    float pend_scale = 1.f, block_scale = 1.f;
+    float total[NB];
+#pragma unroll
+    for (int n = 0; n < NB; ++n) total[n] = 0.f;
+    const __half* gs = nullptr;   // int4 codebooks: the scales of the thread's row
+
+    if (!done) {
+      const Segment& sg = a.seg[segment_of(a, wk.slab)];
+      tb.open(a, sg, (wk.slab - sg.tile0) * kTileRows, tid);
+      tb.request(a, col / a.Bc);
+    }
+    bool new_frag = true;
+
+#pragma unroll 1
+    while (!done || fin_at >= 0) {
+      if (st == fin_at) {
+        // ---- read a finished sum ----
+        fin_at = -1;
+        const int buf = (seg - 1) & 1;
+        wait_phase(d_full + 8 * buf, ((seg - 1) >> 1) & 1, tries, a.error_flag);
+        __syncwarp();
+        tc_fence_after();
+        {
+          float v[NB];
+          tc_load<NB>(tmem_a - kAOff + buf * 16, v);
+          tc_fence_before();
+#pragma unroll
+          for (int n = 0; n < NB; ++n) total[n] = by_block ? fmaf(pend_scale, v[n], total[n]) : v[n];
+        }
+        if (pend_last) {
+          if (!waited) {   // outputs and workspace belong to earlier kernels of the stream until here
+            pdl_wait();
+            waited = true;
+          }
+          const Segment& sg = a.seg[segment_of(a, pend_slab)];
+          const int row = (pend_slab - sg.tile0) * kTileRows + tid;
+          bool store = pend_complete;
+          if (!pend_complete) {
+            // this CTA's share of a left-over tile: slot 0 if its piece begins inside the tile, else slot 1
+            const int part_floats = kTileRows * a.batch;
+            const int slot = (wk.tail_tile0 + wk.t0 / a.S == pend_slab) ? 0 : 1;
+            float* part = a.ws_part + (static_cast<long long>(c) * 2 + slot) * part_floats + tid;
+#pragma unroll
+            for (int n = 0; n < NB; ++n)
+              if (n < a.batch) part[n * kTileRows] = total[n];
+            const unsigned T = a.tail_units, Pt = a.tail_ctas;   // (products below 2^31: checked on the host)
+            const unsigned first_u = (pend_slab - wk.tail_tile0) * a.S;
+            const int c_first = static_cast<int>(((first_u + 1) * Pt - 1) / T), c_last = static_cast<int>(((first_u + a.S) * Pt - 1) / T);
+            __threadfence();   // this thread's sums are visible to the GPU before the ticket is drawn
+            decode_barrier();
+            if (tid == 0) {
+              const int ticket = atomicAdd(a.ws_ticket + pend_slab, 1);
+              if (ticket == c_last - c_first) a.ws_ticket[pend_slab] = 0;   // nobody else touches the counter in this call
+              __threadfence();
+              sts32(last_slot, ticket == c_last - c_first);
+            }
+            decode_barrier();
+            uint32_t last;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(last) : "r"(last_slot) : "memory");
+            if (last) {   // the last to arrive adds every CTA's share, in CTA order
+              __threadfence();
+              store = true;
+#pragma unroll
+              for (int n = 0; n < NB; ++n) total[n] = 0.f;
+#pragma unroll 4
+              for (int qc = c_first; qc <= c_last; ++qc) {
+                const int q_t0 = static_cast<int>(T * qc / Pt);
+                const int q_slot = (wk.tail_tile0 + q_t0 / a.S == pend_slab) ? 0 : 1;
+                const float* p = a.ws_part + (static_cast<long long>(qc) * 2 + q_slot) * part_floats + tid;
+#pragma unroll
+                for (int n = 0; n < NB; ++n)
+                  if (n < a.batch) total[n] += __ldcg(p + n * kTileRows);
+              }
+            }
+          }
+          if (store && row < sg.N) {
+#pragma unroll
+            for (int n = 0; n < NB; ++n)
+              if (n < a.batch) sg.Y[static_cast<long long>(n) * sg.N + row] = __float2half_rn(total[n]);
+          }
+#pragma unroll
+          for (int n = 0; n < NB; ++n) total[n] = 0.f;
+        }
+        if (done) break;
+      }
+      if (seg_left == 0) {
+        // ---- a sum ends (all but the first time), the next one begins ----
+        if (st > 0) {
+          ++seg;
+          fin_at = st;
+          pend_slab = wk.slab;
+          pend_complete = wk.complete(a);
+          pend_scale = block_scale;
+          pend_last = col == frag_end;
+          if (pend_last) {   // to the next fragment
+            wk.k = next_k;
+            if (wk.k == wk.n) {
+              done = true;
+              continue;
+            }
+            wk.slab = wk.k == wk.n_tail ? wk.whole0 : wk.slab + 1;
+            wk.s = 0;
+            col = 0;
+            new_frag = true;
+          }
+        }
+        if (new_frag) {
+          new_frag = false;
+          const int units = wk.fragment_units(a);
+          next_k = wk.k + units;
+          frag_end = col + units * F::UC;
+          bcol = col / a.Bc - 1;
+          block_left = 0;
+          if constexpr (F::I4) {
+            const Segment& sg = a.seg[segment_of(a, wk.slab)];
+            gs = sg.scale + static_cast<long long>(min((wk.slab - sg.tile0) * kTileRows + tid, sg.N - 1)) * (a.K / 128);
+          }
+        }
+        seg_left = ((by_block ? min(frag_end, (bcol + 2) * a.Bc) : frag_end) - col) / F::UC;
+        if (fin_at >= 0) fin_at = st + min(F::STAGES == 2 ? 2 : 1, seg_left);
+      }
+      uint32_t scales[F::STAGES / 2];   // int4 codebooks: of the unit's groups of 128 columns
+      if constexpr (F::I4) {
+#pragma unroll
+        for (int i = 0; i < F::STAGES / 2; ++i)
+          scales[i] = __ldg(reinterpret_cast<const unsigned short*>(gs) + col / 128 + i) * 0x10001u;
+      }
+      wait_phase(idx_full + 8 * islot, ph_i, tries, a.error_flag);
+      uint32_t w[F::RB / 4];
+      {
+        const uint32_t row_at = base + a.idx_off + islot * F::IDX_BYTES + tid * F::RB;
+#pragma unroll
+        for (int i = 0; i < F::RB / 16; ++i) {   // 128-bit reads, conflict-free at every row pitch in use
+          const uint4 v = lds128(row_at + ((16u * i) ^ swz));
+          w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+        }
+        __syncwarp();   // the unit's bytes are in registers: its stage may be refilled
+        if (lane == 0) mbar_arrive(idx_empty + 8 * islot);
+        if (++islot == D) { islot = 0; ph_i ^= 1u; }
+      }
+      if (block_left == 0) {   // another codebook block: its entries were requested a block ago
+        ++bcol;
+        block_left = ((bcol + 1) * a.Bc - col) / F::UC;
+        if constexpr (F::TK == kRow) {
+          tb.write(a, my_table + half * 128, tid);   // the other half: nobody reads it any more
+          tbl = my_table + half * 128 + lane_off;
+          half ^= 1;
+          if (by_block) block_scale = tb.scale();
+        } else if constexpr (F::TK == kWarp) {
+          __syncwarp();   // every lane has left the old table
+          tb.write(a, my_table, tid);
+          __syncwarp();
+        } else if constexpr (F::BUFS == 2) {
+          tb.write(a, my_table + half * F::TABLE, tid);   // last used two blocks ago
+          decode_barrier();
+          tbl = my_table + half * F::TABLE + lane_off;
+          half ^= 1;
+        } else {
+          decode_barrier();
+          tb.write(a, my_table, tid);
+          decode_barrier();
+        }
+        fence_value(tbl);   // look-ups of the new block stay behind the writes
+        // request the next block: of this fragment, or the first of the next one
+        int nb = bcol + 1;
+        if (nb * a.Bc >= frag_end) {
+          nb = -1;
+          if (next_k < wk.n) {
+            const int nslab = next_k == wk.n_tail ? wk.whole0 : wk.slab + 1;
+            const Segment& sg = a.seg[segment_of(a, nslab)];
+            tb.open(a, sg, (nslab - sg.tile0) * kTileRows, tid);
+            nb = 0;
+          }
+        }
+        if (nb >= 0) tb.request(a, nb);
+      }
+      --block_left;
+      auto stage = [&](auto jc) {
+        constexpr int J = decltype(jc)::value;
+        uint32_t r[32];
+        gather<F, J>(r, w, tbl, pat);
+        if constexpr (F::I4) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = mul_f16x2(r[i], scales[J / 2]);
+        }
+        wait_phase(a_empty + 8 * ab, ph_a, tries, a.error_flag);
+        __syncwarp();
+        tc_fence_after();
+        tc_store32(tmem_a + ab * kStageTmem, r);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(a_full + 8 * ab);
+        if (++ab == kAStages) { ab = 0; ph_a ^= 1u; }
+      };
+      [&]<int... J>(std::integer_sequence<int, J...>) {
+        (stage(std::integral_constant<int, J>{}), ...);
+      }(std::make_integer_sequence<int, F::STAGES>{});
+      col += F::UC;
+      --seg_left;
+      ++st;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 5) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols));
+}
+
+// ---------------------------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------------------------
+int env_int(const char* name, int dflt) {
+#ifdef VQ_TUNING
+  if (const char* e = getenv(name)) return atoi(e);
+#else
+  (void)name;
+#endif
+  return dflt;
+}
+
+size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+template <class F, int NB>
+vq_status launch(const StreamCall& call, cudaStream_t s) {
+  auto kern = tile_kernel<F, NB>;
+  constexpr size_t kSmemCap = 112 * 1024;
+  static int attr_set[kMaxDevices] = {};
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return VQ_ERR_CUDA;
+  if (device_sms(&sms) != VQ_OK) return VQ_ERR_CUDA;
+  if (!__atomic_load_n(&attr_set[dev], __ATOMIC_ACQUIRE)) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemCap)) != cudaSuccess) return VQ_ERR_CUDA;
+    __atomic_store_n(&attr_set[dev], 1, __ATOMIC_RELEASE);
+  }
+  const Geometry& g = call.g;
+  TileArgs a = {};
+  if (device_error_counter(&a.error_flag) != VQ_OK) return VQ_ERR_CUDA;
+  a.n_seg = call.n_seg;
+  a.K = g.K;
+  a.batch = call.batch;
+  a.blocks_per_row = g.blocks_per_row;
+  a.Br = g.Br;
+  a.Bc = g.Bc;
+  a.cb_int8 = g.cb_int8;
+  a.S = g.K / F::UC;   // (block columns, and so K, are whole units: tile_covers)
+  int tiles = 0;
+  long long rows_total = 0;
+  for (int i = 0; i < call.n_seg; ++i) {
+    a.seg[i].cb = call.cb[i];
+    a.seg[i].scale = call.scale[i];
+    a.seg[i].Y = call.Y[i];
+    a.seg[i].N = call.N[i];
+    a.seg[i].tile0 = tiles;
+    tiles += (call.N[i] + kTileRows - 1) / kTileRows;
+    rows_total += call.N[i];
+  }
+  if (static_cast<long long>(tiles) * a.S > 0x3fffffff) return VQ_ERR_UNSUPPORTED;
+
+  // ---- shared memory: x stages, index stages, barriers, then the tables on their boundary ----
+  const int x_rows = call.batch <= 8 ? 8 : 16;
+  a.x_row_bytes = x_rows * 128;
+  a.x_bytes = F::STAGES * a.x_row_bytes;
+  auto plan = [&](int D) {
+    a.D = D;
+    a.idx_off = D * a.x_bytes;
+    a.bar_off = a.idx_off + D * F::IDX_BYTES;
+    a.front_bytes = a.bar_off + 512;
+    // (dynamic shared memory starts 1024 bytes into the window)
+    return round_up(1024 + a.front_bytes, F::ALIGN) - 1024 + F::TABLES;
+  };
+  int per_sm = env_int("VQ_TCPS", 4);
+  int D = 2;
+  for (; per_sm >= 2; --per_sm) {
+    const size_t budget = (228 * 1024) / per_sm - 1024;
+    for (D = 3; D >= 2; --D)
+      if (plan(D) <= budget) break;
+    if (D >= 2) break;
+  }
+  if (per_sm < 2) return VQ_ERR_UNSUPPORTED;
+  D = env_int("VQ_TD", D);
+  const size_t smem_bytes = plan(D);
+  if (smem_bytes > kSmemCap || D < 2 || D > kMaxDepth) return VQ_ERR_UNSUPPORTED;
+
+  // ---- persistent CTAs: whole tiles first, the units of the left-over tiles shared evenly ----
+  const long long units = static_cast<long long>(tiles) * a.S;
+  long long P = static_cast<long long>(sms) * per_sm;
+  // A tile is shared by about nine CTAs at most: its last one adds their sums in turn, a chain of reads of the
+  // workspace (4096 x 14336 at batch 16: 41 us with 18 CTAs per tile, 28 us with 9).  Two CTAs per SM at least.
+  if (P > 9LL * tiles) P = 9LL * tiles > 2LL * sms ? 9LL * tiles : 2LL * sms;
+  if (P > units) P = units;
+#ifdef VQ_TUNING
+  if (env_int("VQ_TP", 0) && P > env_int("VQ_TP", 0)) P = env_int("VQ_TP", 0);
+#endif
+  a.q = static_cast<int>(tiles / P);
+  const int left = static_cast<int>(tiles - a.q * P);
+  const long long tail = static_cast<long long>(left) * a.S;
+  a.tail_units = static_cast<int>(tail);
+  a.tail_ctas = static_cast<int>(tail < P ? tail : P);
+  if (tail * (a.tail_ctas + 1) >= (1LL << 31)) return VQ_ERR_UNSUPPORTED;   // 32-bit arithmetic in the kernel
+  // counters at the start, partial sums at the end of the workspace: a call with fewer rows then never writes
+  // sums where one with more rows keeps its counters
+  const size_t ticket_bytes = stream_ticket_bytes(rows_total);
+  if (static_cast<size_t>(tiles) * sizeof(int) > ticket_bytes) return VQ_ERR_UNSUPPORTED;
+  const size_t part_ws = static_cast<size_t>(P) * 2 * kTileRows * call.batch * sizeof(float);
+  const size_t total_ws = stream_workspace_bytes(rows_total, call.batch);
+  if (ticket_bytes + part_ws > total_ws) return VQ_ERR_UNSUPPORTED;
+  if (!call.ws || call.ws_bytes < total_ws) return VQ_ERR_WORKSPACE;
+  a.ws_ticket = static_cast<int*>(call.ws);
+  a.ws_part = reinterpret_cast<float*>(static_cast<char*>(call.ws) + (total_ws - part_ws));
+
+  TileMaps maps;
+  for (int i = 0; i < call.n_seg; ++i) {
+    const uint64_t dims[2] = {static_cast<uint64_t>(g.stride), static_cast<uint64_t>(call.N[i])};
+    const uint64_t strides[1] = {static_cast<uint64_t>(g.stride)};
+    const uint32_t box[2] = {F::RB, kTileRows};
+    if (encode_tensor_map(&maps.idx[i], call.idx[i], 1, 2, dims, strides, box, F::SWIZZLE) != VQ_OK) return VQ_ERR_CUDA;
+  }
+  for (int i = call.n_seg; i < kMaxSegments; ++i) maps.idx[i] = maps.idx[0];
+  {
+    const uint64_t dims[3] = {64, static_cast<uint64_t>(call.batch), static_cast<uint64_t>(g.K / 64)};
+    const uint64_t strides[2] = {static_cast<uint64_t>(g.K) * 2, 128};
+    const uint32_t box[3] = {64, static_cast<uint32_t>(x_rows), F::STAGES};
+    if (encode_tensor_map(&maps.x, call.X, 2, 3, dims, strides, box, 2) != VQ_OK) return VQ_ERR_CUDA;
+  }
+
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(P), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem_bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = env_int("VQ_PDL", 1) ? 1 : 0;
+#ifdef VQ_TUNING
+  if (env_int("VQ_VERBOSE", 0)) fprintf(stderr, "tile launch: grid %d per_sm %d depth %d smem %zu tiles %d S %d q %d tail %d/%d\n", (int)P, per_sm, D, smem_bytes, tiles, a.S, a.q, a.tail_units, a.tail_ctas);
+#endif
+  if (cudaLaunchKernelEx(&cfg, kern, maps, a) != cudaSuccess) return VQ_ERR_CUDA;
+  return check_launch();
+}
+
+template <class F>
+vq_status launch_nb(const StreamCall& call, cudaStream_t s) {
+  return call.batch <= 8 ? launch<F, 8>(call, s) : launch<F, 16>(call, s);
+}
+
+}  // namespace
+
+// Codebook blocks that are whole units of columns (so K is one too).
+bool tile_covers(const Geometry& g) {
+  if (g.d == 2 && g.b == 4) return !g.cb_int4 && g.Bc % 256 == 0;
+  if (g.d == 2 && g.b == 5) return g.Bc % 256 == 0 && (g.Br % 32 == 0 || (!g.cb_int4 && (g.Br == 4 || g.Br == 8 || g.Br == 16)));
+  if (g.d == 2 && g.b == 6) return g.Bc % 128 == 0 && g.Br % 32 == 0;
+  return g.d == 4 && g.b == 8 && g.Bc % 128 == 0 && g.Br % kTileRows == 0 && !g.cb_int4;
+}
+
+// Which calls this kernel serves: those where it was the faster one on B200.  Its time hardly depends on the batch
+// (one pass over the weights for 1..16 sequences) but it has about 4 us more of start-up and summing than the cluster
+// kernels, so it takes over above a number of weights that falls with the batch.  us, other kernels / this one:
+//   row tables (57344 x 8192)      batch 1 49/63, 8 60/64, 9 81/69, 16 97/70; 28672 x 4096: 16 39/27, 9 24/26; 8192 x 8192: 16 20/22
+//   128-row blocks, 2-D (22016 x 4096) 3 18/22, 5 23/22, 8 26/22, 16 45/25; 12288 x 4096: 8 13.5/16, 9 21/18, 16 37/19; 4096 x 11008: 9 17/20, 16 23/21
+//   4-D (27648 x 5120)             1 25/25, 5 28/26, 8 36/26, 16 68/29; 5120 x 13824: 5 20/19, 8 22/19; 15360 x 5120: 8 18/19, 9 22/21.5, 16 38/22
+//   32-row blocks (28672 x 4096)   1 32/27, 8 46/28, 16 59/31; 18176 x 3328: 8 20/21, 16 41/23; 4096 x 14336: 9 22/26, 16 29/28
+//   4-row blocks (28672 x 4096)    1 34/24, 8 38/26, 16 49/29; 4096 x 14336: 1 23/19.5, 16 28/23; 6144 x 4096: 1 10.6/11.8
+// Shapes that the cluster kernels do not take (rows not a multiple of 128, K not one of 256) cost the pair-table kernel
+// more, and a launch per layer: 4160 x 3328 in three layers 21/12, 3328 x 9088 22/16 at batch 5.
+bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
+  if (!tile_covers(g)) return false;
+  long long rows = 0;
+  bool whole = g.K % 256 == 0;
+  for (int i = 0; i < n_seg; ++i) {
+    rows += N[i];
+    whole = whole && N[i] % kTileRows == 0;
+  }
+  const long long w = (rows * g.K) >> 20;   // weights of the call, in 2^20
+  if (g.d == 2 && g.b == 4) return batch >= 12 ? w >= 72 : batch >= 9 && w >= 160;
+  if (g.d == 4) return batch >= 9 ? w >= 64 : batch >= 5 && (w >= 112 || (w >= 64 && g.K >= 8192));
+  if (g.Br < 32) return w >= 48;
+  if (!whole) return w >= (n_seg > 1 ? 12 : 24);
+  if (g.Br % kTileRows == 0) return batch >= 13 ? w >= 44 : batch >= 9 ? w >= 46 : batch >= 5 && w >= 80;
+  return batch >= 13 ? w >= 54 : w >= 100;
+}
+
+vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {
+  const Geometry& g = call.g;
+  if (!tile_covers(g) || call.n_seg < 1 || call.n_seg > kMaxSegments) return VQ_ERR_UNSUPPORTED;
+  if (g.d == 2 && g.b == 4) return launch_nb<Fmt<2, 4, kRow, 1, false>>(call, s);
+  if (g.d == 4) return launch_nb<Fmt<4, 8, kCta, 128, false>>(call, s);
+  if (g.Br % kTileRows == 0) {
+    if (g.b == 6) return g.cb_int4 ? launch_nb<Fmt<2, 6, kCta, 128, true>>(call, s) : launch_nb<Fmt<2, 6, kCta, 128, false>>(call, s);
+    return g.cb_int4 ? launch_nb<Fmt<2, 5, kCta, 128, true>>(call, s) : launch_nb<Fmt<2, 5, kCta, 128, false>>(call, s);
+  }
+  if (g.Br % 32 == 0) {
+    if (g.b == 6) return g.cb_int4 ? launch_nb<Fmt<2, 6, kWarp, 32, true>>(call, s) : launch_nb<Fmt<2, 6, kWarp, 32, false>>(call, s);
+    return g.cb_int4 ? launch_nb<Fmt<2, 5, kWarp, 32, true>>(call, s) : launch_nb<Fmt<2, 5, kWarp, 32, false>>(call, s);
+  }
+  if (g.Br == 16) return launch_nb<Fmt<2, 5, kWarp, 16, false>>(call, s);
+  if (g.Br == 8) return launch_nb<Fmt<2, 5, kWarp, 8, false>>(call, s);
+  return launch_nb<Fmt<2, 5, kWarp, 4, false>>(call, s);
+}
+
+}  // namespace vq

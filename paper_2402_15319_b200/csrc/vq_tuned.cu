@@ -58,7 +58,8 @@ vq_status encode_tensor_map(CUtensorMap* tm, const void* base, int elem_bytes, i
     es[i] = 1u;
     if (i + 1 < rank) st[i] = strides[i];
   }
-  const CUtensorMapSwizzle sw = swizzle == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : swizzle == 1 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE;
+  const CUtensorMapSwizzle sw = swizzle == 2 ? CU_TENSOR_MAP_SWIZZLE_128B : swizzle == 1 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                  : swizzle == 3 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE;
   if (encode(tm, elem_bytes == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_UINT16, static_cast<cuuint32_t>(rank),
              const_cast<void*>(base), d, st, b, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_NONE,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -107,6 +108,22 @@ size_t stream_workspace_bytes(long long rows, int batch) {
 vq_status launch_gemm_tuned(const Geometry& g, const LayerPtrs& p, const __half* X, __half* Y, int batch, void* ws,
                             size_t ws_bytes, cudaStream_t s) {
   vq_status st = VQ_ERR_UNSUPPORTED;
+  if (ws && tile_preferred(g, &g.N, 1, batch)) {   // (it needs the workspace)
+    StreamCall call = {};
+    call.g = g;
+    call.n_seg = 1;
+    call.idx[0] = p.idx;
+    call.cb[0] = p.cb;
+    call.scale[0] = p.scale;
+    call.Y[0] = Y;
+    call.N[0] = g.N;
+    call.X = X;
+    call.batch = batch;
+    call.ws = ws;
+    call.ws_bytes = ws_bytes;
+    st = launch_gemm_tile(call, s);
+    if (st != VQ_ERR_UNSUPPORTED) return st;
+  }
   if (g.cb_int4) {   // int4 codebooks: the 2-D shared-codebook kernels, else warp-private pair tables
     st = launch_gemm_blockcb(g, p, X, Y, batch, s);
     return st != VQ_ERR_UNSUPPORTED ? st : launch_gemm_warptab(g, p, X, Y, batch, s);
