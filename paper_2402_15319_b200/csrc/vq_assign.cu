@@ -1,16 +1,22 @@
 // E-step / VQ_quant (paper Sec. 3, Eq. 5): for every d-vector x of a dense matrix (d adjacent
 // columns of one row) the index of the centroid of its block that minimises
 // (x - c)^T D (x - c), D = diagonal weights of the vector's columns, written in the packed index
-// format the decode path reads.  Arithmetic-bound: (4d + 2) operations per (vector, centroid).
+// format the decode path reads.
 //
 // A CTA takes a tile of 32 rows x 256*d columns; its codebooks go to shared memory as binary32
 // (int8 entries times their block scale, exact).  A thread owns 8 consecutive vectors of a row
-// (one group of 8 indices = b whole bytes of the stream), keeps them and their weights in
-// registers, walks the centroids once (shared-memory broadcasts) and writes its b bytes.
+// (one group of 8 indices = b whole bytes of the stream) and writes its b bytes.
 //
 // The decision is taken in binary32 with every operation rounded separately (no fused
 // multiply-add), terms added left to right, lowest index among equal distances: the same
 // sequence the CPU oracle evaluates, so both sides break near-ties alike.
+//
+// Arithmetic-bound: that sequence is 4 d - 1 operations and a selection per (vector, centroid).  So it is evaluated for a
+// few centroids only.  A first pass ranks all of them by the expanded form of the distance over the first weight,
+//   s = sum_t r_t c_t^2 - 2 r_t x_t c_t,   r_t = D_t / D_0,
+// 2 d - 1 fused multiply-adds (d without weights), two centroids per f32x2 instruction, and keeps the best group of 8 centroids
+// and the best score outside it.  If the two are further apart than both forms' rounding errors can account for
+// (kGap, below), the winner lies in that group and the exact sequence runs over its 8 centroids; else over all of them.
 #include "vq_common.cuh"
 
 namespace vq {
@@ -124,6 +130,238 @@ __global__ void __launch_bounds__(32 * kWarps) assign_kernel(const AssignArgs a)
   }
 }
 
+// ---- two-pass kernel (16 entries and more) -----------------------------------------------------------------------
+// two binary32 values, each operation rounded separately
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+constexpr int kGroup = 8;   // centroids per group of the first pass
+// Error bounds, u = 2^-24, M = sum_t r_t (|x_t| + max |c|)^2, which bounds every partial sum of s and the distance
+// over D_0.  Score: r_t (1 rounding) and -2 r_t x_t (2) and c_t^2 (1) enter 2 d - 1 <= 7 fused steps, each off by at most u M:
+// |s' - s| <= 12 u M.  Distance: d + 3 <= 7 roundings of non-negative terms, 8 u M each side of a comparison.  A centroid that
+// the exact sequence prefers therefore scores within 2 * 12 + 2 * 8 = 40 u M of the best; kGap = 64 u.
+constexpr float kGap = 64.f / 16777216.f;
+
+// shared memory: tables of E / 8 groups; a group = 4 pairs of centroids, a pair = (c_t[m], c_t[m + 1]) for every t, and 16
+// bytes of padding, so that 8 lanes reading 8 different groups hit different banks; then max |c| of each table
+template <int D>
+__host__ __device__ constexpr int group_bytes() { return kGroup * D * 4 + 16; }
+
+template <int D>
+__device__ __forceinline__ void load_pair(uint64_t (&c)[D], const unsigned char* p) {
+  if constexpr (D == 1) {
+    c[0] = *reinterpret_cast<const uint64_t*>(p);
+  } else {
+#pragma unroll
+    for (int i = 0; i < D / 2; ++i) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p + 16 * i);
+      c[2 * i] = v.x;
+      c[2 * i + 1] = v.y;
+    }
+  }
+}
+
+template <int D, bool HD>
+__global__ void __launch_bounds__(32 * kWarps) assign_two_pass_kernel(const AssignArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int GB = group_bytes<D>();
+  constexpr int V = D == 4 ? 4 : 8;   // vectors ranked together (registers)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int seg_cols = 256 * D;
+  const int row0 = blockIdx.y * kRows, col0 = blockIdx.x * seg_cols;
+  const int table_floats = a.entries * D, groups = a.entries / kGroup, table_bytes = groups * GB;
+  const int n_tab = a.br_per_tile * a.bc_per_seg;
+  int* cmax = reinterpret_cast<int*>(smem + n_tab * table_bytes);
+  for (int i = tid; i < n_tab; i += 32 * kWarps) cmax[i] = 0;
+  __syncthreads();
+  {
+    const long long br0 = row0 / a.Br, bc0 = col0 / a.Bc;
+    const long long last_br = (a.N - 1) / a.Br;
+    for (int o = tid; o < n_tab * table_floats; o += 32 * kWarps) {
+      const int tb = o / table_floats, within = o - tb * table_floats;
+      const int lbr = tb / a.bc_per_seg, lbc = tb - lbr * a.bc_per_seg;
+      long long brow = br0 + lbr, bcol = bc0 + lbc;
+      if (brow > last_br) brow = last_br;                        // rows past N: never used
+      if (bcol >= a.blocks_per_row) bcol = a.blocks_per_row - 1;  // columns past K: never used
+      const long long blk = brow * a.blocks_per_row + bcol;
+      float v;
+      if (a.scale == nullptr) v = __half2float(__ldg(static_cast<const __half*>(a.cb) + blk * table_floats + within));
+      else v = __fmul_rn(static_cast<float>(__ldg(static_cast<const int8_t*>(a.cb) + blk * table_floats + within)),
+                         __half2float(__ldg(a.scale + blk)));
+      const int m = within / D, t = within % D;
+      *reinterpret_cast<float*>(smem + tb * table_bytes + (m / kGroup) * GB + (m % kGroup / 2) * (D * 8) + t * 8 + (m & 1) * 4) = v;
+      atomicMax(cmax + tb, __float_as_int(fabsf(v)));   // (non-negative floats order as integers, NaN above all)
+    }
+  }
+  __syncthreads();
+
+  const int grp = blockIdx.x * 32 + lane;   // group of 8 indices within the row
+  if (grp >= a.groups) return;
+  const int col = grp * 8 * D;              // first column of the thread's 8 vectors
+  const int lbc = (col - col0) >> a.bc_shift;   // 0 when the block is wider than the segment
+  const uint64_t minus1 = pack2(-1.f, -1.f);
+
+  for (int r = warp; r < kRows; r += kWarps) {
+    const int n = row0 + r;
+    if (n >= a.N) break;
+    const int tb = (r / a.rows_per_br) * a.bc_per_seg + lbc;
+    const unsigned char* tab = smem + tb * table_bytes;
+    const float c_max = __int_as_float(cmax[tb]);
+    unsigned long long bits = 0;
+#pragma unroll
+    for (int v0 = 0; v0 < 8; v0 += V) {
+      float x[V][D], dw[V][D];
+      {
+        const uint4* src = reinterpret_cast<const uint4*>(a.W + static_cast<long long>(n) * a.K + col + v0 * D);
+#pragma unroll
+        for (int q = 0; q < V * D / 8; ++q) {   // V*D halves
+          const uint4 raw = __ldg(src + q);
+          const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+          for (int h = 0; h < 8; ++h) {
+            const int e = q * 8 + h;
+            const __half_raw hr = {static_cast<unsigned short>((wds[h >> 1] >> (16 * (h & 1))) & 0xffff)};
+            x[e / D][e % D] = __half2float(__half(hr));
+          }
+        }
+      }
+      if constexpr (HD) {
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+#pragma unroll
+          for (int t = 0; t < D; ++t) dw[v][t] = __ldg(a.hdiag + col + (v0 + v) * D + t);
+      }
+
+      // ---- rank the groups ----
+      uint64_t ca[V][D], cr[V][D];   // (-2 r_t x_t) and r_t, twice each
+      float best[V], second[V], gap[V];
+      int gi[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        float m = 0.f;
+        bool usable = true;
+#pragma unroll
+        for (int t = 0; t < D; ++t) {
+          const float rt = HD && t > 0 ? __fdiv_rn(dw[v][t], dw[v][0]) : 1.f;
+          const float at = -2.f * rt * x[v][t], reach = fabsf(x[v][t]) + c_max;
+          ca[v][t] = pack2(at, at);
+          cr[v][t] = pack2(rt, rt);
+          m += rt * reach * reach;
+          usable = usable && (!HD || dw[v][t] >= 0.f);
+        }
+        // in range, so that no term overflows or underflows to where the bounds above do not hold (else: NaN, which makes the
+        // exact sequence run over all centroids)
+        const float dm = HD ? dw[v][0] * m : m;
+        usable = usable && (!HD || dw[v][0] > 0.f) && m > 1e-30f && m < 1e30f && dm > 1e-30f && dm < 1e30f;
+        gap[v] = usable ? kGap * m : __int_as_float(0x7fc00000);
+        best[v] = second[v] = __int_as_float(0x7f800000);
+        gi[v] = 0;
+      }
+      for (int g = 0; g < groups; ++g) {
+        float gm[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) gm[v] = __int_as_float(0x7f800000);
+#pragma unroll
+        for (int p = 0; p < kGroup / 2; ++p) {
+          uint64_t c[D], q[D];
+          load_pair<D>(c, tab + g * GB + p * (D * 8));
+#pragma unroll
+          for (int t = 0; t < D; ++t) q[t] = mul2(c[t], c[t]);
+          if constexpr (!HD) {
+#pragma unroll
+            for (int t = 1; t < D; ++t) q[0] = add2(q[0], q[t]);
+          }
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            uint64_t sc = fma2(ca[v][0], c[0], q[0]);
+#pragma unroll
+            for (int t = 1; t < D; ++t) {
+              if constexpr (HD) sc = fma2(cr[v][t], q[t], sc);
+              sc = fma2(ca[v][t], c[t], sc);
+            }
+            float lo, hi;
+            unpack2(sc, lo, hi);
+            gm[v] = fminf(fminf(gm[v], lo), hi);
+          }
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          second[v] = fminf(second[v], fmaxf(best[v], gm[v]));
+          gi[v] = gm[v] < best[v] ? g : gi[v];
+          best[v] = fminf(best[v], gm[v]);
+        }
+      }
+
+      // ---- the exact sequence over the group that holds the winner (or over all) ----
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const bool sure = second[v] > best[v] + gap[v];
+        uint64_t x2[D], d2[D];
+#pragma unroll
+        for (int t = 0; t < D; ++t) {
+          x2[t] = pack2(x[v][t], x[v][t]);
+          if constexpr (HD) d2[t] = pack2(dw[v][t], dw[v][t]);
+        }
+        float bd = __int_as_float(0x7f800000);   // +inf
+        int bi = 0;
+        const int g1 = sure ? gi[v] + 1 : groups;
+#pragma unroll 1
+        for (int g = sure ? gi[v] : 0; g < g1; ++g) {
+#pragma unroll
+          for (int p = 0; p < kGroup / 2; ++p) {
+            uint64_t c[D];
+            load_pair<D>(c, tab + g * GB + p * (D * 8));
+            float lo = 0.f, hi = 0.f;
+#pragma unroll
+            for (int t = 0; t < D; ++t) {
+              const uint64_t diff = fma2(c[t], minus1, x2[t]);   // x - c, rounded once
+              uint64_t term = mul2(diff, diff);
+              if constexpr (HD) term = mul2(d2[t], term);
+              float tl, th;
+              unpack2(term, tl, th);
+              // (scalar: with a packed sum the product and the sum came out as one rounding)
+              lo = t == 0 ? tl : __fadd_rn(lo, tl);
+              hi = t == 0 ? th : __fadd_rn(hi, th);
+            }
+            if (lo < bd) {
+              bd = lo;
+              bi = g * kGroup + 2 * p;
+            }
+            if (hi < bd) {
+              bd = hi;
+              bi = g * kGroup + 2 * p + 1;
+            }
+          }
+        }
+        bits |= static_cast<unsigned long long>(bi) << ((v0 + v) * a.b);
+      }
+    }
+    uint8_t* dst = a.idx + n * a.stride + static_cast<long long>(grp) * a.b;
+    for (int i = 0; i < a.b; ++i) dst[i] = static_cast<uint8_t>(bits >> (8 * i));
+    if (grp == a.groups - 1)   // padding up to the row stride
+      for (long long i = a.used_bytes; i < a.stride; ++i) a.idx[n * a.stride + i] = 0;
+  }
+}
+
 }  // namespace
 
 // Covers formats with a whole number of 8-index groups per row that do not straddle blocks
@@ -160,10 +398,10 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
   const size_t smem = static_cast<size_t>(a.br_per_tile) * a.bc_per_seg * g.entries * g.d * sizeof(float);
   if (smem > 96 * 1024) return VQ_ERR_UNSUPPORTED;
   const dim3 grid((a.groups + 31) / 32, (g.N + kRows - 1) / kRows, 1);
-  static int attr_set[kMaxDevices][3] = {};
+  static int attr_set[kMaxDevices][9] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return VQ_ERR_CUDA;
-  auto launch = [&](auto kern, int slot) {
+  auto launch = [&](auto kern, int slot, size_t smem) {
     if (!__atomic_load_n(&attr_set[dev][slot], __ATOMIC_ACQUIRE)) {
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess) return VQ_ERR_CUDA;
       __atomic_store_n(&attr_set[dev][slot], 1, __ATOMIC_RELEASE);
@@ -171,9 +409,17 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
     kern<<<grid, 32 * kWarps, smem, s>>>(a);
     return check_launch();
   };
-  if (g.d == 1) return launch(assign_kernel<1>, 0);
-  if (g.d == 2) return launch(assign_kernel<2>, 1);
-  return launch(assign_kernel<4>, 2);
+  // Two passes from 16 entries on (two groups: a winner and the rest).
+  const int n_tab = a.br_per_tile * a.bc_per_seg;
+  const size_t smem2 = static_cast<size_t>(n_tab) * (g.entries / kGroup * (kGroup * g.d * 4 + 16) + 4);
+  if (g.entries >= 2 * kGroup && smem2 <= 96 * 1024) {
+    if (g.d == 1) return hdiag ? launch(assign_two_pass_kernel<1, true>, 3, smem2) : launch(assign_two_pass_kernel<1, false>, 4, smem2);
+    if (g.d == 2) return hdiag ? launch(assign_two_pass_kernel<2, true>, 5, smem2) : launch(assign_two_pass_kernel<2, false>, 6, smem2);
+    return hdiag ? launch(assign_two_pass_kernel<4, true>, 7, smem2) : launch(assign_two_pass_kernel<4, false>, 8, smem2);
+  }
+  if (g.d == 1) return launch(assign_kernel<1>, 0, smem);
+  if (g.d == 2) return launch(assign_kernel<2>, 1, smem);
+  return launch(assign_kernel<4>, 2, smem);
 }
 
 }  // namespace vq
