@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(32 * kWarps) assign_kernel(const AssignArgs a)
   }
 }
 
-// ---- two-pass kernel (16 entries and more) -----------------------------------------------------------------------
+// ---- two-pass kernel -----------------------------------------------------------------------
 // two binary32 values, each operation rounded separately
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   uint64_t r;
@@ -181,10 +181,10 @@ __device__ __forceinline__ void load_pair(uint64_t (&c)[D], const unsigned char*
 }
 
 template <int D, bool HD>
-__global__ void __launch_bounds__(32 * kWarps) assign_two_pass_kernel(const AssignArgs a) {
+__global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_kernel(const AssignArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int GB = group_bytes<D>();
-  constexpr int V = D == 4 ? 4 : 8;   // vectors ranked together (registers)
+  constexpr int V = D == 1 ? 8 : 4;   // vectors ranked together (8 of 2-D: 394 us, 4 and half as many registers again: 375 us)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int seg_cols = 256 * D;
   const int row0 = blockIdx.y * kRows, col0 = blockIdx.x * seg_cols;
@@ -409,10 +409,12 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
     kern<<<grid, 32 * kWarps, smem, s>>>(a);
     return check_launch();
   };
-  // Two passes from 16 entries on (two groups: a winner and the rest).
+  // Two passes from 32 entries on, and for 16 without weights in more than one dimension: with two groups the exact
+  // sequence still runs over half of the centroids.  us, one pass / two (4096 x 4096 if not said): 64 2-D entries on 11008
+  // rows, weighted 572/375, not 564/285; 32 2-D 119/104, 113/76; 256 4-D 724/468, 710/322; 16 2-D 67/82, 64/58; 16 1-D 81/91, 81/83.
   const int n_tab = a.br_per_tile * a.bc_per_seg;
   const size_t smem2 = static_cast<size_t>(n_tab) * (g.entries / kGroup * (kGroup * g.d * 4 + 16) + 4);
-  if (g.entries >= 2 * kGroup && smem2 <= 96 * 1024) {
+  if ((g.entries >= 32 || (g.entries == 16 && g.d > 1 && !hdiag)) && smem2 <= 96 * 1024) {
     if (g.d == 1) return hdiag ? launch(assign_two_pass_kernel<1, true>, 3, smem2) : launch(assign_two_pass_kernel<1, false>, 4, smem2);
     if (g.d == 2) return hdiag ? launch(assign_two_pass_kernel<2, true>, 5, smem2) : launch(assign_two_pass_kernel<2, false>, 6, smem2);
     return hdiag ? launch(assign_two_pass_kernel<4, true>, 7, smem2) : launch(assign_two_pass_kernel<4, false>, 8, smem2);
