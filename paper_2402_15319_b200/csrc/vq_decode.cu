@@ -50,6 +50,7 @@ struct DecodeArgs {
   int br_per_tile;    // codebook block rows a tile touches
   int bc_per_tile;    // codebook block columns a tile touches
   int rows_per_br;    // tile rows that share a block row = min(Br, kTileRows)
+  int wide_tables;    // tables of whole groups of 8 values
 };
 
 template <int D>
@@ -87,7 +88,43 @@ __global__ void __launch_bounds__(32 * kWarps) decode_tile_kernel(const DecodeAr
   const int table_halves = a.entries * D;
 
   // ---- codebooks of the tile -> shared memory, as the fp16 values to be written ----
-  {
+  if (a.wide_tables) {
+    // The tables of a block row are contiguous in memory and in shared memory: 8 values per thread and request (one value at a
+    // time, with two divisions each, the fill was a quarter of the kernel).
+    const long long br0 = row0 / a.Br, last_br = (a.N - 1) / a.Br;
+    const int bc0 = col0 / a.Bc;
+    const int row_chunks = min(a.bc_per_tile, a.blocks_per_row - bc0) * table_halves / 8, row_pitch = a.bc_per_tile * table_halves / 8;
+    for (int o = tid; o < a.br_per_tile * row_chunks; o += 32 * kWarps) {
+      const int lbr = o / row_chunks, within = o - lbr * row_chunks;
+      const long long brow = br0 + lbr < last_br ? br0 + lbr : last_br;   // tile rows past N: any valid block, never stored
+      const long long blk0 = brow * a.blocks_per_row + bc0, at = blk0 * (table_halves / 8) + within;   // in chunks of 8 values
+      uint4 v;
+      if (a.row_scale != nullptr) {   // signed nibbles, kept unscaled (exact in fp16)
+        const uint32_t raw = __ldg(static_cast<const uint32_t*>(a.cb) + at);
+        uint32_t* o32 = reinterpret_cast<uint32_t*>(&v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const __half2 h = __floats2half2_rn(static_cast<float>(static_cast<int>(raw << (28 - 8 * q)) >> 28),
+                                              static_cast<float>(static_cast<int>(raw << (24 - 8 * q)) >> 28));
+          o32[q] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+      } else if (a.scale == nullptr) {
+        v = __ldg(static_cast<const uint4*>(a.cb) + at);
+      } else {   // exact fp32 products, one rounding (normalised: unscaled, exact; the scales are applied together later)
+        const uint2 raw = __ldg(static_cast<const uint2*>(a.cb) + at);
+        const float f = a.norm_codes != nullptr ? 1.f : __half2float(__ldg(a.scale + blk0 + within / (table_halves / 8)));
+        uint32_t* o32 = reinterpret_cast<uint32_t*>(&v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t two = (q < 2 ? raw.x : raw.y) >> (16 * (q & 1));
+          const __half2 h = __floats2half2_rn(f * static_cast<float>(static_cast<int8_t>(two & 0xffu)),
+                                              f * static_cast<float>(static_cast<int8_t>((two >> 8) & 0xffu)));
+          o32[q] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+      }
+      reinterpret_cast<uint4*>(tables)[lbr * row_pitch + within] = v;
+    }
+  } else {
     const long long br0 = row0 / a.Br, bc0 = col0 / a.Bc;
     const long long last_br = (a.N - 1) / a.Br;
     const int n_tab = a.br_per_tile * a.bc_per_tile;
@@ -237,6 +274,7 @@ vq_status launch_decode_tuned(const Geometry& g, const LayerPtrs& p, __half* W, 
   a.br_per_tile = g.Br >= kTileRows ? 1 : kTileRows / g.Br;
   a.bc_per_tile = g.Bc >= a.tile_cols ? 1 : a.tile_cols / g.Bc;
   a.rows_per_br = g.Br >= kTileRows ? kTileRows : g.Br;
+  a.wide_tables = g.entries * g.d % 8 == 0;
   const size_t smem = static_cast<size_t>(a.br_per_tile) * a.bc_per_tile * g.entries * g.d * sizeof(__half);
   if (smem > 96 * 1024) return VQ_ERR_UNSUPPORTED;
   const dim3 grid((g.K + a.tile_cols - 1) / a.tile_cols, (g.N + kTileRows - 1) / kTileRows, 1);
