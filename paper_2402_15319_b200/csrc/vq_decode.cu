@@ -77,6 +77,15 @@ __device__ __forceinline__ uint4 lookup8(const __half* tab, uint32_t v, int b, u
   return out;
 }
 
+// a * b rounded to odd in fp32: truncated, last bit set if anything was cut off.  Rounding that to fp16 gives what rounding the
+// exact product gives (Boldo and Melquiond, "Emulation of FMA and correctly rounded sums: proved algorithms using rounding to
+// odd", 2008: two spare bits suffice, there are 13), without fp64 (11008 x 4096 int8, normalised: 49.9 us with it, 44.4 without).
+// Infinities and NaN pass through: their residual is NaN, which is not above 0.
+__device__ __forceinline__ float product_to_odd(float a, float b) {
+  const float p = __fmul_rz(a, b);
+  return __uint_as_float(__float_as_uint(p) | (fabsf(__fmaf_rn(a, b, -p)) > 0.f ? 1u : 0u));
+}
+
 // Grid (ceil(K / tile_cols), ceil(N / 32)).  Dynamic shared memory: br_per_tile * bc_per_tile
 // tables of entries * D halves.
 template <int D>
@@ -179,7 +188,7 @@ __global__ void __launch_bounds__(32 * kWarps) decode_tile_kernel(const DecodeAr
       if (a.norm_codes != nullptr) {
         // w = binary16(value * scale of the sub-row), the exact product rounded once.  The factor p collects the
         // sub-row's scale and, for int8 / int4 codebooks, the block's / row group's scale: exact in fp32 (22 bits).
-        // fp16 entries: p * entry has 22 significand bits, exact in fp32; integer entries: up to 30 bits, formed in fp64.
+        // fp16 entries: p * entry has 22 significand bits, exact in fp32; integer entries: up to 30 bits, rounded to odd.
         const int col = col0 + seg * 256 + lane_cols;
         const long long blk = static_cast<long long>(n / a.Br) * a.blocks_per_row + (col >> a.bc_shift);
         const int j = col >> a.norm_shift;
@@ -196,12 +205,11 @@ __global__ void __launch_bounds__(32 * kWarps) decode_tile_kernel(const DecodeAr
         } else {
           pf *= a.row_scale != nullptr ? __half2float(__ldg(a.row_scale + static_cast<long long>(n) * (a.K / 128) + col / 128))
                                        : __half2float(__ldg(a.scale + blk));
-          const double pd = static_cast<double>(pf);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const __half2 hv = *reinterpret_cast<const __half2*>(&o32[q]);
-            const __half2 r = __halves2half2(__double2half(pd * static_cast<double>(__low2float(hv))),
-                                             __double2half(pd * static_cast<double>(__high2float(hv))));
+            const __half2 r = __halves2half2(__float2half_rn(product_to_odd(pf, __low2float(hv))),
+                                             __float2half_rn(product_to_odd(pf, __high2float(hv))));
             o32[q] = *reinterpret_cast<const uint32_t*>(&r);
           }
         }
