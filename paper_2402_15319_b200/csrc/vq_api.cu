@@ -3,6 +3,7 @@
 #include <stdlib.h>
 
 #include "vq_common.cuh"
+#include "vq_device.cuh"
 
 namespace vq {
 
@@ -69,9 +70,30 @@ const void* mapped_device_pointer(const void* h) {
   }
   return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
-// X from mapped host memory into device memory: 16-byte pieces, grid-stride.
-__global__ void __launch_bounds__(256) fetch_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, int n16) {
+// X from mapped host memory into device memory: 16-byte pieces, grid-stride.  Bound by the latency of the host link, so there is
+// a piece per thread up to kFetchBlocks blocks.  Programmatic dependent launch on both sides: the product kernel behind it starts
+// and requests its weights while the kernel in front of it finishes; nothing is read before that one is complete (X may be
+// its output, the buffer its input).
+constexpr int kFetchBlocks = 64;
+__global__ void __launch_bounds__(256) fetch_kernel(const uint4* src, uint4* __restrict__ dst, int n16) {
+  vq::dev::pdl_launch_dependents();
+  vq::dev::pdl_wait();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+vq_status launch_fetch(const void* src, void* dst, size_t bytes, cudaStream_t s) {
+  const int n16 = static_cast<int>(bytes / 16);
+  const int blocks = (n16 + 255) / 256;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks < kFetchBlocks ? blocks : kFetchBlocks, 1, 1);
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, fetch_kernel, static_cast<const uint4*>(src), static_cast<uint4*>(dst), n16) != cudaSuccess) return VQ_ERR_CUDA;
+  return vq::check_launch();
 }
 }  // namespace
 
@@ -354,12 +376,8 @@ vq_status vq_gemm_small_batch_host(const vq_format* fmt, const void* d_idx, cons
     const void* dx = mapped_device_pointer(h_X);
     void* dy = const_cast<void*>(mapped_device_pointer(h_Y));
     if (dx && dy && aligned16(dx) && aligned16(dy)) {
-      const int n16 = static_cast<int>(x_bytes / 16);
       if (x_bytes % 16 == 0) {   // whole 16-byte pieces only
-        int blocks = (n16 + 255) / 256;
-        if (blocks > 8) blocks = 8;
-        fetch_kernel<<<blocks, 256, 0, s>>>(static_cast<const uint4*>(dx), static_cast<uint4*>(d_X), n16);
-        if (check_launch() != VQ_OK) return VQ_ERR_CUDA;
+        if (launch_fetch(dx, d_X, x_bytes, s) != VQ_OK) return VQ_ERR_CUDA;
         return vq_gemm_small_batch(fmt, d_idx, d_cb, d_scale, d_X, dy, batch, d_ws, base, stream);
       }
     }
@@ -407,11 +425,7 @@ vq_status vq_gemm_small_batch_grouped_host(const vq_format* fmt, const vq_group_
     mapped = dev[i].d_Y && aligned16(dev[i].d_Y);
   }
   if (mapped) {
-    const int n16 = static_cast<int>(x_bytes / 16);
-    int blocks = (n16 + 255) / 256;
-    if (blocks > 8) blocks = 8;
-    fetch_kernel<<<blocks, 256, 0, s>>>(static_cast<const uint4*>(dx), static_cast<uint4*>(d_X), n16);
-    if (check_launch() != VQ_OK) return VQ_ERR_CUDA;
+    if (launch_fetch(dx, d_X, x_bytes, s) != VQ_OK) return VQ_ERR_CUDA;
     return vq_gemm_small_batch_grouped(fmt, dev, n_members, d_X, batch, d_ws, base, stream);
   }
   size_t off = base + round256(x_bytes);
