@@ -140,11 +140,20 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+_current_raw_stream = None
+
+
 def _stream(stream):
-    if stream is None:
+    """cudaStream_t of `stream`, or of torch's current stream on the current device (its handle directly: a Stream
+    object per call is a microsecond of host time)."""
+    if stream is not None:
+        return stream.cuda_stream
+    global _current_raw_stream
+    if _current_raw_stream is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return stream.cuda_stream
+        raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+        _current_raw_stream = (lambda: raw(device())) if raw else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _current_raw_stream()
 
 
 def vq_pack_info(fmt: VQFormat) -> PackInfo:
@@ -217,9 +226,7 @@ class _CGroupMember(ctypes.Structure):
 
 def vq_gemm_small_batch_grouped(fmt: VQFormat, members, d_X, batch: int, d_ws, stream=None) -> None:
     """members: sequence of (d_idx, d_cb, d_scale, d_Y, n_rows); fmt.n_rows = the sum of the members' rows."""
-    arr = (_CGroupMember * len(members))()
-    for i, (idx, cb, sc, Y, n) in enumerate(members):
-        arr[i] = _CGroupMember(_ptr(idx), _ptr(cb), _ptr(sc), _ptr(Y), int(n))
+    arr = (_CGroupMember * len(members))(*[(_ptr(idx), _ptr(cb), _ptr(sc), _ptr(Y), int(n)) for idx, cb, sc, Y, n in members])
     c = fmt.c()
     _check(load().vq_gemm_small_batch_grouped(ctypes.byref(c), arr, len(members), _ptr(d_X), int(batch), _ptr(d_ws),
                                               d_ws.numel() * d_ws.element_size(), _stream(stream)),
@@ -229,9 +236,7 @@ def vq_gemm_small_batch_grouped(fmt: VQFormat, members, d_X, batch: int, d_ws, s
 def vq_gemm_small_batch_grouped_host(fmt: VQFormat, members, h_X, batch: int, d_ws, stream=None) -> None:
     """members: sequence of (d_idx, d_cb, d_scale, h_Y, n_rows) with HOST outputs; h_X a host tensor (pinned for
     the direct path).  Synchronise before reading the outputs."""
-    arr = (_CGroupMember * len(members))()
-    for i, (idx, cb, sc, Y, n) in enumerate(members):
-        arr[i] = _CGroupMember(_ptr(idx), _ptr(cb), _ptr(sc), _ptr(Y), int(n))
+    arr = (_CGroupMember * len(members))(*[(_ptr(idx), _ptr(cb), _ptr(sc), _ptr(Y), int(n)) for idx, cb, sc, Y, n in members])
     c = fmt.c()
     _check(load().vq_gemm_small_batch_grouped_host(ctypes.byref(c), arr, len(members), _ptr(h_X), int(batch), _ptr(d_ws),
                                                    d_ws.numel() * d_ws.element_size(), _stream(stream)),
