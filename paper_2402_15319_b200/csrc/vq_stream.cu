@@ -384,16 +384,24 @@ struct RowD2B4 {
       const uint32_t xstep = batch * X_ROW_BYTES;
       const uint32_t sw = static_cast<uint32_t>(lane >> 2) << 4;
       const uint32_t t32 = static_cast<uint32_t>(lane & 3) << 5;
+      // Only lanes whose batch row exists read: a 128-bit read costs a wavefront per quarter warp that takes part, and
+      // at one or two sequences three of the four would read what the first one reads (zeros do for their products).
       uint4 b[NB][2];
+      bool on[NB];
+#pragma unroll
+      for (int nb = 0; nb < NB; ++nb) {
+        on[nb] = nb * 8 + (lane >> 2) < batch;
+        b[nb][0] = b[nb][1] = make_uint4(0u, 0u, 0u, 0u);
+      }
 #pragma unroll kUnrollD2
       for (int ww = 0; ww < 8; ++ww) {
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb) {
           // 32 bytes at t*32 of the 128-byte row; the box is swizzled: piece p of row r at p ^ (r & 7)
-          const unsigned char* r = xrow[nb] + ww * xstep;
-          const uint32_t ph = (static_cast<uint32_t>(reinterpret_cast<uintptr_t>(r)) >> 3) & 0x70u;
-          b[nb][0] = *reinterpret_cast<const uint4*>(r + (t32 ^ ph));
-          b[nb][1] = *reinterpret_cast<const uint4*>(r + ((t32 + 16u) ^ ph));
+          const uint32_t r = smem_u32(xrow[nb] + ww * xstep);
+          const uint32_t ph = (r >> 3) & 0x70u;
+          lds128_if(b[nb][0], r + (t32 ^ ph), on[nb]);
+          lds128_if(b[nb][1], r + ((t32 + 16u) ^ ph), on[nb]);
         }
         tile_step<0>(idx, ww, sw, b);
         if constexpr (R > 1) tile_step<1>(idx, ww, sw, b);
