@@ -101,7 +101,9 @@ typedef enum {
   VQ_IMPL_GENERIC = 1,  /* format-generic fp32-FMA kernel (any valid format)                     */
   VQ_IMPL_TUNED = 2,    /* tuned kernel only; VQ_ERR_UNSUPPORTED if none covers the format/shape */
   VQ_IMPL_STREAM = 3    /* the persistent tuned kernel only (the one AUTO picks for large per-row 4-bit
-                           layers and for groups); VQ_ERR_UNSUPPORTED if it does not cover the format */
+                           layers and for groups at small batch); VQ_ERR_UNSUPPORTED if it does not cover
+                           the format.  (AUTO and TUNED also pick the tcgen05 kernel, vq_tile.cu, for large
+                           layers and batches.) */
 } vq_impl;
 
 /* Caller-filled description of one VQ-compressed matrix (paper Sec. 2.1 notation in comments). */
@@ -182,8 +184,8 @@ vq_status vq_gemm_small_batch_impl(const vq_format* fmt, const void* d_idx, cons
  *               pointers (layouts as for vq_gemm_small_batch), its output d_Y (binary16
  *               [batch][n_rows]) and its row count (a multiple of block_rows).
  *   d_X       : device binary16 [batch][K], shared by all members.
- * One kernel serves the whole group where the persistent kernel, the shared-codebook kernels or the
- * pair-table kernel cover the format (vq_grouped_kernel_launches tells); otherwise the members run one
+ * One kernel serves the whole group where the persistent, shared-codebook, pair-table or tcgen05
+ * kernels cover the format (vq_grouped_kernel_launches tells); otherwise the members run one
  * after the other on `stream`.  Results are the same as n_members separate calls.
  * Errors: as vq_gemm_small_batch; SHAPE also if the rows do not add up to fmt->n_rows. */
 #define VQ_MAX_GROUP 4

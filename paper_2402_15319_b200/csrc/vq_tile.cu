@@ -8,6 +8,8 @@
 // decoded tile goes from registers to tensor memory by tcgen05.st, which has its own path (gathers alone ran at
 // 63.0 weights / clk / SM in a probe on resident data, with the stores 60.7, with the products 48.4), and the
 // accumulators live in tensor memory, which leaves registers for 16 gathering warps per SM.
+// Measured: 57344 x 8192, 2-D 4-bit, 16 sequences 96.6 us in the persistent mma.sync kernel, 72.2 here (23 weights / clk / SM: a
+// stage takes about 170 instructions a warp where its gathers need 77, four warps a scheduler issue 57 % of the time).
 //
 // Work.  The rows of a call's layers ("segments") are cut into tiles of 128 rows, a tile's columns into units of
 // UC.  The grid is persistent, four CTAs per SM at most; every CTA takes q whole tiles, and the units
