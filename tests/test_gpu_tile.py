@@ -22,23 +22,23 @@ def _spec(name, N, K, d, b, Br, Bc, cb):
 
 CASES = [
     # row tables (sums scaled per block), one row and four rows per block, a tile of 68 rows at the end
-    (_spec("row_i8", 18500, 4096, 2, 4, 1, 2048, True), (12, 16)),
-    (_spec("row_fp16", 18500, 4096, 2, 4, 1, 256, False), (12,)),
+    (_spec("row_i8", 18500, 4096, 2, 4, 1, 2048, True), (13, 16)),
+    (_spec("row_fp16", 18500, 4096, 2, 4, 1, 256, False), (13,)),
     (_spec("row4_i8", 18500, 4096, 2, 4, 4, 512, True), (16,)),
     # one table for the four warps
     (_spec("cta6_fp16", 11904, 4096, 2, 6, 128, 128, False), (9, 16)),
     (_spec("cta6_odd_k", 6272, 4224, 2, 6, 128, 128, True), (1, 8, 9)),
-    (_spec("cta5_fp16", 11904, 4096, 2, 5, 128, 256, False), (9,)),
+    (_spec("cta5_fp16", 20608, 4096, 2, 5, 128, 256, False), (9,)),
     (_spec("cta_4d_fp16", 13312, 5120, 4, 8, 256, 512, False), (9, 16)),
     (_spec("cta_4d_i8", 13312, 5120, 4, 8, 256, 512, True), (9,)),
     # a table per warp: 32-row blocks (rows end 96 short of a tile), INT4 codebooks, small blocks
     (_spec("warp6_i8", 6176, 4352, 2, 6, 32, 256, True), (1, 8, 9, 16)),
     (_spec("warp6_fp16", 6176, 4352, 2, 6, 32, 256, False), (3,)),
     (_spec("warp6_i4", 6176, 4224, 2, 6, 32, 128, 2), (1, 16)),
-    (_spec("warp5_i4", 6176, 4352, 2, 5, 32, 256, 2), (5,)),
-    (_spec("warp5_4", 12300, 4352, 2, 5, 4, 256, True), (1, 8, 9)),
-    (_spec("warp5_8", 12304, 4352, 2, 5, 8, 256, False), (3,)),
-    (_spec("warp5_16", 12304, 4352, 2, 5, 16, 256, True), (16,)),
+    (_spec("warp5_i4", 13088, 4352, 2, 5, 32, 256, 2), (5,)),
+    (_spec("warp5_4", 13060, 4352, 2, 5, 4, 256, True), (1, 8, 9)),
+    (_spec("warp5_8", 13072, 4352, 2, 5, 8, 256, False), (3,)),
+    (_spec("warp5_16", 13072, 4352, 2, 5, 16, 256, True), (16,)),
 ]
 
 
