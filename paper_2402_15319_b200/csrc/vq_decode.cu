@@ -6,7 +6,7 @@
 // everything is arranged around the stores: a warp turns one 256-column segment of one row into 32
 // adjacent 128-bit stores (lane l owns columns 8l .. 8l+7 = 8/d indices = m = 8b/d bits).  The
 // segment's m index words are fetched by one coalesced 32-bit load (lanes 0..m-1) and handed to
-// their owners by two shuffles and a funnel shift.  A CTA works on a tile of 32 rows x 2048 columns
+// their owners by two shuffles and a funnel shift.  A CTA works on a tile of 8 rows x 2048 columns
 // whose codebooks are first copied into shared memory as final fp16 values (int8 entries as
 // fp16(fp32(scale) * c): one rounding, the value the entry point is specified to write), so a
 // look-up is one shared-memory load of d halves; bank conflicts among the lanes' random entries
@@ -17,16 +17,12 @@
 namespace vq {
 namespace {
 
-#ifndef VQ_DEC_TILE_ROWS
-#define VQ_DEC_TILE_ROWS 32
-#endif
 #ifndef VQ_DEC_TILE_COLS
 #define VQ_DEC_TILE_COLS 2048
 #endif
 #ifndef VQ_DEC_UNROLL
 #define VQ_DEC_UNROLL 8
 #endif
-constexpr int kTileRows = VQ_DEC_TILE_ROWS;
 constexpr int kTileCols = VQ_DEC_TILE_COLS;
 constexpr int kWarps = 8;
 constexpr int kUnroll = VQ_DEC_UNROLL;   // segments of a row whose index loads are in flight together
@@ -49,7 +45,7 @@ struct DecodeArgs {
   int bc_shift;       // log2(Bc): block columns are a power of two
   int br_per_tile;    // codebook block rows a tile touches
   int bc_per_tile;    // codebook block columns a tile touches
-  int rows_per_br;    // tile rows that share a block row = min(Br, kTileRows)
+  int rows_per_br;    // tile rows that share a block row = min(Br, rows of the tile)
   int wide_tables;    // tables of whole groups of 8 values
 };
 
@@ -86,14 +82,15 @@ __device__ __forceinline__ float product_to_odd(float a, float b) {
   return __uint_as_float(__float_as_uint(p) | (fabsf(__fmaf_rn(a, b, -p)) > 0.f ? 1u : 0u));
 }
 
-// Grid (ceil(K / tile_cols), ceil(N / 32)).  Dynamic shared memory: br_per_tile * bc_per_tile
+// Grid (ceil(K / tile_cols), ceil(N / ROWS)).  Dynamic shared memory: br_per_tile * bc_per_tile
 // tables of entries * D halves.
-template <int D>
+// ROWS: rows of a tile, known at compile time (one row a warp at 8: no loop; as an argument it cost 8 %).
+template <int D, int ROWS>
 __global__ void __launch_bounds__(32 * kWarps) decode_tile_kernel(const DecodeArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __half* tables = reinterpret_cast<__half*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int row0 = blockIdx.y * kTileRows, col0 = blockIdx.x * a.tile_cols;
+  const int row0 = blockIdx.y * ROWS, col0 = blockIdx.x * a.tile_cols;
   const int table_halves = a.entries * D;
 
   // ---- codebooks of the tile -> shared memory, as the fp16 values to be written ----
@@ -170,7 +167,7 @@ __global__ void __launch_bounds__(32 * kWarps) decode_tile_kernel(const DecodeAr
   const int segs = min(a.tile_cols, a.K - col0) / 256;
   const int bit0 = lane * m, src_lane = bit0 >> 5, sh = bit0 & 31;
   const int src_lane2 = src_lane + 1 < m ? src_lane + 1 : src_lane;
-  for (int r = warp; r < kTileRows; r += kWarps) {
+  for (int r = warp; r < ROWS; r += kWarps) {
     const int n = row0 + r;
     if (n >= a.N) break;
     const uint32_t* row32 = reinterpret_cast<const uint32_t*>(a.idx + n * a.stride) + static_cast<long long>(col0 / 256) * m;
@@ -241,7 +238,7 @@ __global__ void __launch_bounds__(32 * kWarps) decode_tile_kernel(const DecodeAr
 
 // Formats the tile kernel covers: K a multiple of 256, at most 32 index bits per lane and segment
 // (8 b / d <= 32), block columns a power of two >= 8 that divide or are divided by the tile's columns,
-// block rows that divide or are divided by 32, tables of the tile within 96 KB of shared memory.
+// block rows that divide or are divided by the tile's rows, tables of the tile within 96 KB of shared memory.
 // With norm_codes: block-wise normalisation, sub-rows of a power of two of at least 8 columns.
 vq_status launch_decode_tuned(const Geometry& g, const LayerPtrs& p, __half* W, cudaStream_t s, const void* norm_codes,
                               const void* norm_lut, int norm_block_cols) {
@@ -264,7 +261,17 @@ vq_status launch_decode_tuned(const Geometry& g, const LayerPtrs& p, __half* W, 
     if ((1 << sft) == g.Bc) a.bc_shift = sft;
   if (a.bc_shift < 0) return VQ_ERR_UNSUPPORTED;
   if (a.tile_cols % g.Bc && g.Bc % a.tile_cols) return VQ_ERR_UNSUPPORTED;
-  if (kTileRows % g.Br && g.Br % kTileRows) return VQ_ERR_UNSUPPORTED;
+  // Rows of a tile: one per warp, so that a layer is several waves of short CTAs (with 32, four rows a warp in turn, a
+  // layer was one or two waves: 11008 x 4096 2-D 6-bit 23.3 us, 16 rows 22.0, 8 rows 21.7; 4096 x 14336 32.9 / 28.7 / 27.3;
+  // 512 x 2048 7.4 / 4.9 / 3.2), two where the tile's codebooks are larger than what it writes per row (256 4-D entries,
+  // 11008 x 4096: 22.7 / 22.6 / 25.0) unless that leaves SMs idle (512 x 2048: 7.3 / 4.9 / 3.6).
+  int sms = 0;
+  if (device_sms(&sms) != VQ_OK) return VQ_ERR_CUDA;
+  const long long tile_tables = static_cast<long long>(g.Bc >= a.tile_cols ? 1 : a.tile_cols / g.Bc) * g.entries * g.d * 2;
+  const long long col_tiles = (g.K + a.tile_cols - 1) / a.tile_cols;
+  int rows = tile_tables > 2LL * a.tile_cols && col_tiles * ((g.N + 15) / 16) >= 2LL * sms ? 16 : 8;
+  while (rows < 32 && (g.N + rows - 1) / rows > 65535) rows *= 2;   // (the grid's second dimension)
+  if (rows % g.Br && g.Br % rows) return VQ_ERR_UNSUPPORTED;
   a.idx = p.idx;
   a.cb = p.cb;
   a.scale = g.cb_int8 ? p.scale : nullptr;
@@ -279,14 +286,14 @@ vq_status launch_decode_tuned(const Geometry& g, const LayerPtrs& p, __half* W, 
   a.entries = g.entries;
   a.blocks_per_row = g.blocks_per_row;
   a.m = 8 * g.b / g.d;
-  a.br_per_tile = g.Br >= kTileRows ? 1 : kTileRows / g.Br;
+  a.br_per_tile = g.Br >= rows ? 1 : rows / g.Br;
   a.bc_per_tile = g.Bc >= a.tile_cols ? 1 : a.tile_cols / g.Bc;
-  a.rows_per_br = g.Br >= kTileRows ? kTileRows : g.Br;
+  a.rows_per_br = g.Br >= rows ? rows : g.Br;
   a.wide_tables = g.entries * g.d % 8 == 0;
   const size_t smem = static_cast<size_t>(a.br_per_tile) * a.bc_per_tile * g.entries * g.d * sizeof(__half);
   if (smem > 96 * 1024) return VQ_ERR_UNSUPPORTED;
-  const dim3 grid((g.K + a.tile_cols - 1) / a.tile_cols, (g.N + kTileRows - 1) / kTileRows, 1);
-  static int attr_set[kMaxDevices][3] = {};
+  const dim3 grid((g.K + a.tile_cols - 1) / a.tile_cols, (g.N + rows - 1) / rows, 1);
+  static int attr_set[kMaxDevices][9] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return VQ_ERR_CUDA;
   auto launch = [&](auto kern, int slot) {
@@ -297,9 +304,12 @@ vq_status launch_decode_tuned(const Geometry& g, const LayerPtrs& p, __half* W, 
     kern<<<grid, 32 * kWarps, smem, s>>>(a);
     return check_launch();
   };
-  if (g.d == 1) return launch(decode_tile_kernel<1>, 0);
-  if (g.d == 2) return launch(decode_tile_kernel<2>, 1);
-  return launch(decode_tile_kernel<4>, 2);
+  auto by_rows = [&](auto k8, auto k16, auto k32, int slot) {
+    return rows == 8 ? launch(k8, slot) : rows == 16 ? launch(k16, slot + 1) : launch(k32, slot + 2);
+  };
+  if (g.d == 1) return by_rows(decode_tile_kernel<1, 8>, decode_tile_kernel<1, 16>, decode_tile_kernel<1, 32>, 0);
+  if (g.d == 2) return by_rows(decode_tile_kernel<2, 8>, decode_tile_kernel<2, 16>, decode_tile_kernel<2, 32>, 3);
+  return by_rows(decode_tile_kernel<4, 8>, decode_tile_kernel<4, 16>, decode_tile_kernel<4, 32>, 6);
 }
 
 }  // namespace vq
