@@ -43,16 +43,19 @@ __device__ __forceinline__ uint2 lds64(uint32_t addr) {
   return v;
 }
 __device__ __forceinline__ void fence_value(uint32_t& v) { asm volatile("" : "+r"(v)::"memory"); }
+// Reads of a stage that the copy engine refills: the "memory" clobber keeps them in front of the release of the stage.  (Volatile
+// alone does not: without the clobber a read may sink past the barrier arrival to where its value is used.)
 // 128-bit shared load that only lanes with `on` perform; the others keep `v`.
 __device__ __forceinline__ void lds128_if(uint4& v, uint32_t addr, bool on) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];\n\t}"
       : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w)
-      : "r"(addr), "r"(static_cast<int>(on)));
+      : "r"(addr), "r"(static_cast<int>(on))
+      : "memory");
 }
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
   uint4 v;
-  asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+  asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
   return v;
 }
 __device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {

@@ -892,6 +892,7 @@ stream_kernel(const __grid_constant__ Maps maps, const StreamArgs a) {
         atomicAdd(a.error_flag, 1);
         break;
       }
+      fence_proxy_async();   // the consumers' reads of the slot (released by their arrivals) before the copy engine's writes
       const int sg = segment_of(wk_.slab);
       const int row0 = (wk_.slab - a.seg[sg].slab0) * slab_rows;
       const uint32_t stage = sbase + a.stage_off + slot * a.stage_bytes;

@@ -484,6 +484,7 @@ __global__ void __launch_bounds__(kThreads, 4) tile_kernel(const __grid_constant
       while (wk.k < wk.n && idle < kPolls) {
         if (++idle > 1) __nanosleep(kPollSleep);   // (polls without a pause take issue slots from the decoding warps)
         if (wi.k < wi.n && mbar_test(idx_empty + 8 * slot_i, ph_i)) {
+          fence_proxy_async();   // the warps' reads of the stage (released by their arrivals) before the copy engine's writes
           const int g = segment_of(a, wi.slab);
           mbar_arrive_expect_tx(idx_full + 8 * slot_i, F::IDX_BYTES);
           tma_box_2d(base + a.idx_off + slot_i * F::IDX_BYTES, &maps.idx[g], wi.s * F::RB, (wi.slab - a.seg[g].tile0) * kTileRows,

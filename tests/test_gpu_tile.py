@@ -78,3 +78,28 @@ def test_tile_kernel_group_of_ragged_layers():
     for spec, L, dY in keep:
         Y, A = orc.gemm(oracle_fmt(spec), L.idx, L.cb, L.scale, X, threads=8)
         assert_outputs_close(dY.cpu().numpy(), Y, A, spec.name)
+
+
+@pytest.mark.parametrize("spec,batch", [
+    (_spec("row_fp16_long", 7424, 14336, 2, 4, 1, 256, False), 16),
+    (_spec("row_i8_long", 9728, 11008, 2, 4, 1, 256, True), 16),
+    (_spec("warp6_i4_long", 14784, 7168, 2, 6, 96, 256, 2), 10),
+], ids=lambda v: v.name if hasattr(v, "name") else None)
+def test_every_launch_reads_its_indices_before_they_are_replaced(spec, batch):
+    """Launches in a row, all rows of all of them bit-identical: the index bytes of a unit are read before their stage is refilled
+    (where a table changes with every unit, the warps wait for global memory between the two)."""
+    import torch
+    L = draw(spec, 63)
+    dev = DeviceLayer(spec, L)
+    X = vq_synth.make_x(spec, 64, batch)
+    dX = torch.from_numpy(X).cuda()
+    Ys = torch.empty((60, batch, spec.N), dtype=torch.float16, device="cuda")
+    torch.cuda.synchronize()
+    for Y in Ys:
+        vq.vq_gemm_small_batch(dev.fmt, dev.idx, dev.cb, dev.scale, dX, Y, batch, dev.ws)
+    torch.cuda.synchronize()
+    same = (Ys.view(torch.int16) == Ys[0].view(torch.int16)).flatten(1).all(1)
+    assert bool(same.all()), f"{int((~same).sum())} of {len(Ys)} launches differ from the first"
+    rows = _rows(spec.N)
+    Y, A = orc.gemm(oracle_fmt(spec), L.idx, L.cb, L.scale, X, rows=rows, threads=8)
+    assert_outputs_close(Ys[0].cpu().numpy()[:, rows], Y, A, spec.name)
