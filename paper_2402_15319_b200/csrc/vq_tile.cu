@@ -200,7 +200,10 @@ __device__ __forceinline__ void tc_load(uint32_t addr, float (&v)[NB]) {
   }
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < NB; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < NB; ++i) {
+    asm volatile("" : "+r"(r[i]));   // used behind the wait only
+    v[i] = __uint_as_float(r[i]);
+  }
 }
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
