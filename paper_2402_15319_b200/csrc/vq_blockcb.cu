@@ -452,6 +452,8 @@ blockcb_kernel(const __grid_constant__ BlockMaps maps, const BlockArgs a_in, con
   // Activations of the CTA's column range: chunk i, 16-byte piece j of a lane's 64 columns, batch
   // row m, lane quarter tt at ((i*8 + j)*batch + m)*4 + tt.
   pdl_wait();   // the activations (and Y) belong to the previous kernel until here
+  const __half* X = a.X;
+  fence_pointer(X);
   {
     uint4* xs = reinterpret_cast<uint4*>(smem + a.x_off);
     const int n16 = n * 32;   // 16-byte pieces per batch row
@@ -464,7 +466,7 @@ blockcb_kernel(const __grid_constant__ BlockMaps maps, const BlockArgs a_in, con
       xv[u] = make_uint4(0u, 0u, 0u, 0u);
       if (item < total) {
         const int m = item / n16, q = item - m * n16;
-        xv[u] = __ldg(reinterpret_cast<const uint4*>(a.X + static_cast<long long>(m) * a.K + c0 * 256) + q);
+        xv[u] = ldg128_l2(reinterpret_cast<const uint4*>(X + static_cast<long long>(m) * a.K + c0 * 256) + q);
       }
     }
     if constexpr (PRIV) {
@@ -486,7 +488,7 @@ blockcb_kernel(const __grid_constant__ BlockMaps maps, const BlockArgs a_in, con
     }
     for (int item = tid + kInReg * T::THREADS; item < total; item += T::THREADS) {
       const int m = item / n16, q = item - m * n16;
-      put(item, __ldg(reinterpret_cast<const uint4*>(a.X + static_cast<long long>(m) * a.K + c0 * 256) + q));
+      put(item, ldg128_l2(reinterpret_cast<const uint4*>(X + static_cast<long long>(m) * a.K + c0 * 256) + q));
     }
   }
   __syncthreads();

@@ -82,6 +82,16 @@ __device__ __forceinline__ uint4 ldg128_nc(const void* p) {
   asm volatile("ld.global.nc.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
+// Loads from L2 of data that an earlier kernel of the stream may write while this one is already resident (it was launched
+// early): the non-coherent path is for data that does not change while the kernel lives, and a line of L1 may be older than the
+// wait.  Not volatile, so that the requests of a loop overlap: the pointer passes through fence_pointer() behind pdl_wait().
+__device__ __forceinline__ uint4 ldg128_l2(const void* p) {
+  uint4 v;
+  asm("ld.global.cg.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+template <class T>
+__device__ __forceinline__ void fence_pointer(T*& p) { asm volatile("" : "+l"(p)::"memory"); }
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t r;

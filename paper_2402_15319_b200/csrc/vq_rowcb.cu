@@ -382,6 +382,8 @@ __global__ void __launch_bounds__(256, VQ_ROW_MIN_CTAS) rowcb_kernel(const RowAr
 
   // ---- activations of the CTA's column range ----
   pdl_wait();   // the activations (and Y) belong to the previous kernel until here
+  const __half* X = a.X;
+  fence_pointer(X);
   // XS: window k of this column part = steps s0 + k*kWindow ..; buffer k & 1 of the part's pair
   const uint32_t win_bytes = kWindow * CHUNKS * a.batch * 64;
   const uint32_t part_x = smem_base + a.x_offset + wk * 2 * win_bytes;
@@ -397,7 +399,7 @@ __global__ void __launch_bounds__(256, VQ_ROW_MIN_CTAS) rowcb_kernel(const RowAr
         const int step = col / P::STEP_COLS, within = col % P::STEP_COLS;
         const int tt = within / LANE_COLS, chunk = (within % LANE_COLS) / 8;
         cp_async16(part_x + (k & 1) * win_bytes + (((step * CHUNKS + chunk) * a.batch + m) * 4 + tt) * 16,
-                   a.X + static_cast<long long>(m) * a.K + static_cast<long long>(w0) * P::STEP_COLS + col);
+                   X + static_cast<long long>(m) * a.K + static_cast<long long>(w0) * P::STEP_COLS + col);
       }
     }
     cp_async_commit();
@@ -409,12 +411,12 @@ __global__ void __launch_bounds__(256, VQ_ROW_MIN_CTAS) rowcb_kernel(const RowAr
     const int n8 = (cta_s1 - cta_s0) * (P::STEP_COLS / 8);
     uint4* xs = reinterpret_cast<uint4*>(smem + a.x_offset);
     for (int m = 0; m < a.batch; ++m) {
-      const uint4* src = reinterpret_cast<const uint4*>(a.X + static_cast<long long>(m) * a.K + col0);
+      const uint4* src = reinterpret_cast<const uint4*>(X + static_cast<long long>(m) * a.K + col0);
       for (int c8 = tid; c8 < n8; c8 += blockDim.x) {
         const int col = c8 * 8;
         const int step = col / P::STEP_COLS, within = col % P::STEP_COLS;
         const int tt = within / LANE_COLS, chunk = (within % LANE_COLS) / 8;
-        xs[((step * CHUNKS + chunk) * a.batch + m) * 4 + tt] = P::permute_x(__ldg(src + c8));
+        xs[((step * CHUNKS + chunk) * a.batch + m) * 4 + tt] = P::permute_x(ldg128_l2(src + c8));
       }
     }
   }
