@@ -15,8 +15,9 @@
 // few centroids only.  A first pass ranks all of them by the expanded form of the distance over the first weight,
 //   s = sum_t r_t c_t^2 - 2 r_t x_t c_t,   r_t = D_t / D_0,
 // 2 d - 1 fused multiply-adds (d without weights), two centroids per f32x2 instruction, and keeps the best group of 8 centroids
-// and the best score outside it.  If the two are further apart than both forms' rounding errors can account for
-// (kGap, below), the winner lies in that group and the exact sequence runs over its 8 centroids; else over all of them.
+// (for large or one-dimensional codebooks the two best) and the best score outside.  If that one is further from the best than
+// both forms' rounding errors can account for (the gap, below), the winner lies in the group or groups kept and the exact
+// sequence runs over their centroids; else over all of them.
 #include "vq_common.cuh"
 
 namespace vq {
@@ -36,6 +37,7 @@ struct AssignArgs {
   int used_bytes;       // bytes of a row that hold indices; the rest of the stride is zero-filled
   int bc_shift;         // log2(Bc)
   int br_per_tile, bc_per_seg, rows_per_br;
+  int find_equal;    // two-pass kernel: leave repeated entries aside
 };
 
 template <int D>
@@ -155,11 +157,16 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 }
 
 constexpr int kGroup = 8;   // centroids per group of the first pass
-// Error bounds, u = 2^-24, M = sum_t r_t (|x_t| + max |c|)^2, which bounds every partial sum of s and the distance
-// over D_0.  Score: r_t (1 rounding) and -2 r_t x_t (2) and c_t^2 (1) enter 2 d - 1 <= 7 fused steps, each off by at most u M:
-// |s' - s| <= 12 u M.  Distance: d + 3 <= 7 roundings of non-negative terms, 8 u M each side of a comparison.  A centroid that
-// the exact sequence prefers therefore scores within 2 * 12 + 2 * 8 = 40 u M of the best; kGap = 64 u.
-constexpr float kGap = 64.f / 16777216.f;
+// The gap, u = 2^-24.  For a centroid c let d be its distance over D_0 and M = sum_t r_t (|x_t| + |c_t|)^2, which bounds d, |s| and
+// every partial sum of both.  Score: r_t (1 rounding), -2 r_t x_t (2) and c_t^2 (1) enter 2 d - 1 <= 7 fused steps, each off by at
+// most u M; the group's number in its low bits moves it by less than 2 groups u M.  Distance: d + 3 <= 7 roundings of
+// non-negative terms, 8 u M.  So a centroid that the exact sequence prefers to the best scored one scores within
+//   2 (12 + 8 + 2 groups) u M of it, M the larger of the two; kGapBase, kGapGroup: a fifth more.  (The group's number only with
+// TOP2, below.)
+// And |c_t| <= |x_t| + |x_t - c_t| gives M <= 5 X + 5 d, X = sum_t r_t x_t^2, for each of them, with d within 17 u of the best
+// scored centroid's, which is its score plus X.  (With the block's largest |c| in that bound's place one far centroid left every
+// vector of its block undecided: 4096 x 4096, 64 2-D entries, weighted, one of them at 30 sigma 270 us, now 145 as without it.)
+constexpr float kGapBase = 5.f * 48.f / 16777216.f, kGapGroup = 5.f * 5.f / 16777216.f;
 
 // shared memory: tables of E / 8 groups; a group = 4 pairs of centroids, a pair = (c_t[m], c_t[m + 1]) for every t, and 16
 // bytes of padding, so that 8 lanes reading 8 different groups hit different banks; then max |c| of each table
@@ -180,7 +187,8 @@ __device__ __forceinline__ void load_pair(uint64_t (&c)[D], const unsigned char*
   }
 }
 
-template <int D, bool HD>
+// TOP2: the two best groups are kept, with the group's number in the low bits of its score; else the best group only.
+template <int D, bool HD, bool TOP2>
 __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_kernel(const AssignArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int GB = group_bytes<D>();
@@ -213,6 +221,51 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
     }
   }
   __syncthreads();
+  // An entry equal to one of lower index is never the answer: it becomes NaN, which both passes leave aside.  (As a tie with its
+  // twin it would send every vector near the two to the exact sequence over all groups: 4096 x 4096, 64 2-D entries, weighted, a
+  // quarter of them zero 215 us, now 146.)
+  if (a.find_equal) {
+    uint32_t equal = 0;   // (1024 entries at most: four a thread)
+    const int n_ent = n_tab * a.entries;
+    for (int o = tid, k = 0; o < n_ent; o += 32 * kWarps, ++k) {
+      const unsigned char* tab = smem + (o >> a.b) * table_bytes;
+      const int m = o & (a.entries - 1);
+      const float* own = reinterpret_cast<const float*>(tab + (m / kGroup) * GB + (m % kGroup / 2) * (D * 8));
+      float me[D];
+#pragma unroll
+      for (int t = 0; t < D; ++t) me[t] = own[2 * t + (m & 1)];
+      bool eq = false;
+      auto compare = [&](const unsigned char* pair, bool upper) {
+        uint64_t c[D];
+        load_pair<D>(c, pair);
+        bool eq_lo = true, eq_hi = upper;
+#pragma unroll
+        for (int t = 0; t < D; ++t) {
+          float lo, hi;
+          unpack2(c[t], lo, hi);
+          eq_lo = eq_lo && lo == me[t];
+          eq_hi = eq_hi && hi == me[t];
+        }
+        eq = eq || eq_lo || eq_hi;
+      };
+      for (int g = 0; g < m / kGroup; ++g) {
+#pragma unroll
+        for (int p = 0; p < kGroup / 2; ++p) compare(tab + g * GB + p * (D * 8), true);
+      }
+      for (int p = 0; p < m % kGroup / 2; ++p) compare(tab + (m / kGroup) * GB + p * (D * 8), true);
+      if (m & 1) compare(reinterpret_cast<const unsigned char*>(own), false);
+      if (eq) equal |= 1u << k;
+    }
+    __syncthreads();
+    for (int o = tid, k = 0; o < n_ent; o += 32 * kWarps, ++k)
+      if (equal >> k & 1) {
+        const int m = o & (a.entries - 1);
+        float* p = reinterpret_cast<float*>(smem + (o >> a.b) * table_bytes + (m / kGroup) * GB + (m % kGroup / 2) * (D * 8)) + (m & 1);
+#pragma unroll
+        for (int t = 0; t < D; ++t) p[2 * t] = __int_as_float(0x7fc00000);
+      }
+    __syncthreads();
+  }
 
   const int grp = blockIdx.x * 32 + lane;   // group of 8 indices within the row
   if (grp >= a.groups) return;
@@ -253,33 +306,53 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
 
       // ---- rank the groups ----
       uint64_t ca[V][D], cr[V][D];   // (-2 r_t x_t) and r_t, twice each
-      float best[V], second[V], gap[V];
+      float best[V], second[V], third[V], xx[V];
       int gi[V];
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        float m = 0.f;
-        bool usable = true;
+        float sq = 0.f;
+        if constexpr (!HD) {
 #pragma unroll
-        for (int t = 0; t < D; ++t) {
-          const float rt = HD && t > 0 ? __fdiv_rn(dw[v][t], dw[v][0]) : 1.f;
-          const float at = -2.f * rt * x[v][t], reach = fabsf(x[v][t]) + c_max;
-          ca[v][t] = pack2(at, at);
-          cr[v][t] = pack2(rt, rt);
-          m += rt * reach * reach;
-          usable = usable && (!HD || dw[v][t] >= 0.f);
+          for (int t = 0; t < D; ++t) {
+            const float at = -2.f * x[v][t];
+            ca[v][t] = pack2(at, at);
+            sq += x[v][t] * x[v][t];
+          }
+          // infinity or NaN among the values: NaN, which makes the exact sequence run over all centroids.  (Values are multiples
+          // of 2^-24 below 2^23, so that nothing else overflows or underflows.)
+          xx[v] = sq + c_max < 1e30f ? sq : __int_as_float(0x7fc00000);
+        } else {
+          float m = 0.f, base = dw[v][0], far = 0.f;
+          bool usable = true;
+          if (base == 0.f) {   // a first weight of zero counts as 2^-40 of the largest, and the gap takes in what that adds
+#pragma unroll
+            for (int t = 1; t < D; ++t) base = fmaxf(base, dw[v][t] * 0x1p-40f);
+            far = (fabsf(x[v][0]) + c_max) * (fabsf(x[v][0]) + c_max);
+          }
+#pragma unroll
+          for (int t = 0; t < D; ++t) {
+            const float rt = t > 0 ? __fdiv_rn(dw[v][t], base) : 1.f;
+            const float at = -2.f * rt * x[v][t], reach = fabsf(x[v][t]) + c_max;
+            ca[v][t] = pack2(at, at);
+            cr[v][t] = pack2(rt, rt);
+            m += rt * reach * reach;
+            sq += rt * x[v][t] * x[v][t];
+            usable = usable && dw[v][t] >= 0.f;
+          }
+          // in range, so that no term overflows or underflows to where the bounds above do not hold; what single terms lose to
+          // underflow is less than the gap that 1e-30 over the weights' base adds
+          const float dm = base * m;
+          usable = usable && base > 0.f && m > 1e-30f && m < 1e30f && dm > 1e-30f && dm < 1e30f;
+          sq += 1e-30f + __fdividef(1e-30f, base) + far * (2.f / kGapBase);
+          xx[v] = usable ? sq : __int_as_float(0x7fc00000);
         }
-        // in range, so that no term overflows or underflows to where the bounds above do not hold (else: NaN, which makes the
-        // exact sequence run over all centroids)
-        const float dm = HD ? dw[v][0] * m : m;
-        usable = usable && (!HD || dw[v][0] > 0.f) && m > 1e-30f && m < 1e30f && dm > 1e-30f && dm < 1e30f;
-        gap[v] = usable ? kGap * m : __int_as_float(0x7fc00000);
-        best[v] = second[v] = __int_as_float(0x7f800000);
+        best[v] = second[v] = third[v] = __int_as_float(0x7f800000);
         gi[v] = 0;
       }
       for (int g = 0; g < groups; ++g) {
         float gm[V];
 #pragma unroll
-        for (int v = 0; v < V; ++v) gm[v] = __int_as_float(0x7f800000);
+        for (int v = 0; v < V; ++v) gm[v] = __int_as_float(0x7f7fffff);   // (a group of NaN: finite with any number in its low bits)
 #pragma unroll
         for (int p = 0; p < kGroup / 2; ++p) {
           uint64_t c[D], q[D];
@@ -305,16 +378,28 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
         }
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-          second[v] = fminf(second[v], fmaxf(best[v], gm[v]));
-          gi[v] = gm[v] < best[v] ? g : gi[v];
-          best[v] = fminf(best[v], gm[v]);
+          float k = gm[v];
+          if constexpr (TOP2) {
+            k = __int_as_float((__float_as_int(k) & ~(groups - 1)) | g);
+            third[v] = fminf(third[v], fmaxf(second[v], k));
+          } else {
+            gi[v] = k < best[v] ? g : gi[v];
+          }
+          second[v] = fminf(second[v], fmaxf(best[v], k));
+          best[v] = fminf(best[v], k);
         }
       }
 
-      // ---- the exact sequence over the group that holds the winner (or over all) ----
+      // ---- the exact sequence over the groups that can hold the winner, in order ----
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        const bool sure = second[v] > best[v] + gap[v];
+        const float limit = best[v] + (kGapBase + (TOP2 ? kGapGroup * groups : 0.f)) * (xx[v] + fmaxf(best[v] + xx[v], 0.f));
+        int g1 = gi[v], g2 = 0, count = second[v] > limit ? 1 : groups;
+        if constexpr (TOP2) {
+          g1 = __float_as_int(best[v]) & (groups - 1);
+          g2 = __float_as_int(second[v]) & (groups - 1);
+          count = second[v] > limit ? 1 : third[v] > limit ? 2 : groups;
+        }
         uint64_t x2[D], d2[D];
 #pragma unroll
         for (int t = 0; t < D; ++t) {
@@ -323,9 +408,9 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
         }
         float bd = __int_as_float(0x7f800000);   // +inf
         int bi = 0;
-        const int g1 = sure ? gi[v] + 1 : groups;
 #pragma unroll 1
-        for (int g = sure ? gi[v] : 0; g < g1; ++g) {
+        for (int i = 0; i < count; ++i) {
+          const int g = count == 1 ? g1 : !TOP2 || count == groups ? i : i == 0 ? min(g1, g2) : max(g1, g2);
 #pragma unroll
           for (int p = 0; p < kGroup / 2; ++p) {
             uint64_t c[D];
@@ -398,7 +483,7 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
   const size_t smem = static_cast<size_t>(a.br_per_tile) * a.bc_per_seg * g.entries * g.d * sizeof(float);
   if (smem > 96 * 1024) return VQ_ERR_UNSUPPORTED;
   const dim3 grid((a.groups + 31) / 32, (g.N + kRows - 1) / kRows, 1);
-  static int attr_set[kMaxDevices][9] = {};
+  static int attr_set[kMaxDevices][13] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return VQ_ERR_CUDA;
   auto launch = [&](auto kern, int slot, size_t smem) {
@@ -409,15 +494,24 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
     kern<<<grid, 32 * kWarps, smem, s>>>(a);
     return check_launch();
   };
-  // Two passes from 32 entries on, and for 16 without weights in more than one dimension: with two groups the exact
-  // sequence still runs over half of the centroids.  us, one pass / two (4096 x 4096 if not said): 64 2-D entries on 11008
-  // rows, weighted 572/375, not 564/285; 32 2-D 119/104, 113/76; 256 4-D 724/468, 710/322; 16 2-D 67/82, 64/58; 16 1-D 81/91, 81/83.
+  // Which kernel: the faster one.  us, one pass / two passes on 4096 x 4096, weighted and not: 16 2-D entries 66/- 63/60, 4-D 70/-
+  // 54/49, 1-D 80/91 80/83; 32 1-D 137/131 137/115, 2-D 115/100 110/72, 4-D 114/143 99/66; 64 1-D 257/193 257/177, 2-D 215/145
+  // 211/109, 4-D 201/185 186/102; 128 1-D 497/366 497/339, 2-D 412/236 408/187, 4-D 374/277 360/175; 256 1-D 976/1130 975/1060
+  // (neighbours closer than the gap), 2-D 808/420 805/345, 4-D 723/468 709/321.
   const int n_tab = a.br_per_tile * a.bc_per_seg;
   const size_t smem2 = static_cast<size_t>(n_tab) * (g.entries / kGroup * (kGroup * g.d * 4 + 16) + 4);
-  if ((g.entries >= 32 || (g.entries == 16 && g.d > 1 && !hdiag)) && smem2 <= 96 * 1024) {
-    if (g.d == 1) return hdiag ? launch(assign_two_pass_kernel<1, true>, 3, smem2) : launch(assign_two_pass_kernel<1, false>, 4, smem2);
-    if (g.d == 2) return hdiag ? launch(assign_two_pass_kernel<2, true>, 5, smem2) : launch(assign_two_pass_kernel<2, false>, 6, smem2);
-    return hdiag ? launch(assign_two_pass_kernel<4, true>, 7, smem2) : launch(assign_two_pass_kernel<4, false>, 8, smem2);
+  const bool two = g.d == 1 ? g.entries >= 32 && g.entries <= 128 : g.d == 4 && hdiag ? g.entries >= 64 : g.entries >= (hdiag ? 32 : 16);
+  // The search for repeated entries grows with a tile's entries times those of a codebook, the ranking with the latter only.  us, not
+  // weighted: 4 of 61 for 32 codebooks of 16 2-D entries, 9 of 117 for 16 of 64 4-D ones, 1 of 109 for 4 of 64 2-D ones.  Not
+  // beyond that (a codebook per row and 256 columns: ties then cost up to 1.4 times the one-pass kernel's time).
+  a.find_equal = n_tab * g.entries <= (g.entries == 16 ? 512 : 1024);
+  if (two && smem2 <= 96 * 1024) {
+    const bool top2 = g.entries >= 128;
+    if (g.d == 1) return hdiag ? launch(assign_two_pass_kernel<1, true, true>, 3, smem2) : launch(assign_two_pass_kernel<1, false, true>, 4, smem2);
+    if (g.d == 2 && top2) return hdiag ? launch(assign_two_pass_kernel<2, true, true>, 5, smem2) : launch(assign_two_pass_kernel<2, false, true>, 6, smem2);
+    if (g.d == 2) return hdiag ? launch(assign_two_pass_kernel<2, true, false>, 7, smem2) : launch(assign_two_pass_kernel<2, false, false>, 8, smem2);
+    if (top2) return hdiag ? launch(assign_two_pass_kernel<4, true, true>, 9, smem2) : launch(assign_two_pass_kernel<4, false, true>, 10, smem2);
+    return hdiag ? launch(assign_two_pass_kernel<4, true, false>, 11, smem2) : launch(assign_two_pass_kernel<4, false, false>, 12, smem2);
   }
   if (g.d == 1) return launch(assign_kernel<1>, 0, smem);
   if (g.d == 2) return launch(assign_kernel<2>, 1, smem);

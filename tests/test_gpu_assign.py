@@ -53,6 +53,20 @@ def _special(spec, L, W, h):
     return W, h
 
 
+def _far(spec, L, W, h):
+    L.cb[:, 3] = 100 if spec.int8 else 1.0           # one centroid of every block far outside
+    return W, h
+
+
+def _dead(spec, L, W, h):
+    """First weights of zero, entries that differ in their first value alone, values that repeat."""
+    h = h.copy()
+    h[::8 * spec.d] = 0.0
+    L.cb[:, 1::3, 1:] = L.cb[:, :1, 1:]
+    L.cb[:, 5::8] = L.cb[:, 2:3]
+    return W, h
+
+
 def _assign(f, W, cb, scale, h):
     """The oracle's sequence; a distance that is no number is never the smaller one (index 0 if none is)."""
     C = cb.reshape(f.n_blocks, f.entries, f.d).astype(np.float32)
@@ -78,7 +92,7 @@ def _assign(f, W, cb, scale, h):
 
 
 @pytest.mark.parametrize("weighted", [False, True])
-@pytest.mark.parametrize("change", [_ties, _near, _small, _large, _overflow, _special], ids=lambda f: f.__name__[1:])
+@pytest.mark.parametrize("change", [_ties, _near, _small, _large, _overflow, _special, _far, _dead], ids=lambda f: f.__name__[1:])
 @pytest.mark.parametrize("spec", SPECS, ids=lambda s: s.name)
 def test_undecided_rankings(spec, change, weighted):
     import torch
