@@ -78,9 +78,10 @@ typedef enum {
  *   d_scale : binary16 [N][K/128]; w[n][k] = scale[n][k/128] * c.  K % 128 == 0.
  * vq_decode_weights decodes it with its tile kernel; the skinny GEMM runs in the tuned shared-codebook
  * kernels for 2-D formats with 5- or 6-bit indices (blocks of 32, 64 or a multiple of 128 rows and a
- * multiple of 128 columns, K a multiple of 256) and in the pair-table kernel for the block shapes that
- * one takes (see vq_impl); in both a looked-up pair is fp16(scale * c), the value vq_decode_weights
- * writes; other formats of this codebook type run in the format-generic kernel (VQ_IMPL_TUNED returns
+ * multiple of 128 columns, K a multiple of 256), for large layers and batches of 5- or 6-bit formats with
+ * blocks of a multiple of 32 rows in the tcgen05 kernel, and in the pair-table kernel for the block shapes
+ * that one takes (see vq_impl); in all of them a looked-up pair is fp16(scale * c), the value
+ * vq_decode_weights writes; other formats of this codebook type run in the format-generic kernel (VQ_IMPL_TUNED returns
  * VQ_ERR_UNSUPPORTED for them); vq_assign_indices does not take it. */
 typedef enum {
   VQ_CB_FP16 = 0,         /* binary16 entries                                                        */
@@ -100,10 +101,11 @@ typedef enum {
   VQ_IMPL_AUTO = 0,     /* tuned kernel when one covers the format/shape, else the generic one   */
   VQ_IMPL_GENERIC = 1,  /* format-generic fp32-FMA kernel (any valid format)                     */
   VQ_IMPL_TUNED = 2,    /* tuned kernel only; VQ_ERR_UNSUPPORTED if none covers the format/shape */
-  VQ_IMPL_STREAM = 3    /* the persistent tuned kernel only (the one AUTO picks for large per-row 4-bit
+  VQ_IMPL_STREAM = 3,   /* the persistent tuned kernel only (the one AUTO picks for large per-row 4-bit
                            layers and for groups at small batch); VQ_ERR_UNSUPPORTED if it does not cover
-                           the format.  (AUTO and TUNED also pick the tcgen05 kernel, vq_tile.cu, for large
-                           layers and batches.) */
+                           the format */
+  VQ_IMPL_TILE = 4      /* the tcgen05 kernel only (the one AUTO and TUNED pick for large layers and
+                           batches); VQ_ERR_UNSUPPORTED if it does not cover the format and batch */
 } vq_impl;
 
 /* Caller-filled description of one VQ-compressed matrix (paper Sec. 2.1 notation in comments). */
@@ -186,7 +188,8 @@ vq_status vq_gemm_small_batch_impl(const vq_format* fmt, const void* d_idx, cons
  *   d_X       : device binary16 [batch][K], shared by all members.
  * One kernel serves the whole group where the persistent, shared-codebook, pair-table or tcgen05
  * kernels cover the format (vq_grouped_kernel_launches tells); otherwise the members run one
- * after the other on `stream`.  Results are the same as n_members separate calls.
+ * after the other on `stream`.  The sums are those of n_members separate calls; where the group runs in
+ * another kernel than a member alone, they may be added in another order and round differently.
  * Errors: as vq_gemm_small_batch; SHAPE also if the rows do not add up to fmt->n_rows. */
 #define VQ_MAX_GROUP 4
 typedef struct {
@@ -198,8 +201,9 @@ typedef struct {
 } vq_group_member;
 vq_status vq_gemm_small_batch_grouped(const vq_format* fmt, const vq_group_member* members, int n_members,
                                       const void* d_X, int batch, void* d_ws, size_t ws_bytes, void* stream);
-/* Kernels a grouped call of this format launches: 1 (one kernel for the group) or n_members.
- * Host only; 0 for invalid arguments. */
+/* Kernels a grouped call of this format launches: 1 (one kernel for the group) or n_members.  It knows the
+ * members' rows together only: the answer holds for members of a multiple of 128 rows each (others may
+ * take as many as n_members).  Host only; 0 for invalid arguments. */
 int vq_grouped_kernel_launches(const vq_format* fmt, int n_members, int batch);
 
 /* Same computation with HOST activations and outputs: copies h_X (binary16 [batch][K]) to the

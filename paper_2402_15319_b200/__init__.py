@@ -2,7 +2,7 @@
 C-ABI library libvq_b200.so.  Importing the package loads nothing; the first call loads the
 shared library and raises if it has not been built."""
 from .binding import (  # noqa: F401
-    VQ_CB_FP16, VQ_CB_INT8_SCALED, VQ_CB_INT4_G128, VQ_IMPL_AUTO, VQ_IMPL_GENERIC, VQ_IMPL_TUNED, VQ_IMPL_STREAM,
+    VQ_CB_FP16, VQ_CB_INT8_SCALED, VQ_CB_INT4_G128, VQ_IMPL_AUTO, VQ_IMPL_GENERIC, VQ_IMPL_TUNED, VQ_IMPL_STREAM, VQ_IMPL_TILE,
     VQError, VQFormat, PackInfo, lib_path, load, exported_symbols,
     vq_norm_info, vq_decode_weights_normalized, vq_gemm_small_batch_normalized,
     vq_pack_info, vq_workspace_bytes, vq_workspace_bytes_host, vq_decode_weights, vq_gemv,

@@ -9,7 +9,7 @@ import os
 from dataclasses import dataclass
 
 VQ_CB_FP16, VQ_CB_INT8_SCALED, VQ_CB_INT4_G128 = 0, 1, 2
-VQ_IMPL_AUTO, VQ_IMPL_GENERIC, VQ_IMPL_TUNED, VQ_IMPL_STREAM = 0, 1, 2, 3
+VQ_IMPL_AUTO, VQ_IMPL_GENERIC, VQ_IMPL_TUNED, VQ_IMPL_STREAM, VQ_IMPL_TILE = 0, 1, 2, 3, 4
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_PKG, "libvq_b200.so")

@@ -173,12 +173,12 @@ vq_status vq_gemm_small_batch_impl(const vq_format* fmt, const void* d_idx, cons
   if (!aligned16(d_X) || !aligned16(d_Y)) return VQ_ERR_ALIGN;
   if (!d_ws || ws_bytes < vq_workspace_bytes(fmt, batch)) return VQ_ERR_WORKSPACE;
   if (!aligned16(d_ws)) return VQ_ERR_ALIGN;
-  if (impl != VQ_IMPL_AUTO && impl != VQ_IMPL_GENERIC && impl != VQ_IMPL_TUNED && impl != VQ_IMPL_STREAM) return VQ_ERR_UNSUPPORTED;
+  if (impl < VQ_IMPL_AUTO || impl > VQ_IMPL_TILE) return VQ_ERR_UNSUPPORTED;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const __half* X = static_cast<const __half*>(d_X);
   __half* Y = static_cast<__half*>(d_Y);
-  if (impl == VQ_IMPL_STREAM) {
-    if (g.cb_int4) return VQ_ERR_UNSUPPORTED;
+  if (impl == VQ_IMPL_STREAM || impl == VQ_IMPL_TILE) {
+    if (impl == VQ_IMPL_STREAM && g.cb_int4) return VQ_ERR_UNSUPPORTED;
     StreamCall call = {};
     call.g = g;
     call.n_seg = 1;
@@ -191,7 +191,7 @@ vq_status vq_gemm_small_batch_impl(const vq_format* fmt, const void* d_idx, cons
     call.batch = batch;
     call.ws = d_ws;
     call.ws_bytes = ws_bytes;
-    return launch_gemm_stream(call, s);
+    return impl == VQ_IMPL_STREAM ? launch_gemm_stream(call, s) : launch_gemm_tile(call, s);
   }
   if (impl != VQ_IMPL_GENERIC) {
     st = launch_gemm_tuned(g, p, X, Y, batch, d_ws, ws_bytes, s);

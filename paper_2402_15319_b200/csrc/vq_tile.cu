@@ -36,7 +36,7 @@
 // workspace; the CTA that draws the tile's last ticket adds them in CTA order (results do not depend on
 // timing) and resets the counter.
 //
-// Every wait is bounded; a wait that runs out increments a device counter, the role stops waiting for anything
+// Every wait on a barrier is bounded; a wait that runs out increments a device counter, the role stops waiting for anything
 // else and still arrives on every barrier it owes, so that the kernel ends.
 #include <cstdio>
 #include <cstdlib>
@@ -58,7 +58,7 @@ constexpr int kAStages = 3;           // decoded stages in tensor memory
 constexpr int kTmemCols = 128;        // 2 x 16 accumulator columns, 3 x 32 weight columns
 constexpr int kAOff = 32;
 constexpr int kDecodeWarps = 4, kThreads = 192;
-constexpr int kMaxDepth = 6;          // unit stages at most
+constexpr int kMaxDepth = 3;          // unit stages at most
 constexpr int kWaitTries = 1 << 18;
 constexpr int kPolls = 1 << 20;       // polls without progress before the producer gives up
 constexpr unsigned kPollSleep = 500;  // ns between polls of the producer
@@ -857,7 +857,7 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   int D = 2;
   for (; per_sm >= 2; --per_sm) {
     const size_t budget = (228 * 1024) / per_sm - 1024;
-    for (D = 3; D >= 2; --D)
+    for (D = kMaxDepth; D >= 2; --D)
       if (plan(D) <= budget) break;
     if (D >= 2) break;
   }
@@ -932,7 +932,7 @@ vq_status launch_nb(const StreamCall& call, cudaStream_t s) {
 
 }  // namespace
 
-// Codebook blocks that are whole units of columns (so K is one too).
+// Codebook blocks that are whole units of columns (so K is one too).  (Row tables: from batch 9 on only, see launch_gemm_tile.)
 bool tile_covers(const Geometry& g) {
   if (g.d == 2 && g.b == 4) return !g.cb_int4 && g.Bc % 256 == 0;
   if (g.d == 2 && g.b == 5) return g.Bc % 256 == 0 && (g.Br % 32 == 0 || (!g.cb_int4 && (g.Br == 4 || g.Br == 8 || g.Br == 16)));
@@ -974,7 +974,7 @@ bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
 vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {
   const Geometry& g = call.g;
   if (!tile_covers(g) || call.n_seg < 1 || call.n_seg > kMaxSegments) return VQ_ERR_UNSUPPORTED;
-  if (g.d == 2 && g.b == 4) return launch_nb<Fmt<2, 4, kRow, 1, false>>(call, s);
+  if (g.d == 2 && g.b == 4) return call.batch <= 8 ? VQ_ERR_UNSUPPORTED : launch<Fmt<2, 4, kRow, 1, false>, 16>(call, s);
   if (g.d == 4) return launch_nb<Fmt<4, 8, kCta, 128, false>>(call, s);
   if (g.Br % kTileRows == 0) {
     if (g.b == 6) return g.cb_int4 ? launch_nb<Fmt<2, 6, kCta, 128, true>>(call, s) : launch_nb<Fmt<2, 6, kCta, 128, false>>(call, s);

@@ -88,6 +88,30 @@ class DeviceLayer:
         return dW.cpu().numpy()
 
 
+def kernels_launched(call):
+    """Names of the kernels that call() launches, in order (captured in a graph, not run)."""
+    import torch
+    from cuda.bindings import driver
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    handle = driver.CUgraph(graph.raw_cuda_graph())
+
+    def ok(result):
+        assert result[0] == driver.CUresult.CUDA_SUCCESS, result
+        return result[1:]
+
+    (_, count) = ok(driver.cuGraphGetNodes(handle))
+    (nodes, _) = ok(driver.cuGraphGetNodes(handle, count))
+    names = []
+    for node in nodes[:count]:
+        if ok(driver.cuGraphNodeGetType(node))[0] == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            p = ok(driver.cuGraphKernelNodeGetParams(node))[0]
+            name = ok(driver.cuKernelGetName(p.kern) if int(p.kern) else driver.cuFuncGetName(p.func))[0]
+            names.append(name.decode())
+    return names
+
+
 def assert_outputs_close(Y_gpu: np.ndarray, Y_ref: np.ndarray, A_ref: np.ndarray, what=""):
     """The acceptance bound: per element |y_gpu - y_ref| <= 1e-3 * sum_k |W x|."""
     assert Y_gpu.shape == Y_ref.shape, (Y_gpu.shape, Y_ref.shape)

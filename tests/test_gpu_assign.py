@@ -15,6 +15,8 @@ SPECS = [
     vq_synth.LayerSpec("d2b4", N=36, K=1024, d=2, b=4, Br=4, Bc=512, int8=False),
     vq_synth.LayerSpec("d2b6", N=64, K=512, d=2, b=6, Br=32, Bc=128, int8=False),
     vq_synth.LayerSpec("d2b8", N=64, K=512, d=2, b=8, Br=64, Bc=256, int8=True),
+    vq_synth.LayerSpec("d1b6", N=40, K=512, d=1, b=6, Br=8, Bc=256, int8=False),
+    vq_synth.LayerSpec("d4b6", N=64, K=1024, d=4, b=6, Br=32, Bc=512, int8=False),
     vq_synth.LayerSpec("d4b5", N=36, K=1024, d=4, b=5, Br=4, Bc=256, int8=False),
     vq_synth.LayerSpec("d4b8", N=64, K=1024, d=4, b=8, Br=64, Bc=512, int8=True),
 ]
