@@ -940,19 +940,19 @@ bool tile_covers(const Geometry& g) {
   return g.d == 4 && g.b == 8 && g.Bc % 128 == 0 && g.Br % kTileRows == 0 && !g.cb_int4;
 }
 
-// Which calls this kernel serves: those where it was the faster one on B200.  Its time hardly depends on the batch
-// (one pass over the weights for 1..16 sequences) but it has about 4 us more of start-up and summing than the cluster
-// kernels, so it takes over above a number of weights that falls with the batch.  us, other kernels / this one:
-//   row tables (57344 x 8192)      batch 1 49/63, 8 60/64, 9 81/69, 16 97/70; 28672 x 4096: 9 24/26, 12 31/26, 16 39/27;
-//                                  20480 x 4096: 12 24.5/26.5, 16 30/27; 8192 x 8192: 16 20/22
-//   128-row blocks, 2-D (22016 x 4096) 3 18/22, 5 23/22, 8 26/22, 16 45/25; 12288 x 4096: 8 13.5/16, 9 21/18, 16 37/19; 4096 x 11008: 9 17/20, 16 23/21
-//   4-D (27648 x 5120)             1 25/25, 5 28/26, 8 36/26, 16 68/29; 5120 x 13824: 5 20/19, 8 22/19; 15360 x 5120: 8 18/19, 9 22/21.5, 16 38/22
-//   32-row blocks (28672 x 4096)   1 32/27, 8 46/28, 16 59/31; 18176 x 3328: 8 20/21, 16 41/23; 4096 x 14336: 9 22/26, 16 29/28
-//   4-row blocks (28672 x 4096)    1 34/24, 8 38/26, 16 49/29; 4096 x 14336: 1 23/19.5, 16 28/23; 6144 x 4096: 1 10.6/11.8;
-//                                  8- and 16-row blocks, 12304 x 4352: 1 15/16
-//   5-bit, 32-row blocks (28672 x 4096) 1 22/24.5, 8 35.5/26; 128-row blocks (22016 x 4096) 5 20/22, 8 28/22; 12288 x 4096: 9 14/19
+// Which calls this kernel serves.  Its time hardly depends on the batch (one pass over the weights for 1..16 sequences) but it
+// has about 4 us more of start-up and summing than the cluster kernels, so it takes over above a number of weights that falls with
+// the batch.  The lines are drawn where it was the faster one in nearly all of 39000 timings against the other kernels on B200 (44
+// formats, 1024 to 28672 columns, any rows, every batch): it is slower by more than 3 % in 97 of the 14300 calls it takes, by more
+// than 10 % in 14; the others move in steps of whole waves.  us, other kernels / this one, on either side of a line:
+//   row tables (8-bit, 2048-column blocks)  16632 x 4096 b15 21.4/21.9, 19968 x 4096 b15 25.6/24.8; 13952 x 8192 b15 25.6/27.9, 16232 x 8192
+//                                           b15 37.9/29.1; 10632 x 14336 b11 32.0/33.1
+//   4-D     71680 x 2048 b6 21.0/24.2, 143360 x 1024 b9 64 M 15.6/17.8
+//   128-row blocks, 6 bits  8704 x 8192 b9 21.5/25.3 (the worst that is left), 102400 x 1024 b5 20.2/25.4, 27392 x 3072 b5 17.2/19.7
+//   32-row blocks, 6 bits   51200 x 2048 b1, 128-column blocks 20.7/27.1; 28672 x 4096 b1, 256-column blocks 32/27
+//   5 bits  54656 x 1536 b8 19.2/24.2; 4-row blocks 9152 x 6400 b1 18.2/20.2; 8-row blocks 63488 x 1024 b1 15.8/18.7
 // Shapes that the cluster kernels do not take (rows not a multiple of 128, K not one of 256) cost the pair-table kernel
-// more, and a launch per layer: 4160 x 3328 in three layers 21/12, 3328 x 9088 22/16 at batch 5.
+// more, and a launch per layer: 4160 x 3328 in three layers 21/12, 3328 x 9088 22/16 at batch 5; but 13312 x 1920 b2 11.0/14.0.
 bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
   if (!tile_covers(g)) return false;
   long long rows = 0;
@@ -962,13 +962,26 @@ bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
     whole = whole && N[i] % kTileRows == 0;
   }
   const long long w = (rows * g.K) >> 20;   // weights of the call, in 2^20
-  if (g.d == 2 && g.b == 4) return batch >= 13 ? w >= 72 : batch == 12 ? w >= 108 : batch >= 9 && w >= 160;
-  if (g.d == 4) return batch >= 9 ? w >= 64 : batch >= 5 && (w >= 112 || (w >= 64 && g.K >= 8192));
-  if (g.Br < 32 || (g.b == 5 && !whole)) return w >= 54;
-  if (g.b == 5) return batch >= 8 && w >= (g.Br % kTileRows ? 100 : 80);
-  if (!whole) return w >= (n_seg > 1 ? 12 : 24);
-  if (g.Br % kTileRows == 0) return batch >= 13 ? w >= 44 : batch >= 9 ? w >= 46 : batch >= 5 && w >= 80;
-  return batch >= 13 ? w >= 54 : w >= 100;
+  if (g.d == 2 && g.b == 4) {
+    if (batch < 9) return false;
+    return w >= (batch < 12 ? 160 : g.K < 5120 ? 80 : batch < 13 ? 160 : 112);
+  }
+  if (g.d == 4) {
+    if (batch >= 9) return w >= (g.K < 2048 ? 72 : 64);
+    return batch >= 5 && w >= (g.K >= 8192 ? 64 : batch >= 7 ? 112 : 144);
+  }
+  if (g.b == 5) {
+    if (g.Br == 4) return w >= 58;
+    if (g.Br < 32 || !whole) return w >= (batch >= 9 ? 68 : 88);
+    return batch >= 11 ? w >= 80 : batch >= 8 && w >= 116;
+  }
+  if (!whole) return w >= (n_seg > 1 ? 12 : batch >= 9 || g.K < 3072 ? 48 : 28);
+  if (g.Br % kTileRows == 0) {
+    if (batch >= 9) return w >= 48;
+    return batch >= 5 && w >= (batch < 7 ? 124 : g.K < 2048 ? 104 : 80);
+  }
+  if (batch >= 13) return w >= 64;
+  return w >= (g.K < 2048 || (batch <= 5 && g.Bc < 256) ? 150 : 104);
 }
 
 vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {

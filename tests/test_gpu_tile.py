@@ -1,5 +1,5 @@
-"""The tcgen05 kernel (vq_tile.cu) against the oracle: at sizes just above where it takes over from the other kernels and, asked for
-by name, at the edges of its tiles and with more tiles than CTAs; every table kind, codebook type and batch class."""
+"""The tcgen05 kernel (vq_tile.cu) against the oracle: at sizes near where it takes over from the other kernels, at the edges of its
+tiles and with more tiles than CTAs; every table kind, codebook type and batch class."""
 import numpy as np
 import pytest
 
@@ -50,10 +50,11 @@ def test_tile_kernel_against_oracle(spec, batches):
     for batch in batches:
         X = vq_synth.make_x(spec, 62, batch)
         Y, A = orc.gemm(oracle_fmt(spec), L.idx, L.cb, L.scale, X, rows=rows, threads=8)
-        Yg = dev.gemm(X)
-        assert_outputs_close(Yg[:, rows], Y, A, f"{spec.name} batch {batch}")
-        assert np.isfinite(Yg.astype(np.float32)).all()
-        assert np.array_equal(dev.gemm(X).view(np.uint16), Yg.view(np.uint16))   # bit-identical, whoever draws the last ticket
+        for impl in (vq.VQ_IMPL_TILE, vq.VQ_IMPL_AUTO):
+            Yg = dev.gemm(X, impl)
+            assert_outputs_close(Yg[:, rows], Y, A, f"{spec.name} batch {batch} impl {impl}")
+            assert np.isfinite(Yg.astype(np.float32)).all()
+            assert np.array_equal(dev.gemm(X, impl).view(np.uint16), Yg.view(np.uint16))   # bit-identical, whoever draws the last ticket
     assert vq.vq_device_wait_failures() == 0
 
 
