@@ -1,5 +1,5 @@
-"""vq_decode_weights at the sizes where its tile changes: 8 rows, 16 where the codebooks outweigh a row, 32 where the grid would
-be too tall."""
+"""vq_decode_weights at the sizes where its tile changes: 8 rows, 16 where the codebooks outweigh a row, 16 and 32 where the grid
+would be too tall."""
 import numpy as np
 import pytest
 
@@ -25,14 +25,15 @@ def test_decode_bit_exact(spec):
     assert np.array_equal(DeviceLayer(spec, L).decode().view(np.uint16), W16)
 
 
-def test_more_rows_than_a_grid_of_small_tiles_holds():
+@pytest.mark.parametrize("times,d,b", [(8200, 1, 2), (16400, 2, 6)], ids=["16 rows", "32 rows"])   # 524,800 and 1,049,600 rows
+def test_more_rows_than_a_grid_of_small_tiles_holds(times, d, b):
     import torch
-    times, K = 8200, 256
-    part = vq_synth.LayerSpec("part", N=64, K=K, d=1, b=2, Br=64, Bc=256, int8=True)
+    K = 256
+    part = vq_synth.LayerSpec("part", N=64, K=K, d=d, b=b, Br=64, Bc=256, int8=True)
     L = draw(part, 43)
     dev = DeviceLayer(part, L)
     want = torch.from_numpy(dev.decode().view(np.int16)).cuda()
-    tall = vq_synth.LayerSpec("tall", N=64 * times, K=K, d=1, b=2, Br=64, Bc=256, int8=True)   # 524,800 rows
+    tall = vq_synth.LayerSpec("tall", N=64 * times, K=K, d=d, b=b, Br=64, Bc=256, int8=True)
     W = torch.empty((tall.N, K), dtype=torch.float16, device="cuda")
     rep = [t.repeat(times, *[1] * (t.dim() - 1)) for t in (dev.idx, dev.cb, dev.scale)]
     torch.cuda.synchronize()
