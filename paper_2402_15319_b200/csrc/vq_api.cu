@@ -179,6 +179,7 @@ vq_status vq_gemm_small_batch_impl(const vq_format* fmt, const void* d_idx, cons
   __half* Y = static_cast<__half*>(d_Y);
   if (impl == VQ_IMPL_STREAM || impl == VQ_IMPL_TILE) {
     if (impl == VQ_IMPL_STREAM && g.cb_int4) return VQ_ERR_UNSUPPORTED;
+    if (impl == VQ_IMPL_TILE && g.d == 2 && g.b == 4 && batch <= 8) return VQ_ERR_UNSUPPORTED;   // (by name from batch 9 on only)
     StreamCall call = {};
     call.g = g;
     call.n_seg = 1;

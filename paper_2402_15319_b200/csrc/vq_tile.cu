@@ -5,36 +5,35 @@
 // What bounds it.  Every pair of weights costs one 32-bit shared-memory gather, 32 of them a clock and SM: 64
 // weights / clk / SM at most.  So everything else is kept off the shared-memory port and out of the gathering warps:
 // activations are never loaded by a warp (the tensor core reads them from shared memory as the B operand), the
-// decoded tile goes from registers to tensor memory by tcgen05.st, which has its own path (gathers alone ran at
-// 63.0 weights / clk / SM in a probe on resident data, with the stores 60.7, with the products 48.4), and the
+// decoded tile goes from registers to tensor memory by tcgen05.st, which has its own path, and the
 // accumulators live in tensor memory, which leaves registers for 16 gathering warps per SM.
-// Measured: 57344 x 8192, 2-D 4-bit, 16 sequences 96.6 us in the persistent mma.sync kernel, 72.2 here (23 weights / clk / SM: a
-// stage takes about 170 instructions a warp where its gathers need 77, four warps a scheduler issue 57 % of the time).
 //
-// Work.  The rows of a call's layers ("segments") are cut into tiles of 128 rows, a tile's columns into units of
-// UC.  The grid is persistent, four CTAs per SM at most; every CTA takes q whole tiles, and the units
-// of the tiles left over form one sequence that is cut into equal contiguous pieces, one per CTA.  A CTA walks its
-// piece first, so that shared tiles are summed while everyone still computes whole ones.
+// Work.  One persistent CTA per SM.  The rows of a call's layers ("segments") are cut into tiles of 128 rows, a tile's columns
+// into units of UC, four units make a step: one for each of the CTA's four quads of decoding warps, which split the columns of
+// a tile among them.  A CTA takes q whole tiles; the steps of the tiles left over form one sequence that is cut into equal
+// contiguous pieces, one per CTA, walked first, so that shared tiles are summed while everyone still computes whole
+// ones.  (With four CTAs of one quad each per SM a tile was shared by four times as many CTAs, whose sums met in the workspace.)
 //
-// Roles (192 threads).  Warps 0..3 decode: thread = weight row = lane of tensor memory.  A thread reads its row's
-// indices of a unit from the stage the producer filled, looks up 32 pairs (64 columns) and stores them as
-// 32 columns of tensor memory; three such stages are in flight.  Warp 4 (one thread) produces: index and
-// activation boxes by TMA; index boxes run ahead of the programmatic-dependency wait, activations come after it.
-// Warp 5 issues the products (one elected lane, warp-uniform control flow: with a divergent branch in place of
-// elect.sync an issue took five times as long) and owns the tensor memory.
+// Roles (672 threads).  Warps 0..15 decode, four to a quad: thread = weight row = lane of tensor memory.  A thread reads its
+// row's indices of a unit from the stage the copy engine filled, looks up 32 pairs (64 columns) and stores them as
+// 32 columns of tensor memory, of which the quad has two such stages.  Warps 16..19 serve a quad each: they request its index and
+// activation boxes by TMA (index boxes run ahead of the programmatic-dependency wait, activations come after it) and issue its
+// products (one elected lane, warp-uniform control flow: with a divergent branch in place of elect.sync an issue took
+// five times as long).  Warp 20 owns the tensor memory, adds the quads' sums and stores outputs or shares of them.
 //
 // Tables.  One 32-bit word per entry and lane, bank = lane: no conflicts whatever the indices.  Three kinds:
-//   row  : 16 entries of the lane's own row, two tables per warp (256-byte entry pitch), so that the index byte
-//          enters the address by one byte permute and the next block's table is written beside the current one;
+//   row  : 16 entries of the lane's own row; two warps' tables alternate (256-byte entry pitch), so that the index byte
+//          enters the address by one byte permute;
 //   warp : blocks of 4, 8, 16 or a multiple of 32 rows, every warp replicates its own rows' codebooks;
-//   CTA  : blocks of a multiple of 128 rows, one table for the four warps.
+//   CTA  : blocks of a multiple of 128 rows, one table for the four warps of a quad.
 // 8-bit codebooks with row tables keep the entries as exact integers in fp16 and multiply the fp32 sums of a block by its
 // scale; the other tables hold fp16(scale * c), the value vq_decode_weights writes.  4-bit codebooks multiply
 // the looked-up pair by the scale of the row and its group of 128 columns, the same value again.
 //
-// Sums.  A tile whose units all belong to one CTA is rounded to fp16 and stored.  A shared tile's parts go to the
-// workspace; the CTA that draws the tile's last ticket adds them in CTA order (results do not depend on
-// timing) and resets the counter.
+// Sums.  Each quad accumulates into its own columns of tensor memory and hands its sums over through shared memory, where the
+// results warp adds them in quad order.  A tile whose steps all belong to one CTA is rounded to fp16 and stored.  A shared
+// tile's parts go to the workspace; the CTA that draws the tile's last ticket adds them in CTA order when it has done its own
+// work (results do not depend on timing) and resets the counter.
 //
 // Every wait on a barrier is bounded; a wait that runs out increments a device counter, the role stops waiting for anything
 // else and still arrives on every barrier it owes, so that the kernel ends.
@@ -53,15 +52,14 @@ using namespace dev;
 
 constexpr int kTileRows = 128;
 constexpr int kStageCols = 64;        // columns a thread decodes between two hand-overs to the tensor core
-constexpr int kStageTmem = 32;        // ... and the tensor-memory columns they take
-constexpr int kAStages = 3;           // decoded stages in tensor memory
-constexpr int kTmemCols = 128;        // 2 x 16 accumulator columns, 3 x 32 weight columns
-constexpr int kAOff = 32;
-constexpr int kDecodeWarps = 4, kThreads = 192;
-constexpr int kMaxDepth = 3;          // unit stages at most
+constexpr int kQuads = 4;             // groups of four decoding warps
+constexpr int kDecodeWarps = 4 * kQuads, kResultsWarp = kDecodeWarps + kQuads, kThreads = 32 * (kResultsWarp + 1);
+constexpr int kAStages = 2;           // decoded stages of a quad in tensor memory, 32 columns each
+constexpr int kTmemCols = 512;        // per quad 2 x 16 accumulator columns, then per quad 2 x 32 weight columns
+constexpr int kAOff = 32 * kQuads;
+constexpr int kMaxDepth = 4;          // unit stages of a quad at most
 constexpr int kWaitTries = 1 << 18;
-constexpr int kPolls = 1 << 20;       // polls without progress before the producer gives up
-constexpr unsigned kPollSleep = 500;  // ns between polls of the producer
+constexpr int kBarBytes = 640;        // barriers and the words beside them
 constexpr uint32_t kMagic = 0x64646464u;   // high byte of fp16 1024.0
 constexpr uint32_t kBias2 = 0x64806480u;   // fp16 pair (1152, 1152)
 // tcgen05.mma kind::f16: D fp32, A and B fp16, both K-major, N = 16, M = 128
@@ -84,13 +82,13 @@ struct TileArgs {
   int* ws_ticket;     // [tile], zero between calls
   int* error_flag;
   int K, batch;
-  int S;              // units per tile
+  int S, steps;       // units and steps (of a unit per quad) of a tile
   int q;              // whole tiles per CTA
-  int tail_units, tail_ctas;   // units of the left-over tiles and the CTAs that share them
+  int tail_tile0, tail_steps, tail_ctas;   // the tiles left over and the CTAs that share their steps
   int blocks_per_row, Br, Bc, cb_int8;
-  int D;              // unit stages
-  int x_bytes, x_row_bytes;    // activation stage; bytes of one 64-column group of it
-  int idx_off, bar_off, front_bytes;   // dynamic shared memory: x stages, index stages, barriers, | tables
+  int D;              // unit stages of a quad
+  int x_bytes, x_row_bytes;    // activations of a unit; bytes of one 64-column group of them
+  int idx_off, red_off, bar_off, front_bytes;   // dynamic shared memory: activations, indices, sums, barriers, | tables
 };
 
 struct TileMaps {
@@ -104,30 +102,25 @@ struct Fmt {
   static constexpr int D = D_, B = B_, TK = TK_, BR = BR_;
   static constexpr bool I4 = I4_;
   static constexpr int E = 1 << B;
-  // Columns of a unit: 256 where a row of 128 is no whole number of 16-byte pieces (5 bits) and for row tables (half as
-  // many unit changes: 69.5 against 73.6 us on 57344 x 8192 at batch 16), else 128 (more stages in flight).
+  // Columns of a unit: 256 where a row of 128 is no whole number of 16-byte pieces (5 bits) and for row tables, else 128.
   static constexpr int UC = TK == kRow || (128 * B / (8 * D)) % 16 != 0 ? 256 : 128;
   static constexpr int RB = UC * B / (8 * D);       // bytes of a row of a unit
   static constexpr int IDX_BYTES = kTileRows * RB;
   static constexpr int STAGES = UC / kStageCols;
-  static constexpr int TABLE = TK == kRow ? 4096 : E * 128;              // bytes of a warp's (CTA's) table
+  static constexpr int TABLE = TK == kRow ? 4096 : E * 128;   // row: of two warps, whose 128-byte entries alternate
   static constexpr int BUFS = TK == kCta && D == 2 ? 2 : 1;
-  static constexpr int TABLES = TK == kCta ? BUFS * TABLE : kDecodeWarps * TABLE;
+  static constexpr int TABLES = TK == kRow ? kDecodeWarps / 2 * TABLE : TK == kWarp ? kDecodeWarps * TABLE : kQuads * BUFS * TABLE;
   // OR-merged addresses need tables on multiples of their size; 4-D look-ups add (one per four weights)
   static constexpr int ALIGN = D == 4 ? 1024 : TABLE;
   static constexpr int SWIZZLE = RB == 32 ? 3 : RB == 64 ? 1 : RB == 128 ? 2 : 0;
+  // columns of sums that the quads hand over at a time from batch 9 on: all where sums are scaled per block, fewer where tables fill the memory
+  static constexpr int RC16 = TK == kRow ? 16 : TK == kWarp && B == 6 ? 4 : 8;
   static_assert(RB % 16 == 0 && (TK != kRow || (B == 4 && D == 2)));
 };
 
 // ---- small device helpers ------------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {   // has phase `parity` completed?
-  uint32_t done;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-               : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-  return done != 0;
 }
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {   // the same, blocking for a short time
   uint32_t done;
@@ -147,7 +140,7 @@ __device__ __forceinline__ void wait_phase(uint32_t bar, uint32_t parity, int& t
     }
   }
 }
-__device__ __forceinline__ void decode_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }   // the four decoding warps
+__device__ __forceinline__ void quad_barrier(int quad) { asm volatile("bar.sync %0, 128;" ::"r"(1 + quad) : "memory"); }
 __device__ __forceinline__ void tma_box_3d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, uint32_t bar) {
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                ::"r"(dst), "l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
@@ -208,6 +201,11 @@ __device__ __forceinline__ void tc_load(uint32_t addr, float (&v)[NB]) {
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
+__device__ __forceinline__ float lds32f(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ uint32_t mul_f16x2(uint32_t a, uint32_t b) {
   uint32_t r;
   asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
@@ -228,54 +226,74 @@ __device__ __forceinline__ uint32_t nibble_pair(uint32_t byte) {   // two signed
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// A CTA's walk over its units: its piece of the left-over tiles first, then its q whole tiles.
+// A CTA's walk over its fragments (steps [s0, s1) of one tile): its piece of the left-over tiles first, then its whole tiles.
 struct Walk {
-  int n, n_tail, t0, t1, slab, s, k, whole0, tail_tile0;
+  int tile, s0, s1, left, whole, whole_end;
+  bool valid;
 
-  __device__ __forceinline__ void init(const TileArgs& a, int c, int ctas) {
-    t0 = t1 = 0;
-    if (c < a.tail_ctas) {   // (the host keeps tail_units * tail_ctas below 2^31)
-      t0 = static_cast<int>(static_cast<unsigned>(a.tail_units) * static_cast<unsigned>(c) / static_cast<unsigned>(a.tail_ctas));
-      t1 = static_cast<int>(static_cast<unsigned>(a.tail_units) * static_cast<unsigned>(c + 1) / static_cast<unsigned>(a.tail_ctas));
+  __device__ __forceinline__ void init(const TileArgs& a, int c) {
+    int t0 = 0, t1 = 0;
+    if (c < a.tail_ctas) {   // (the host keeps tail_steps * tail_ctas below 2^31)
+      t0 = static_cast<int>(static_cast<unsigned>(a.tail_steps) * static_cast<unsigned>(c) / static_cast<unsigned>(a.tail_ctas));
+      t1 = static_cast<int>(static_cast<unsigned>(a.tail_steps) * static_cast<unsigned>(c + 1) / static_cast<unsigned>(a.tail_ctas));
     }
-    n_tail = t1 - t0;
-    n = n_tail + a.q * a.S;
-    whole0 = c * a.q;
-    tail_tile0 = a.q * ctas;
-    k = 0;
-    slab = whole0;
-    s = 0;
-    if (n_tail > 0) {
-      slab = tail_tile0 + t0 / a.S;
-      s = t0 % a.S;
+    whole = c * a.q;
+    whole_end = whole + a.q;
+    tile = a.tail_tile0 + t0 / a.steps - 1;
+    left = t1 - t0;
+    next(a, t0 % a.steps);
+  }
+  __device__ __forceinline__ void next(const TileArgs& a, int first = 0) {
+    valid = true;
+    s0 = 0;
+    s1 = a.steps;
+    if (left > 0) {
+      ++tile;
+      s0 = first;
+      s1 = min(a.steps, first + left);
+      left -= s1 - s0;
+    } else if (whole < whole_end) {
+      tile = whole++;
+    } else {
+      valid = false;
     }
   }
-  __device__ __forceinline__ void next(const TileArgs& a) {
-    ++k;
-    if (k == n_tail) {
-      slab = whole0;
-      s = 0;
-    } else if (++s == a.S) {
-      s = 0;
-      ++slab;
+  __device__ __forceinline__ bool complete(const TileArgs& a) const { return s0 == 0 && s1 == a.steps; }
+  // units of the fragment that are quad k's
+  __device__ __forceinline__ void range(const TileArgs& a, int k, int& u, int& end) const {
+    const int u0 = kQuads * s0, n = min(kQuads * s1, a.S) - u0;
+    u = u0 + n * k / kQuads;
+    end = u0 + n * (k + 1) / kQuads;
+  }
+};
+// ... and over one quad's units, fragments without any left out.
+struct Units {
+  Walk f;
+  int u, end;
+  __device__ __forceinline__ void settle(const TileArgs& a, int k) {
+    while (u == end) {
+      f.next(a);
+      if (!f.valid) return;
+      f.range(a, k, u, end);
     }
   }
-  __device__ __forceinline__ bool slab_end(const TileArgs& a) const { return s == a.S - 1 || k == n_tail - 1; }
-  __device__ __forceinline__ int fragment_units(const TileArgs& a) const {   // of the current tile, from here on
-    return k < n_tail ? min(n_tail - k, a.S - s) : a.S - s;
+  __device__ __forceinline__ void init(const TileArgs& a, int c, int k) {
+    f.init(a, c);
+    if (!f.valid) return;
+    f.range(a, k, u, end);
+    settle(a, k);
   }
-  __device__ __forceinline__ bool complete(const TileArgs& a) const {   // does this CTA hold every unit of the tile?
-    if (k >= n_tail) return true;
-    const int first = (slab - tail_tile0) * a.S;
-    return first >= t0 && first + a.S <= t1;
+  __device__ __forceinline__ void next(const TileArgs& a, int k) {
+    ++u;
+    settle(a, k);
   }
 };
 
-__device__ __forceinline__ int segment_of(const TileArgs& a, int slab) {
+__device__ __forceinline__ int segment_of(const TileArgs& a, int tile) {
   int g = 0;
 #pragma unroll
   for (int i = 1; i < kMaxSegments; ++i)
-    if (i < a.n_seg && slab >= a.seg[i].tile0) g = i;
+    if (i < a.n_seg && tile >= a.seg[i].tile0) g = i;
   return g;
 }
 
@@ -423,7 +441,7 @@ __device__ __forceinline__ void gather(uint32_t (&r)[32], const uint32_t (&w)[F:
 }
 
 template <class F, int NB>
-__global__ void __launch_bounds__(kThreads, 4) tile_kernel(const __grid_constant__ TileMaps maps, const TileArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant__ TileMaps maps, const TileArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -437,327 +455,352 @@ __global__ void __launch_bounds__(kThreads, 4) tile_kernel(const __grid_constant
       return;
     }
   }
-  const int D = a.D;
-  const uint32_t idx_full = base + a.bar_off, idx_empty = idx_full + 8 * kMaxDepth, x_full = idx_empty + 8 * kMaxDepth,
-                 x_empty = x_full + 8 * kMaxDepth, a_full = x_empty + 8 * kMaxDepth, a_empty = a_full + 8 * kAStages,
-                 d_full = a_empty + 8 * kAStages, tmem_slot = d_full + 16, last_slot = tmem_slot + 4;
-  if (warp == 4 && lane == 0) {
-    for (int i = 0; i < D; ++i) {
-      mbar_init(idx_full + 8 * i, 1);
-      mbar_init(idx_empty + 8 * i, kDecodeWarps);
-      mbar_init(x_full + 8 * i, 1);
-      mbar_init(x_empty + 8 * i, 1);
+  constexpr bool kExact = F::TK == kRow && !F::I4;   // 8-bit row tables hold unscaled entries: sums are scaled per block
+  constexpr int RC = NB == 8 ? 8 : F::RC16;          // columns of sums handed over at a time
+  const int D = a.D, c = blockIdx.x;
+  const bool by_block = kExact && a.cb_int8;
+  const int block_units = a.Bc / F::UC;
+  const int quad = warp < kDecodeWarps ? warp >> 2 : warp & 3;
+  // barriers of a quad: indices and activations of a unit, decoded stages full and consumed, sums ready; then the CTA's
+  const uint32_t bars = base + a.bar_off, qb = bars + quad * 112;
+  const uint32_t idx_full = qb, x_full = qb + 32, a_full = qb + 64, a_empty = qb + 80, d_full = qb + 96;
+  const uint32_t red_full = bars + 448, red_empty = red_full + 8, tmem_slot = red_full + 16, n_last = tmem_slot + 4, last_tile = n_last + 4;
+  const uint32_t idx_at = base + a.idx_off + quad * D * F::IDX_BYTES, x_at = base + quad * D * a.x_bytes;
+  const bool service = warp >= kDecodeWarps && warp < kResultsWarp;
+
+  Units wi, wm;   // (service warps) the next unit whose indices are to be requested, to be multiplied
+  int islot = 0;
+  auto request_indices = [&]() {
+    if (elect_one()) {
+      const int g = segment_of(a, wi.f.tile);
+      mbar_arrive_expect_tx(idx_full + 8 * islot, F::IDX_BYTES);
+      tma_box_2d(idx_at + islot * F::IDX_BYTES, &maps.idx[g], wi.u * F::RB, (wi.f.tile - a.seg[g].tile0) * kTileRows, idx_full + 8 * islot);
     }
-    for (int i = 0; i < kAStages; ++i) {
-      mbar_init(a_full + 8 * i, kDecodeWarps);
-      mbar_init(a_empty + 8 * i, 1);
+    __syncwarp();
+    if (++islot == D) islot = 0;
+    wi.next(a, quad);
+  };
+  if (service) {
+    wi.init(a, c, quad);
+    wm = wi;
+    if (elect_one()) {
+      prefetch_tensormap(&maps.idx[0]);
+      for (int i = 0; i < D; ++i) {
+        mbar_init(idx_full + 8 * i, 1);
+        mbar_init(x_full + 8 * i, 1);
+      }
+      for (int i = 0; i < kAStages; ++i) {
+        mbar_init(a_full + 8 * i, 4);
+        mbar_init(a_empty + 8 * i, 1);
+        mbar_init(d_full + 8 * i, 1);
+      }
+      mbar_init_fence();
+      prefetch_tensormap(&maps.x);
     }
-    mbar_init(d_full, 1);
-    mbar_init(d_full + 8, 1);
-    mbar_init_fence();
-  }
-  if (warp == 5) {
+    __syncwarp();
+    for (int i = 0; i < D && wi.f.valid; ++i) request_indices();   // (weights do not depend on the previous kernel)
+  } else if (warp == kResultsWarp) {
+    if (lane == 0) {
+      mbar_init(red_full, kDecodeWarps);
+      mbar_init(red_empty, 1);
+      mbar_init_fence();
+      sts32(n_last, 0u);
+    }
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tmem_slot), "n"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // The next kernel's CTAs may come as soon as this one's leave: a CTA of this kernel fills an SM, so that they take no slot
+  // beside it, and their indices arrive while the last sums of this call are added.
+  if (tid == 0) pdl_launch_dependents();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(tmem_slot) : "memory");
-  const int c = blockIdx.x;
-  Walk wk;
-  wk.init(a, c, gridDim.x);
-  constexpr bool kExact = F::TK == kRow && !F::I4;   // 8-bit row tables hold unscaled entries: sums are scaled per block
-  const bool by_block = kExact && a.cb_int8;
-  const int block_units = by_block ? a.Bc / F::UC : 1;
+  int tries = kWaitTries;
 
-  if (warp == 4) {
-    // ---- producer ------------------------------------------------------------------------------------------
-    if (lane == 0) {
-      prefetch_tensormap(&maps.x);
-      for (int i = 0; i < a.n_seg; ++i) prefetch_tensormap(&maps.idx[i]);
-      // Index and activation boxes in two independent sequences, each as far ahead as its own stages allow: one
-      // thread polls both (in one sequence the activations of a unit were requested only when the unit before it had been
-      // read, and their latency showed in every unit).
-      Walk wi = wk;
-      int slot_i = 0, slot_x = 0, idle = 0;
-      uint32_t ph_i = 1, ph_x = 1;   // parity of the empty barriers: the first D polls succeed at once
-      bool started = false;
-      while (wk.k < wk.n && idle < kPolls) {
-        if (++idle > 1) __nanosleep(kPollSleep);   // (polls without a pause take issue slots from the decoding warps)
-        if (wi.k < wi.n && mbar_test(idx_empty + 8 * slot_i, ph_i)) {
-          fence_proxy_async();   // the warps' reads of the stage (released by their arrivals) before the copy engine's writes
-          const int g = segment_of(a, wi.slab);
-          mbar_arrive_expect_tx(idx_full + 8 * slot_i, F::IDX_BYTES);
-          tma_box_2d(base + a.idx_off + slot_i * F::IDX_BYTES, &maps.idx[g], wi.s * F::RB, (wi.slab - a.seg[g].tile0) * kTileRows,
-                     idx_full + 8 * slot_i);
-          if (++slot_i == D) { slot_i = 0; ph_i ^= 1u; }
-          wi.next(a);
-          idle = 0;
-        }
-        if (!started && wi.k < min(D, wi.n)) continue;   // weights first: they do not depend on the previous kernel
-        if (!started) {
-          pdl_wait();   // the activations belong to the previous kernel of the stream until here
-          started = true;
-        }
-        if (mbar_test(x_empty + 8 * slot_x, ph_x)) {
-          mbar_arrive_expect_tx(x_full + 8 * slot_x, a.x_bytes);
-          tma_box_3d(base + slot_x * a.x_bytes, &maps.x, 0, 0, wk.s * F::STAGES, x_full + 8 * slot_x);
-          if (++slot_x == D) { slot_x = 0; ph_x ^= 1u; }
-          wk.next(a);
-          idle = 0;
-        }
+  if (service) {
+    // ---- service: a quad's copies and products ---------------------------------------------------------------
+    Units wx = wm;
+    int xslot = 0;
+    auto request_x = [&]() {
+      if (elect_one()) {
+        mbar_arrive_expect_tx(x_full + 8 * xslot, a.x_bytes);
+        tma_box_3d(x_at + xslot * a.x_bytes, &maps.x, 0, 0, wx.u * F::STAGES, x_full + 8 * xslot);
       }
-      if (wk.k < wk.n) {   // gave up: let this CTA's own copies land before its shared memory goes away
-        atomicAdd(a.error_flag, 1);
-        __nanosleep(1000000);
-      }
-    }
-    __syncwarp();
-  } else if (warp == 5) {
-    // ---- products ------------------------------------------------------------------------------------------
-    int tries = kWaitTries;
-    int ab = 0, xs = 0, seg = 0;
-    uint32_t ph_a = 0, ph_x = 0;
-    uint32_t fresh = 1;   // the next product starts a sum
-    int block_left = by_block ? block_units - wk.s % block_units : 0;   // units left in the codebook block
-    for (; wk.k < wk.n; wk.next(a)) {
-      wait_phase(x_full + 8 * xs, ph_x, tries, a.error_flag);
+      __syncwarp();
+      if (++xslot == D) xslot = 0;
+      wx.next(a, quad);
+    };
+    pdl_wait();   // the activations belong to the previous kernel of the stream until here
+    for (int i = 0; i < D && wx.f.valid; ++i) request_x();
+    int slot = 0, seg = 0, seg_left = 0, st = 0;
+    uint32_t ph = 0, fresh = 1;
+    for (; wm.f.valid; ++st) {
+      if (seg_left == 0) seg_left = (by_block ? min(wm.end, (wm.u / block_units + 1) * block_units) : wm.end) - wm.u;
+      wait_phase(x_full + 8 * slot, ph, tries, a.error_flag);
+#pragma unroll
       for (int j = 0; j < F::STAGES; ++j) {
-        wait_phase(a_full + 8 * ab, ph_a, tries, a.error_flag);
+        // a quad fills its two decoded stages in turn: stage j's use number is st * STAGES / 2 + j / 2
+        wait_phase(a_full + 8 * (j & 1), F::STAGES == 2 ? st & 1 : (j >> 1) & 1, tries, a.error_flag);
         __syncwarp();
         tc_fence_after();
-        const uint64_t xd = b_descriptor(base + xs * a.x_bytes + j * a.x_row_bytes);   // (+ 2 q: 32-byte steps of K)
-        const uint32_t at = tmem + kAOff + ab * kStageTmem, dt = tmem + (seg & 1) * 16;
+        const uint64_t xd = b_descriptor(x_at + slot * a.x_bytes + j * a.x_row_bytes);   // (+ 2 q: 32-byte steps of K)
+        const uint32_t at = tmem + kAOff + (quad * 2 + (j & 1)) * 32, dt = tmem + quad * 32 + (seg & 1) * 16;
         if (elect_one()) {   // (also after a wait that ran out: the operands are in bounds whatever they hold)
           tc_mma(dt, at, xd, fresh ^ 1u);
 #pragma unroll
           for (int q = 1; q < 4; ++q) tc_mma(dt, at + 8 * q, xd + 2 * q, 1u);
-          tc_commit(a_empty + 8 * ab);
+          tc_commit(a_empty + 8 * (j & 1));
+          if (j == F::STAGES - 1 && seg_left == 1) tc_commit(d_full + 8 * (seg & 1));
         }
         __syncwarp();
         fresh = 0;
-        if (++ab == kAStages) { ab = 0; ph_a ^= 1u; }
+        if (j == 0) {
+          // the quad read all its indices of the unit before it handed over the first stage: the copy may be replaced
+          if (wi.f.valid) {
+            fence_proxy_async();   // the warps' reads (released by their arrivals) before the copy engine's writes
+            request_indices();
+          }
+        } else if (j == 1) {
+          // a stage decoded into the place of the last one of the unit before: that unit's products are complete
+          if (st > 0 && wx.f.valid) request_x();
+        }
       }
-      const bool frag_end = wk.slab_end(a);
-      const bool seg_end = frag_end || (by_block && block_left == 1);
-      if (elect_one()) {
-        tc_commit(x_empty + 8 * xs);
-        if (seg_end) tc_commit(d_full + 8 * (seg & 1));
-      }
-      __syncwarp();
-      if (seg_end) {
+      if (--seg_left == 0) {
         ++seg;
         fresh = 1;
       }
-      block_left = seg_end ? block_units : block_left - 1;   // (after a fragment's end the next one starts at column 0)
-      if (++xs == D) { xs = 0; ph_x ^= 1u; }
+      if (++slot == D) { slot = 0; ph ^= 1u; }
+      wm.next(a, quad);
     }
+    if (tries == 0) __nanosleep(1000000);   // gave up: let this CTA's own copies land before its shared memory goes away
+  } else if (warp == kResultsWarp) {
+    // ---- results: adds the quads' sums of a fragment, stores the outputs or this CTA's share of them --------------
+    pdl_wait();   // outputs and workspace belong to earlier kernels of the stream until here
+    Walk f;
+    f.init(a, c);
+    const unsigned T = a.tail_steps, Pt = a.tail_ctas;   // (products below 2^31: checked on the host)
+    const int first_tile = a.tail_tile0 + static_cast<int>(T * c / (Pt ? Pt : 1u)) / a.steps;
+    uint32_t ph = 0;
+    int listed = 0;
+    for (; f.valid; f.next(a)) {
+      const bool complete = f.complete(a);
+      const Segment& sg = a.seg[segment_of(a, f.tile)];
+      const int row = (f.tile - sg.tile0) * kTileRows + 4 * lane;
+      // this CTA's share of a left-over tile: slot 0 if its piece begins inside the tile, else slot 1
+      float* part = a.ws_part + (static_cast<long long>(c) * 2 + (f.tile == first_tile ? 0 : 1)) * (kTileRows * a.batch) + 4 * lane;
+      for (int n0 = 0; n0 < a.batch; n0 += RC) {
+        wait_phase(red_full, ph, tries, a.error_flag);
+        __syncwarp();
+        const int cols = min(RC, a.batch - n0);
+        for (int n = 0; n < cols; ++n) {
+          float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int k = 0; k < kQuads; ++k) {
+            const uint4 v = lds128(base + a.red_off + ((k * min(RC, a.batch) + n) * kTileRows + 4 * lane) * 4);
+            s.x += __uint_as_float(v.x); s.y += __uint_as_float(v.y); s.z += __uint_as_float(v.z); s.w += __uint_as_float(v.w);
+          }
+          if (!complete) {
+            *reinterpret_cast<float4*>(part + (n0 + n) * kTileRows) = s;
+          } else {
+            __half* y = sg.Y + static_cast<long long>(n0 + n) * sg.N + row;
+            const __half2 lo = __floats2half2_rn(s.x, s.y), hi = __floats2half2_rn(s.z, s.w);
+            if (sg.N % 4 == 0) {   // (rows 4 l .. 4 l + 3 then exist together, 8-byte aligned)
+              if (row < sg.N) *reinterpret_cast<uint2*>(y) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            } else {
+              if (row < sg.N) y[0] = __low2half(lo);
+              if (row + 1 < sg.N) y[1] = __high2half(lo);
+              if (row + 2 < sg.N) y[2] = __low2half(hi);
+              if (row + 3 < sg.N) y[3] = __high2half(hi);
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(red_empty);
+        ph ^= 1u;
+      }
+      if (!complete) {
+        __threadfence();   // this lane's sums are visible to the GPU before the ticket is drawn
+        __syncwarp();
+        if (lane == 0) {
+          const unsigned first_s = (f.tile - a.tail_tile0) * a.steps;
+          const int c_first = static_cast<int>(((first_s + 1) * Pt - 1) / T), c_last = static_cast<int>(((first_s + a.steps) * Pt - 1) / T);
+          const int ticket = atomicAdd(a.ws_ticket + f.tile, 1);
+          if (ticket == c_last - c_first) {   // every share of the tile is there: this CTA adds them when it has done its own work
+            a.ws_ticket[f.tile] = 0;          // nobody else touches the counter in this call
+            sts32(last_tile + 4 * listed, f.tile);
+            ++listed;
+          }
+        }
+      }
+    }
+    if (lane == 0) sts32(n_last, listed);
+    __threadfence();
   } else {
     // ---- decode ----------------------------------------------------------------------------------------------
     // One loop over units; what is not done in every unit stands in one place each (a codebook block, a running sum
-    // and a fragment are whole units).  With the sums read in three places the kernel had 110 to 195 KB of code and ran four
-    // times slower; with all of it checked in every stage a stage took 220 instructions a warp instead of 110.
-    int tries = kWaitTries;
+    // and a fragment are whole units): the loop has to stay small enough for the instruction cache.
+    const int qt = tid & 127;   // row of the tile
     Tables<F> tb;
-    const uint32_t my_table = tables + (F::TK == kCta ? 0 : warp * F::TABLE);
+    const uint32_t my_table = tables + (F::TK == kRow ? (warp >> 1) * F::TABLE + (warp & 1) * 128 : F::TK == kWarp ? warp * F::TABLE : quad * F::BUFS * F::TABLE);
     const uint32_t lane_off = F::D == 4 ? (lane & 15) * 8 : lane * 4;
     const uint32_t pat = ((my_table >> 12) & 0xFu) * 0x10101010u;
-    const uint32_t swz = F::RB == 32 ? ((tid >> 2) & 1) << 4 : F::RB == 64 ? ((tid >> 1) & 3) << 4 : F::RB == 128 ? (tid & 7) << 4 : 0;
-    const uint32_t tmem_a = tmem + (static_cast<uint32_t>(warp * 32) << 16) + kAOff;
+    const uint32_t swz = F::RB == 32 ? ((qt >> 2) & 1) << 4 : F::RB == 64 ? ((qt >> 1) & 3) << 4 : F::RB == 128 ? (qt & 7) << 4 : 0;
+    const uint32_t tmem_lane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    const uint32_t tmem_a = tmem_lane + kAOff + quad * 64, tmem_d = tmem_lane + quad * 32;
+    const uint32_t red_at = base + a.red_off + (quad * min(RC, a.batch) * kTileRows + qt) * 4;
     uint32_t tbl = my_table + lane_off;
     int half = 0;
-    int ab = 0, islot = 0;
-    uint32_t ph_a = 1, ph_i = 0;
+    uint32_t ph_i = 0, ph_red = 1;
 
-    // The walk by fragments (the CTA's units of one tile): first column of the current unit, end column.
-    int col = wk.s * F::UC, frag_end = 0, next_k = 0;
-    int block_left = 0, seg_left = 0;   // units left in the codebook block, the running sum
-    int bcol = 0;
-    // The sum that is complete but not yet read (`pend_*`): it is read a unit or two later, when the tensor core has caught up.
-    int st = 0, fin_at = -1, seg = 0;
-    int pend_slab = 0;
-    bool pend_last = false, pend_complete = false, done = wk.n == 0, waited = false;
+    Walk f;        // the fragment after the current one
+    f.init(a, c);
+    int tile = f.tile, u, end;   // the current fragment: next unit of the quad, end
+    f.range(a, quad, u, end);
+    f.next(a);
+    int bcol = u / block_units - 1, block_left = 0;   // codebook block column, units left in it
+    bool asked = u < end;                             // are the entries of the next block to be used on their way?
+    if (asked) {
+      const Segment& sg = a.seg[segment_of(a, tile)];
+      tb.open(a, sg, (tile - sg.tile0) * kTileRows, qt);
+      tb.request(a, bcol + 1);
+    }
+    // The running sum, and one that is complete but not yet read (`pend_*`): it is read a unit or two later, when the tensor
+    // core has caught up.
+    int st = 0, seg = 0, seg_left = 0, seg_units = 0, fin_at = -1;
+    bool open_sum = false, first_sum = true, more = true, pend_last = false, pend_zero = false;
     float pend_scale = 1.f, block_scale = 1.f;
-    float total[NB];
-#pragma unroll
-    for (int n = 0; n < NB; ++n) total[n] = 0.f;
     const __half* gs = nullptr;   // int4 codebooks: the scales of the thread's row
 
-    if (!done) {
-      const Segment& sg = a.seg[segment_of(a, wk.slab)];
-      tb.open(a, sg, (wk.slab - sg.tile0) * kTileRows, tid);
-      tb.request(a, col / a.Bc);
-    }
-    bool new_frag = true;
-
 #pragma unroll 1
-    while (!done || fin_at >= 0) {
+    for (;;) {
       if (st == fin_at) {
         // ---- read a finished sum ----
         fin_at = -1;
-        const int buf = (seg - 1) & 1;
-        wait_phase(d_full + 8 * buf, ((seg - 1) >> 1) & 1, tries, a.error_flag);
-        __syncwarp();
-        tc_fence_after();
-        {
-          float v[NB];
-          tc_load<NB>(tmem_a - kAOff + buf * 16, v);
+        float v[NB];
+#pragma unroll
+        for (int n = 0; n < NB; ++n) v[n] = 0.f;
+        if (!pend_zero) {
+          const int buf = (seg - 1) & 1;
+          wait_phase(d_full + 8 * buf, ((seg - 1) >> 1) & 1, tries, a.error_flag);
+          __syncwarp();
+          tc_fence_after();
+          tc_load<NB>(tmem_d + buf * 16, v);
           tc_fence_before();
-#pragma unroll
-          for (int n = 0; n < NB; ++n) total[n] = by_block ? fmaf(pend_scale, v[n], total[n]) : v[n];
         }
-        if (pend_last) {
-          if (!waited) {   // outputs and workspace belong to earlier kernels of the stream until here
-            pdl_wait();
-            waited = true;
-          }
-          const Segment& sg = a.seg[segment_of(a, pend_slab)];
-          const int row = (pend_slab - sg.tile0) * kTileRows + tid;
-          bool store = pend_complete;
-          if (!pend_complete) {
-            // this CTA's share of a left-over tile: slot 0 if its piece begins inside the tile, else slot 1
-            const int part_floats = kTileRows * a.batch;
-            const int slot = (wk.tail_tile0 + wk.t0 / a.S == pend_slab) ? 0 : 1;
-            float* part = a.ws_part + (static_cast<long long>(c) * 2 + slot) * part_floats + tid;
 #pragma unroll
-            for (int n = 0; n < NB; ++n)
-              if (n < a.batch) part[n * kTileRows] = total[n];
-            const unsigned T = a.tail_units, Pt = a.tail_ctas;   // (products below 2^31: checked on the host)
-            const unsigned first_u = (pend_slab - wk.tail_tile0) * a.S;
-            const int c_first = static_cast<int>(((first_u + 1) * Pt - 1) / T), c_last = static_cast<int>(((first_u + a.S) * Pt - 1) / T);
-            __threadfence();   // this thread's sums are visible to the GPU before the ticket is drawn
-            decode_barrier();
-            if (tid == 0) {
-              const int ticket = atomicAdd(a.ws_ticket + pend_slab, 1);
-              if (ticket == c_last - c_first) a.ws_ticket[pend_slab] = 0;   // nobody else touches the counter in this call
-              __threadfence();
-              sts32(last_slot, ticket == c_last - c_first);
-            }
-            decode_barrier();
-            uint32_t last;
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(last) : "r"(last_slot) : "memory");
-            if (last) {   // the last to arrive adds every CTA's share, in CTA order
-              __threadfence();
-              store = true;
+        for (int h = 0; h < NB / RC; ++h) {
+          if (h * RC >= a.batch) break;
+          if (first_sum) wait_phase(red_empty, ph_red, tries, a.error_flag);
 #pragma unroll
-              for (int n = 0; n < NB; ++n) total[n] = 0.f;
-#pragma unroll 4
-              for (int qc = c_first; qc <= c_last; ++qc) {
-                const int q_t0 = static_cast<int>(T * qc / Pt);
-                const int q_slot = (wk.tail_tile0 + q_t0 / a.S == pend_slab) ? 0 : 1;
-                const float* p = a.ws_part + (static_cast<long long>(qc) * 2 + q_slot) * part_floats + tid;
-#pragma unroll
-                for (int n = 0; n < NB; ++n)
-                  if (n < a.batch) total[n] += __ldcg(p + n * kTileRows);
+          for (int n = 0; n < RC; ++n)
+            if (h * RC + n < a.batch) {
+              const uint32_t at = red_at + n * kTileRows * 4;
+              float s = v[h * RC + n];
+              if (by_block) {
+                if (first_sum) s *= pend_scale;
+                else s = fmaf(pend_scale, s, lds32f(at));
               }
+              sts32f(at, s);
             }
+          if (pend_last) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(red_full);
+            ph_red ^= 1u;
           }
-          if (store && row < sg.N) {
-#pragma unroll
-            for (int n = 0; n < NB; ++n)
-              if (n < a.batch) sg.Y[static_cast<long long>(n) * sg.N + row] = __float2half_rn(total[n]);
-          }
-#pragma unroll
-          for (int n = 0; n < NB; ++n) total[n] = 0.f;
         }
-        if (done) break;
+        first_sum = pend_last;
+        if (!more) break;
       }
       if (seg_left == 0) {
         // ---- a sum ends (all but the first time), the next one begins ----
-        if (st > 0) {
-          ++seg;
-          fin_at = st;
-          pend_slab = wk.slab;
-          pend_complete = wk.complete(a);
+        if (open_sum) {
+          open_sum = false;
+          pend_zero = seg_units == 0;
           pend_scale = block_scale;
-          pend_last = col == frag_end;
+          pend_last = u == end;
+          if (!pend_zero) ++seg;
+          fin_at = st;
           if (pend_last) {   // to the next fragment
-            wk.k = next_k;
-            if (wk.k == wk.n) {
-              done = true;
-              // The next kernel may start once all is decoded: earlier, its CTAs take the slots that this grid leaves free on
-              // some SMs and stay where they land (8B-class block 66.8 against 66.0 us, 70B at batch 16 166.7 against 161.9).
-              // Every CTA has its tensor memory by then, so one that waits for some never waits for itself.
-              pdl_launch_dependents();
+            if (!f.valid) {
+              more = false;
               continue;
             }
-            wk.slab = wk.k == wk.n_tail ? wk.whole0 : wk.slab + 1;
-            wk.s = 0;
-            col = 0;
-            new_frag = true;
+            tile = f.tile;
+            f.range(a, quad, u, end);
+            f.next(a);
+            bcol = u / block_units - 1;
+            block_left = 0;
           }
         }
-        if (new_frag) {
-          new_frag = false;
-          const int units = wk.fragment_units(a);
-          next_k = wk.k + units;
-          frag_end = col + units * F::UC;
-          bcol = col / a.Bc - 1;
-          block_left = 0;
-          if constexpr (F::I4) {
-            const Segment& sg = a.seg[segment_of(a, wk.slab)];
-            gs = sg.scale + static_cast<long long>(min((wk.slab - sg.tile0) * kTileRows + tid, sg.N - 1)) * (a.K / 128);
-          }
-        }
-        seg_left = ((by_block ? min(frag_end, (bcol + 2) * a.Bc) : frag_end) - col) / F::UC;
+        open_sum = true;
+        seg_units = seg_left = (by_block ? min(end, (bcol + 2) * block_units) : end) - u;
+        if (seg_left == 0) continue;   // nothing of the fragment is this quad's
         if (fin_at >= 0) fin_at = st + min(F::STAGES == 2 ? 2 : 1, seg_left);
+        if constexpr (F::I4) {
+          const Segment& sg = a.seg[segment_of(a, tile)];
+          gs = sg.scale + static_cast<long long>(min((tile - sg.tile0) * kTileRows + qt, sg.N - 1)) * (a.K / 128);
+        }
       }
       uint32_t scales[F::STAGES / 2];   // int4 codebooks: of the unit's groups of 128 columns
       if constexpr (F::I4) {
 #pragma unroll
         for (int i = 0; i < F::STAGES / 2; ++i)
-          scales[i] = __ldg(reinterpret_cast<const unsigned short*>(gs) + col / 128 + i) * 0x10001u;
+          scales[i] = __ldg(reinterpret_cast<const unsigned short*>(gs) + u * (F::UC / 128) + i) * 0x10001u;
       }
       wait_phase(idx_full + 8 * islot, ph_i, tries, a.error_flag);
       uint32_t w[F::RB / 4];
       {
-        const uint32_t row_at = base + a.idx_off + islot * F::IDX_BYTES + tid * F::RB;
+        const uint32_t row_at = idx_at + islot * F::IDX_BYTES + qt * F::RB;
 #pragma unroll
         for (int i = 0; i < F::RB / 16; ++i) {   // 128-bit reads, conflict-free at every row pitch in use
           const uint4 v = lds128(row_at + ((16u * i) ^ swz));
           w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
         }
-        __syncwarp();   // the unit's bytes are in registers: its stage may be refilled
-        if (lane == 0) mbar_arrive(idx_empty + 8 * islot);
         if (++islot == D) { islot = 0; ph_i ^= 1u; }
       }
       if (block_left == 0) {   // another codebook block: its entries were requested a block ago
         ++bcol;
-        block_left = ((bcol + 1) * a.Bc - col) / F::UC;
+        block_left = (bcol + 1) * block_units - u;
+        if (!asked) {
+          const Segment& sg = a.seg[segment_of(a, tile)];
+          tb.open(a, sg, (tile - sg.tile0) * kTileRows, qt);
+          tb.request(a, bcol);
+        }
         if constexpr (F::TK == kRow) {
-          tb.write(a, my_table + half * 128, tid);   // the other half: nobody reads it any more
-          tbl = my_table + half * 128 + lane_off;
-          half ^= 1;
+          tb.write(a, my_table, qt);   // (a lane reads what it wrote itself)
           if (by_block) block_scale = tb.scale();
         } else if constexpr (F::TK == kWarp) {
           __syncwarp();   // every lane has left the old table
-          tb.write(a, my_table, tid);
+          tb.write(a, my_table, qt);
           __syncwarp();
         } else if constexpr (F::BUFS == 2) {
-          tb.write(a, my_table + half * F::TABLE, tid);   // last used two blocks ago
-          decode_barrier();
+          tb.write(a, my_table + half * F::TABLE, qt);   // last used two blocks ago
+          quad_barrier(quad);
           tbl = my_table + half * F::TABLE + lane_off;
           half ^= 1;
         } else {
-          decode_barrier();
-          tb.write(a, my_table, tid);
-          decode_barrier();
+          quad_barrier(quad);
+          tb.write(a, my_table, qt);
+          quad_barrier(quad);
         }
         fence_value(tbl);   // look-ups of the new block stay behind the writes
         // request the next block: of this fragment, or the first of the next one
-        int nb = bcol + 1;
-        if (nb * a.Bc >= frag_end) {
-          nb = -1;
-          if (next_k < wk.n) {
-            const int nslab = next_k == wk.n_tail ? wk.whole0 : wk.slab + 1;
-            const Segment& sg = a.seg[segment_of(a, nslab)];
-            tb.open(a, sg, (nslab - sg.tile0) * kTileRows, tid);
-            nb = 0;
+        asked = false;
+        if ((bcol + 1) * block_units < end) {
+          tb.request(a, bcol + 1);
+          asked = true;
+        } else if (f.valid) {
+          int nu, nend;
+          f.range(a, quad, nu, nend);
+          if (nu < nend) {
+            const Segment& sg = a.seg[segment_of(a, f.tile)];
+            tb.open(a, sg, (f.tile - sg.tile0) * kTileRows, qt);
+            tb.request(a, nu / block_units);
+            asked = true;
           }
         }
-        if (nb >= 0) tb.request(a, nb);
       }
       --block_left;
       auto stage = [&](auto jc) {
@@ -768,19 +811,19 @@ __global__ void __launch_bounds__(kThreads, 4) tile_kernel(const __grid_constant
 #pragma unroll
           for (int i = 0; i < 32; ++i) r[i] = mul_f16x2(r[i], scales[J / 2]);
         }
-        wait_phase(a_empty + 8 * ab, ph_a, tries, a.error_flag);
+        // (the place's use number is st * STAGES / 2 + J / 2)
+        wait_phase(a_empty + 8 * (J & 1), F::STAGES == 2 ? (st & 1) ^ 1 : ((J >> 1) & 1) ^ 1, tries, a.error_flag);
         __syncwarp();
         tc_fence_after();
-        tc_store32(tmem_a + ab * kStageTmem, r);
+        tc_store32(tmem_a + (J & 1) * 32, r);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(a_full + 8 * ab);
-        if (++ab == kAStages) { ab = 0; ph_a ^= 1u; }
+        if (lane == 0) mbar_arrive(a_full + 8 * (J & 1));
       };
       [&]<int... J>(std::integer_sequence<int, J...>) {
         (stage(std::integral_constant<int, J>{}), ...);
       }(std::make_integer_sequence<int, F::STAGES>{});
-      col += F::UC;
+      ++u;
       --seg_left;
       ++st;
     }
@@ -788,7 +831,29 @@ __global__ void __launch_bounds__(kThreads, 4) tile_kernel(const __grid_constant
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 5) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols));
+  if (warp == kResultsWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols));
+  // ---- the shared tiles whose last share came from this CTA: every share is added, in CTA order ----
+  uint32_t listed;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(listed) : "r"(n_last) : "memory");
+  for (uint32_t i = 0; i < listed; ++i) {
+    uint32_t slab;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(slab) : "r"(last_tile + 4 * i) : "memory");
+    const int tile = static_cast<int>(slab);
+    const unsigned T = a.tail_steps, Pt = a.tail_ctas;
+    const unsigned first_s = (tile - a.tail_tile0) * a.steps;
+    const int c_first = static_cast<int>(((first_s + 1) * Pt - 1) / T), c_last = static_cast<int>(((first_s + a.steps) * Pt - 1) / T);
+    const Segment& sg = a.seg[segment_of(a, tile)];
+    const int r = tid & 127, row = (tile - sg.tile0) * kTileRows + r;
+    for (int n = tid >> 7; n < a.batch && tid < kThreads / 128 * 128; n += kThreads / 128) {
+      float s = 0.f;
+#pragma unroll 4
+      for (int qc = c_first; qc <= c_last; ++qc) {
+        const int q_slot = a.tail_tile0 + static_cast<int>(T * qc / Pt) / a.steps == tile ? 0 : 1;
+        s += __ldcg(a.ws_part + ((static_cast<long long>(qc) * 2 + q_slot) * a.batch + n) * kTileRows + r);
+      }
+      if (row < sg.N) sg.Y[static_cast<long long>(n) * sg.N + row] = __float2half_rn(s);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -808,7 +873,7 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 template <class F, int NB>
 vq_status launch(const StreamCall& call, cudaStream_t s) {
   auto kern = tile_kernel<F, NB>;
-  constexpr size_t kSmemCap = 112 * 1024;
+  constexpr size_t kSmemCap = 227 * 1024;
   static int attr_set[kMaxDevices] = {};
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return VQ_ERR_CUDA;
@@ -828,6 +893,7 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   a.Bc = g.Bc;
   a.cb_int8 = g.cb_int8;
   a.S = g.K / F::UC;   // (block columns, and so K, are whole units: tile_covers)
+  a.steps = (a.S + kQuads - 1) / kQuads;
   int tiles = 0;
   long long rows_total = 0;
   for (int i = 0; i < call.n_seg; ++i) {
@@ -841,45 +907,38 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   }
   if (static_cast<long long>(tiles) * a.S > 0x3fffffff) return VQ_ERR_UNSUPPORTED;
 
-  // ---- shared memory: x stages, index stages, barriers, then the tables on their boundary ----
+  // ---- shared memory: activations, indices, sums, barriers, then the tables on their boundary ----
   const int x_rows = call.batch <= 8 ? 8 : 16;
+  constexpr int RC = NB == 8 ? 8 : F::RC16;
   a.x_row_bytes = x_rows * 128;
   a.x_bytes = F::STAGES * a.x_row_bytes;
   auto plan = [&](int D) {
     a.D = D;
-    a.idx_off = D * a.x_bytes;
-    a.bar_off = a.idx_off + D * F::IDX_BYTES;
-    a.front_bytes = a.bar_off + 512;
+    a.idx_off = kQuads * D * a.x_bytes;
+    a.red_off = a.idx_off + kQuads * D * F::IDX_BYTES;
+    a.bar_off = a.red_off + kQuads * (call.batch < RC ? call.batch : RC) * kTileRows * 4;
+    a.front_bytes = a.bar_off + kBarBytes;
     // (dynamic shared memory starts 1024 bytes into the window)
     return round_up(1024 + a.front_bytes, F::ALIGN) - 1024 + F::TABLES;
   };
-  int per_sm = env_int("VQ_TCPS", 4);
-  int D = 2;
-  for (; per_sm >= 2; --per_sm) {
-    const size_t budget = (228 * 1024) / per_sm - 1024;
-    for (D = kMaxDepth; D >= 2; --D)
-      if (plan(D) <= budget) break;
-    if (D >= 2) break;
-  }
-  if (per_sm < 2) return VQ_ERR_UNSUPPORTED;
-  D = env_int("VQ_TD", D);
-  const size_t smem_bytes = plan(D);
+  int D = env_int("VQ_TD", kMaxDepth);
+  while (D > 2 && plan(D) > kSmemCap) --D;
+  size_t smem_bytes = plan(D);
   if (smem_bytes > kSmemCap || D < 2 || D > kMaxDepth) return VQ_ERR_UNSUPPORTED;
+  if (smem_bytes < 120 * 1024) smem_bytes = 120 * 1024;   // one CTA per SM: the next kernel's go where one has left
 
-  // ---- persistent CTAs: whole tiles first, the units of the left-over tiles shared evenly ----
-  const long long units = static_cast<long long>(tiles) * a.S;
-  long long P = static_cast<long long>(sms) * per_sm;
-  // A tile is shared by about nine CTAs at most: its last one adds their sums in turn, a chain of reads of the
-  // workspace (4096 x 14336 at batch 16: 41 us with 18 CTAs per tile, 28 us with 9).  Two CTAs per SM at least.
-  if (P > 9LL * tiles) P = 9LL * tiles > 2LL * sms ? 9LL * tiles : 2LL * sms;
-  if (P > units) P = units;
+  // ---- persistent CTAs: whole tiles first, the steps of the left-over tiles shared evenly ----
+  const long long steps = static_cast<long long>(tiles) * a.steps;
+  long long P = sms < kMaxStreamCtas ? sms : kMaxStreamCtas;
+  if (P > steps) P = steps;
 #ifdef VQ_TUNING
   if (env_int("VQ_TP", 0) && P > env_int("VQ_TP", 0)) P = env_int("VQ_TP", 0);
 #endif
   a.q = static_cast<int>(tiles / P);
   const int left = static_cast<int>(tiles - a.q * P);
-  const long long tail = static_cast<long long>(left) * a.S;
-  a.tail_units = static_cast<int>(tail);
+  const long long tail = static_cast<long long>(left) * a.steps;
+  a.tail_tile0 = static_cast<int>(a.q * P);
+  a.tail_steps = static_cast<int>(tail);
   a.tail_ctas = static_cast<int>(tail < P ? tail : P);
   if (tail * (a.tail_ctas + 1) >= (1LL << 31)) return VQ_ERR_UNSUPPORTED;   // 32-bit arithmetic in the kernel
   // counters at the start, partial sums at the end of the workspace: a call with fewer rows then never writes
@@ -919,7 +978,7 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = env_int("VQ_PDL", 1) ? 1 : 0;
 #ifdef VQ_TUNING
-  if (env_int("VQ_VERBOSE", 0)) fprintf(stderr, "tile launch: grid %d per_sm %d depth %d smem %zu tiles %d S %d q %d tail %d/%d\n", (int)P, per_sm, D, smem_bytes, tiles, a.S, a.q, a.tail_units, a.tail_ctas);
+  if (env_int("VQ_VERBOSE", 0)) fprintf(stderr, "tile launch: grid %d depth %d smem %zu tiles %d S %d steps %d q %d tail %d/%d\n", (int)P, D, smem_bytes, tiles, a.S, a.steps, a.q, a.tail_steps, a.tail_ctas);
 #endif
   if (cudaLaunchKernelEx(&cfg, kern, maps, a) != cudaSuccess) return VQ_ERR_CUDA;
   return check_launch();
@@ -955,6 +1014,9 @@ bool tile_covers(const Geometry& g) {
 // more, and a launch per layer: 4160 x 3328 in three layers 21/12, 3328 x 9088 22/16 at batch 5; but 13312 x 1920 b2 11.0/14.0.
 bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
   if (!tile_covers(g)) return false;
+#ifdef VQ_TUNING
+  if (env_int("VQ_TILE", -1) >= 0) return env_int("VQ_TILE", 0) != 0;
+#endif
   long long rows = 0;
   bool whole = g.K % 256 == 0;
   for (int i = 0; i < n_seg; ++i) {
@@ -987,7 +1049,7 @@ bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
 vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {
   const Geometry& g = call.g;
   if (!tile_covers(g) || call.n_seg < 1 || call.n_seg > kMaxSegments) return VQ_ERR_UNSUPPORTED;
-  if (g.d == 2 && g.b == 4) return call.batch <= 8 ? VQ_ERR_UNSUPPORTED : launch<Fmt<2, 4, kRow, 1, false>, 16>(call, s);
+  if (g.d == 2 && g.b == 4) return launch_nb<Fmt<2, 4, kRow, 1, false>>(call, s);
   if (g.d == 4) return launch_nb<Fmt<4, 8, kCta, 128, false>>(call, s);
   if (g.Br % kTileRows == 0) {
     if (g.b == 6) return g.cb_int4 ? launch_nb<Fmt<2, 6, kCta, 128, true>>(call, s) : launch_nb<Fmt<2, 6, kCta, 128, false>>(call, s);
