@@ -83,11 +83,14 @@ struct TileArgs {
   int* error_flag;
   int K, batch;
   int S, steps;       // units and steps (of a unit per quad) of a tile
+  unsigned steps_inv, share_inv, share1_inv, block_inv;   // 2^32 / divisor, rounded up, for divide()
   int q;              // whole tiles per CTA
-  int tail_tile0, tail_steps, tail_ctas;   // the tiles left over and the CTAs that share their steps
+  int tail_tile0;     // the tiles left over: their steps are shared by the CTAs,
+  int share, longer;  // share + 1 each for the first `longer` CTAs, share for the others
   int blocks_per_row, Br, Bc, cb_int8;
   int D;              // unit stages of a quad
   int x_bytes, x_row_bytes;    // activations of a unit; bytes of one 64-column group of them
+  int red_cols;       // columns of sums handed over at a time, a multiple of 4
   int idx_off, red_off, bar_off, front_bytes;   // dynamic shared memory: activations, indices, sums, barriers, | tables
 };
 
@@ -128,17 +131,16 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {   // t
                : "=r"(done) : "r"(bar), "r"(parity) : "memory");
   return done != 0;
 }
-// Bounded wait for phase `parity`; `tries` is the role's budget: 0 once a wait has run out, so that later ones return at once.
-__device__ __forceinline__ void wait_phase(uint32_t bar, uint32_t parity, int& tries, int* error_flag) {
-  if (mbar_try(bar, parity)) return;
+// Bounded wait for phase `parity`; `tries` is the role's budget: 0 once a wait has run out, so that later ones return at once
+// (the role reports it at its end: one place keeps the code small).
+__device__ __forceinline__ void wait_phase(uint32_t bar, uint32_t parity, int& tries) {
+  int left = tries;
 #pragma unroll 1
-  for (int i = 0; !mbar_try(bar, parity);) {
-    if (++i >= tries) {
-      if (tries && (threadIdx.x & 31) == 0) atomicAdd(error_flag, 1);
+  while (!mbar_try(bar, parity))
+    if (--left <= 0) {
       tries = 0;
       break;
     }
-  }
 }
 __device__ __forceinline__ void quad_barrier(int quad) { asm volatile("bar.sync %0, 128;" ::"r"(1 + quad) : "memory"); }
 __device__ __forceinline__ void tma_box_3d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, uint32_t bar) {
@@ -178,22 +180,12 @@ __device__ __forceinline__ void tc_store32(uint32_t addr, const uint32_t (&r)[32
       : "memory");
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
-template <int NB>   // NB accumulator columns of the thread's row
-__device__ __forceinline__ void tc_load(uint32_t addr, float (&v)[NB]) {
-  uint32_t r[NB];
-  if constexpr (NB == 8) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(addr) : "memory");
-  } else {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-                   "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(addr) : "memory");
-  }
+__device__ __forceinline__ void tc_load4(uint32_t addr, float (&v)[4]) {   // four accumulator columns of the thread's row
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < NB; ++i) {
+  for (int i = 0; i < 4; ++i) {
     asm volatile("" : "+r"(r[i]));   // used behind the wait only
     v[i] = __uint_as_float(r[i]);
   }
@@ -226,22 +218,27 @@ __device__ __forceinline__ uint32_t nibble_pair(uint32_t byte) {   // two signed
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
+// x / d for x * d < 2^32 and inv = ceil(2^32 / d)  (d = 1: inv = 0)
+__device__ __forceinline__ int divide(int x, unsigned inv) { return inv ? static_cast<int>(__umulhi(static_cast<unsigned>(x), inv)) : x; }
+// first step of CTA c's piece of the left-over tiles, and the CTA whose piece holds step x
+__device__ __forceinline__ int first_step(const TileArgs& a, int c) { return c * a.share + min(c, a.longer); }
+__device__ __forceinline__ int step_owner(const TileArgs& a, int x) {
+  const int n = a.longer * (a.share + 1);
+  return x < n ? divide(x, a.share1_inv) : a.longer + divide(x - n, a.share_inv);
+}
+
 // A CTA's walk over its fragments (steps [s0, s1) of one tile): its piece of the left-over tiles first, then its whole tiles.
 struct Walk {
   int tile, s0, s1, left, whole, whole_end;
   bool valid;
 
   __device__ __forceinline__ void init(const TileArgs& a, int c) {
-    int t0 = 0, t1 = 0;
-    if (c < a.tail_ctas) {   // (the host keeps tail_steps * tail_ctas below 2^31)
-      t0 = static_cast<int>(static_cast<unsigned>(a.tail_steps) * static_cast<unsigned>(c) / static_cast<unsigned>(a.tail_ctas));
-      t1 = static_cast<int>(static_cast<unsigned>(a.tail_steps) * static_cast<unsigned>(c + 1) / static_cast<unsigned>(a.tail_ctas));
-    }
+    const int t0 = first_step(a, c), ahead = divide(t0, a.steps_inv);
     whole = c * a.q;
     whole_end = whole + a.q;
-    tile = a.tail_tile0 + t0 / a.steps - 1;
-    left = t1 - t0;
-    next(a, t0 % a.steps);
+    tile = a.tail_tile0 + ahead - 1;
+    left = first_step(a, c + 1) - t0;
+    next(a, t0 - ahead * a.steps);
   }
   __device__ __forceinline__ void next(const TileArgs& a, int first = 0) {
     valid = true;
@@ -440,7 +437,7 @@ __device__ __forceinline__ void gather(uint32_t (&r)[32], const uint32_t (&w)[F:
   }
 }
 
-template <class F, int NB>
+template <class F>
 __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant__ TileMaps maps, const TileArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -456,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     }
   }
   constexpr bool kExact = F::TK == kRow && !F::I4;   // 8-bit row tables hold unscaled entries: sums are scaled per block
-  constexpr int RC = NB == 8 ? 8 : F::RC16;          // columns of sums handed over at a time
+  const int red_cols = a.red_cols;
   const int D = a.D, c = blockIdx.x;
   const bool by_block = kExact && a.cb_int8;
   const int block_units = a.Bc / F::UC;
@@ -468,8 +465,10 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   const uint32_t idx_at = base + a.idx_off + quad * D * F::IDX_BYTES, x_at = base + quad * D * a.x_bytes;
   const bool service = warp >= kDecodeWarps && warp < kResultsWarp;
 
-  Units wi, wm;   // (service warps) the next unit whose indices are to be requested, to be multiplied
-  int islot = 0;
+  int tries = kWaitTries;
+  // (service warps) the next unit whose indices are to be requested; columns of the units requested first
+  Units wi;
+  int islot = 0, xu[kMaxDepth] = {};
   auto request_indices = [&]() {
     if (elect_one()) {
       const int g = segment_of(a, wi.f.tile);
@@ -478,13 +477,9 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     }
     __syncwarp();
     if (++islot == D) islot = 0;
-    wi.next(a, quad);
   };
   if (service) {
-    wi.init(a, c, quad);
-    wm = wi;
     if (elect_one()) {
-      prefetch_tensormap(&maps.idx[0]);
       for (int i = 0; i < D; ++i) {
         mbar_init(idx_full + 8 * i, 1);
         mbar_init(x_full + 8 * i, 1);
@@ -495,10 +490,16 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         mbar_init(d_full + 8 * i, 1);
       }
       mbar_init_fence();
-      prefetch_tensormap(&maps.x);
     }
     __syncwarp();
-    for (int i = 0; i < D && wi.f.valid; ++i) request_indices();   // (weights do not depend on the previous kernel)
+    wi.init(a, c, quad);
+#pragma unroll
+    for (int i = 0; i < kMaxDepth; ++i)
+      if (i < D && wi.f.valid) {   // (weights do not depend on the previous kernel)
+        request_indices();
+        xu[i] = wi.u + 1;
+        wi.next(a, quad);
+      }
   } else if (warp == kResultsWarp) {
     if (lane == 0) {
       mbar_init(red_full, kDecodeWarps);
@@ -517,32 +518,38 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   if (tid == 0) pdl_launch_dependents();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(tmem_slot) : "memory");
-  int tries = kWaitTries;
 
   if (service) {
     // ---- service: a quad's copies and products ---------------------------------------------------------------
-    Units wx = wm;
     int xslot = 0;
-    auto request_x = [&]() {
+    auto request_x = [&](int u) {
       if (elect_one()) {
         mbar_arrive_expect_tx(x_full + 8 * xslot, a.x_bytes);
-        tma_box_3d(x_at + xslot * a.x_bytes, &maps.x, 0, 0, wx.u * F::STAGES, x_full + 8 * xslot);
+        tma_box_3d(x_at + xslot * a.x_bytes, &maps.x, 0, 0, u * F::STAGES, x_full + 8 * xslot);
       }
       __syncwarp();
       if (++xslot == D) xslot = 0;
-      wx.next(a, quad);
     };
     pdl_wait();   // the activations belong to the previous kernel of the stream until here
-    for (int i = 0; i < D && wx.f.valid; ++i) request_x();
+#pragma unroll
+    for (int i = 0; i < kMaxDepth; ++i)
+      if (xu[i]) request_x(xu[i] - 1);
+    Walk f;
+    f.init(a, c);
+    int u = 0, end = 0, x_next = -1;   // the unit to be multiplied; column of the unit whose activations are to be requested
     int slot = 0, seg = 0, seg_left = 0, st = 0;
     uint32_t ph = 0, fresh = 1;
-    for (; wm.f.valid; ++st) {
-      if (seg_left == 0) seg_left = (by_block ? min(wm.end, (wm.u / block_units + 1) * block_units) : wm.end) - wm.u;
-      wait_phase(x_full + 8 * slot, ph, tries, a.error_flag);
+    for (;; ++st) {
+      if (u == end) {
+        for (; f.valid && u == end; f.next(a)) f.range(a, quad, u, end);
+        if (u == end) break;
+      }
+      if (seg_left == 0) seg_left = (by_block ? min(end, (divide(u, a.block_inv) + 1) * block_units) : end) - u;
+      wait_phase(x_full + 8 * slot, ph, tries);
 #pragma unroll
       for (int j = 0; j < F::STAGES; ++j) {
         // a quad fills its two decoded stages in turn: stage j's use number is st * STAGES / 2 + j / 2
-        wait_phase(a_full + 8 * (j & 1), F::STAGES == 2 ? st & 1 : (j >> 1) & 1, tries, a.error_flag);
+        wait_phase(a_full + 8 * (j & 1), F::STAGES == 2 ? st & 1 : (j >> 1) & 1, tries);
         __syncwarp();
         tc_fence_after();
         const uint64_t xd = b_descriptor(x_at + slot * a.x_bytes + j * a.x_row_bytes);   // (+ 2 q: 32-byte steps of K)
@@ -564,7 +571,12 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           }
         } else if (j == 1) {
           // a stage decoded into the place of the last one of the unit before: that unit's products are complete
-          if (st > 0 && wx.f.valid) request_x();
+          if (x_next >= 0) request_x(x_next);
+          x_next = -1;
+          if (wi.f.valid) {
+            x_next = wi.u;
+            wi.next(a, quad);
+          }
         }
       }
       if (--seg_left == 0) {
@@ -572,7 +584,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         fresh = 1;
       }
       if (++slot == D) { slot = 0; ph ^= 1u; }
-      wm.next(a, quad);
+      ++u;
     }
     if (tries == 0) __nanosleep(1000000);   // gave up: let this CTA's own copies land before its shared memory goes away
   } else if (warp == kResultsWarp) {
@@ -580,8 +592,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     pdl_wait();   // outputs and workspace belong to earlier kernels of the stream until here
     Walk f;
     f.init(a, c);
-    const unsigned T = a.tail_steps, Pt = a.tail_ctas;   // (products below 2^31: checked on the host)
-    const int first_tile = a.tail_tile0 + static_cast<int>(T * c / (Pt ? Pt : 1u)) / a.steps;
+    const int first_tile = f.tile;   // (of the CTA's piece, if it has one)
     uint32_t ph = 0;
     int listed = 0;
     for (; f.valid; f.next(a)) {
@@ -590,15 +601,17 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       const int row = (f.tile - sg.tile0) * kTileRows + 4 * lane;
       // this CTA's share of a left-over tile: slot 0 if its piece begins inside the tile, else slot 1
       float* part = a.ws_part + (static_cast<long long>(c) * 2 + (f.tile == first_tile ? 0 : 1)) * (kTileRows * a.batch) + 4 * lane;
-      for (int n0 = 0; n0 < a.batch; n0 += RC) {
-        wait_phase(red_full, ph, tries, a.error_flag);
+      const int first_s = (f.tile - a.tail_tile0) * a.steps;
+      const int shares = complete ? 1 : step_owner(a, first_s + a.steps - 1) - step_owner(a, first_s) + 1;
+      for (int n0 = 0; n0 < a.batch; n0 += red_cols) {
+        wait_phase(red_full, ph, tries);
         __syncwarp();
-        const int cols = min(RC, a.batch - n0);
+        const int cols = min(red_cols, a.batch - n0);
         for (int n = 0; n < cols; ++n) {
           float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int k = 0; k < kQuads; ++k) {
-            const uint4 v = lds128(base + a.red_off + ((k * min(RC, a.batch) + n) * kTileRows + 4 * lane) * 4);
+            const uint4 v = lds128(base + a.red_off + ((k * red_cols + n) * kTileRows + 4 * lane) * 4);
             s.x += __uint_as_float(v.x); s.y += __uint_as_float(v.y); s.z += __uint_as_float(v.z); s.w += __uint_as_float(v.w);
           }
           if (!complete) {
@@ -624,10 +637,8 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         __threadfence();   // this lane's sums are visible to the GPU before the ticket is drawn
         __syncwarp();
         if (lane == 0) {
-          const unsigned first_s = (f.tile - a.tail_tile0) * a.steps;
-          const int c_first = static_cast<int>(((first_s + 1) * Pt - 1) / T), c_last = static_cast<int>(((first_s + a.steps) * Pt - 1) / T);
           const int ticket = atomicAdd(a.ws_ticket + f.tile, 1);
-          if (ticket == c_last - c_first) {   // every share of the tile is there: this CTA adds them when it has done its own work
+          if (ticket == shares - 1) {   // every share of the tile is there: this CTA adds them when it has done its own work
             a.ws_ticket[f.tile] = 0;          // nobody else touches the counter in this call
             sts32(last_tile + 4 * listed, f.tile);
             ++listed;
@@ -635,8 +646,10 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         }
       }
     }
-    if (lane == 0) sts32(n_last, listed);
-    __threadfence();
+    if (lane == 0 && listed) {
+      sts32(n_last, listed);
+      __threadfence();   // the tickets before the shares are read
+    }
   } else {
     // ---- decode ----------------------------------------------------------------------------------------------
     // One loop over units; what is not done in every unit stands in one place each (a codebook block, a running sum
@@ -649,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     const uint32_t swz = F::RB == 32 ? ((qt >> 2) & 1) << 4 : F::RB == 64 ? ((qt >> 1) & 3) << 4 : F::RB == 128 ? (qt & 7) << 4 : 0;
     const uint32_t tmem_lane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     const uint32_t tmem_a = tmem_lane + kAOff + quad * 64, tmem_d = tmem_lane + quad * 32;
-    const uint32_t red_at = base + a.red_off + (quad * min(RC, a.batch) * kTileRows + qt) * 4;
+    const uint32_t red_at = base + a.red_off + (quad * red_cols * kTileRows + qt) * 4;
     uint32_t tbl = my_table + lane_off;
     int half = 0;
     uint32_t ph_i = 0, ph_red = 1;
@@ -659,7 +672,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     int tile = f.tile, u, end;   // the current fragment: next unit of the quad, end
     f.range(a, quad, u, end);
     f.next(a);
-    int bcol = u / block_units - 1, block_left = 0;   // codebook block column, units left in it
+    int bcol = divide(u, a.block_inv) - 1, block_left = 0;   // codebook block column, units left in it
     bool asked = u < end;                             // are the entries of the next block to be used on their way?
     if (asked) {
       const Segment& sg = a.seg[segment_of(a, tile)];
@@ -678,38 +691,39 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       if (st == fin_at) {
         // ---- read a finished sum ----
         fin_at = -1;
-        float v[NB];
-#pragma unroll
-        for (int n = 0; n < NB; ++n) v[n] = 0.f;
+        const int buf = (seg - 1) & 1;
         if (!pend_zero) {
-          const int buf = (seg - 1) & 1;
-          wait_phase(d_full + 8 * buf, ((seg - 1) >> 1) & 1, tries, a.error_flag);
+          wait_phase(d_full + 8 * buf, ((seg - 1) >> 1) & 1, tries);
           __syncwarp();
           tc_fence_after();
-          tc_load<NB>(tmem_d + buf * 16, v);
-          tc_fence_before();
         }
+        // (columns from the batch on are not used by anyone)
+#pragma unroll 1
+        for (int n0 = 0; n0 < a.batch; n0 += red_cols) {
+          if (first_sum) wait_phase(red_empty, ph_red, tries);
+          __syncwarp();
+#pragma unroll 1
+          for (int n = 0; n < red_cols; n += 4) {
+            float v[4];
+            tc_load4(tmem_d + buf * 16 + n0 + n, v);
 #pragma unroll
-        for (int h = 0; h < NB / RC; ++h) {
-          if (h * RC >= a.batch) break;
-          if (first_sum) wait_phase(red_empty, ph_red, tries, a.error_flag);
-#pragma unroll
-          for (int n = 0; n < RC; ++n)
-            if (h * RC + n < a.batch) {
-              const uint32_t at = red_at + n * kTileRows * 4;
-              float s = v[h * RC + n];
-              if (by_block) {
-                if (first_sum) s *= pend_scale;
-                else s = fmaf(pend_scale, s, lds32f(at));
+            for (int i = 0; i < 4; ++i) {
+              const uint32_t at = red_at + (n + i) * kTileRows * 4;
+              float s = pend_zero ? 0.f : v[i];
+              if (kExact) {
+                const float before = lds32f(at);
+                s = fmaf(pend_scale, s, first_sum ? 0.f : before);
               }
               sts32f(at, s);
             }
+          }
           if (pend_last) {
             __syncwarp();
             if (lane == 0) mbar_arrive(red_full);
             ph_red ^= 1u;
           }
         }
+        tc_fence_before();
         first_sum = pend_last;
         if (!more) break;
       }
@@ -730,7 +744,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
             tile = f.tile;
             f.range(a, quad, u, end);
             f.next(a);
-            bcol = u / block_units - 1;
+            bcol = divide(u, a.block_inv) - 1;
             block_left = 0;
           }
         }
@@ -749,7 +763,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         for (int i = 0; i < F::STAGES / 2; ++i)
           scales[i] = __ldg(reinterpret_cast<const unsigned short*>(gs) + u * (F::UC / 128) + i) * 0x10001u;
       }
-      wait_phase(idx_full + 8 * islot, ph_i, tries, a.error_flag);
+      wait_phase(idx_full + 8 * islot, ph_i, tries);
       uint32_t w[F::RB / 4];
       {
         const uint32_t row_at = idx_at + islot * F::IDX_BYTES + qt * F::RB;
@@ -797,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           if (nu < nend) {
             const Segment& sg = a.seg[segment_of(a, f.tile)];
             tb.open(a, sg, (f.tile - sg.tile0) * kTileRows, qt);
-            tb.request(a, nu / block_units);
+            tb.request(a, divide(nu, a.block_inv));
             asked = true;
           }
         }
@@ -812,7 +826,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           for (int i = 0; i < 32; ++i) r[i] = mul_f16x2(r[i], scales[J / 2]);
         }
         // (the place's use number is st * STAGES / 2 + J / 2)
-        wait_phase(a_empty + 8 * (J & 1), F::STAGES == 2 ? (st & 1) ^ 1 : ((J >> 1) & 1) ^ 1, tries, a.error_flag);
+        wait_phase(a_empty + 8 * (J & 1), F::STAGES == 2 ? (st & 1) ^ 1 : ((J >> 1) & 1) ^ 1, tries);
         __syncwarp();
         tc_fence_after();
         tc_store32(tmem_a + (J & 1) * 32, r);
@@ -828,6 +842,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       ++st;
     }
   }
+  if (tries == 0 && lane == 0) atomicAdd(a.error_flag, 1);   // a wait of this warp ran out
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -839,18 +854,17 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     uint32_t slab;
     asm volatile("ld.shared.b32 %0, [%1];" : "=r"(slab) : "r"(last_tile + 4 * i) : "memory");
     const int tile = static_cast<int>(slab);
-    const unsigned T = a.tail_steps, Pt = a.tail_ctas;
-    const unsigned first_s = (tile - a.tail_tile0) * a.steps;
-    const int c_first = static_cast<int>(((first_s + 1) * Pt - 1) / T), c_last = static_cast<int>(((first_s + a.steps) * Pt - 1) / T);
+    const int s0 = (tile - a.tail_tile0) * a.steps;
+    const int c_first = step_owner(a, s0), c_last = step_owner(a, s0 + a.steps - 1);
     const Segment& sg = a.seg[segment_of(a, tile)];
     const int r = tid & 127, row = (tile - sg.tile0) * kTileRows + r;
+    const int per_cta = 2 * a.batch * kTileRows;
     for (int n = tid >> 7; n < a.batch && tid < kThreads / 128 * 128; n += kThreads / 128) {
-      float s = 0.f;
+      // the first CTA's share lies in its second slot unless its piece begins with the tile
+      const float* p = a.ws_part + static_cast<long long>(c_first) * per_cta + n * kTileRows + r;
+      float s = __ldcg(p + (first_step(a, c_first) == s0 ? 0 : a.batch * kTileRows));
 #pragma unroll 4
-      for (int qc = c_first; qc <= c_last; ++qc) {
-        const int q_slot = a.tail_tile0 + static_cast<int>(T * qc / Pt) / a.steps == tile ? 0 : 1;
-        s += __ldcg(a.ws_part + ((static_cast<long long>(qc) * 2 + q_slot) * a.batch + n) * kTileRows + r);
-      }
+      for (int qc = c_first + 1; qc <= c_last; ++qc) s += __ldcg(p += per_cta);
       if (row < sg.N) sg.Y[static_cast<long long>(n) * sg.N + row] = __float2half_rn(s);
     }
   }
@@ -870,9 +884,9 @@ int env_int(const char* name, int dflt) {
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-template <class F, int NB>
+template <class F>
 vq_status launch(const StreamCall& call, cudaStream_t s) {
-  auto kern = tile_kernel<F, NB>;
+  auto kern = tile_kernel<F>;
   constexpr size_t kSmemCap = 227 * 1024;
   static int attr_set[kMaxDevices] = {};
   int dev = 0, sms = 0;
@@ -909,14 +923,15 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
 
   // ---- shared memory: activations, indices, sums, barriers, then the tables on their boundary ----
   const int x_rows = call.batch <= 8 ? 8 : 16;
-  constexpr int RC = NB == 8 ? 8 : F::RC16;
+  const int cols = call.batch <= 8 ? 8 : F::RC16;
+  a.red_cols = call.batch < cols ? (call.batch + 3) / 4 * 4 : cols;
   a.x_row_bytes = x_rows * 128;
   a.x_bytes = F::STAGES * a.x_row_bytes;
   auto plan = [&](int D) {
     a.D = D;
     a.idx_off = kQuads * D * a.x_bytes;
     a.red_off = a.idx_off + kQuads * D * F::IDX_BYTES;
-    a.bar_off = a.red_off + kQuads * (call.batch < RC ? call.batch : RC) * kTileRows * 4;
+    a.bar_off = a.red_off + kQuads * a.red_cols * kTileRows * 4;
     a.front_bytes = a.bar_off + kBarBytes;
     // (dynamic shared memory starts 1024 bytes into the window)
     return round_up(1024 + a.front_bytes, F::ALIGN) - 1024 + F::TABLES;
@@ -938,9 +953,14 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   const int left = static_cast<int>(tiles - a.q * P);
   const long long tail = static_cast<long long>(left) * a.steps;
   a.tail_tile0 = static_cast<int>(a.q * P);
-  a.tail_steps = static_cast<int>(tail);
-  a.tail_ctas = static_cast<int>(tail < P ? tail : P);
-  if (tail * (a.tail_ctas + 1) >= (1LL << 31)) return VQ_ERR_UNSUPPORTED;   // 32-bit arithmetic in the kernel
+  if (steps * a.steps >= (1LL << 31) || steps * (tail / P + 1) >= (1LL << 31) || static_cast<long long>(a.S) * a.S >= (1LL << 31)) return VQ_ERR_UNSUPPORTED;   // divide()
+  a.share = static_cast<int>(tail / P);
+  a.longer = static_cast<int>(tail % P);
+  auto inverse = [](long long d) { return d > 1 ? static_cast<unsigned>(((1LL << 32) + d - 1) / d) : 0u; };
+  a.steps_inv = inverse(a.steps);
+  a.share_inv = inverse(a.share);
+  a.share1_inv = inverse(a.share + 1);
+  a.block_inv = inverse(g.Bc / F::UC);
   // counters at the start, partial sums at the end of the workspace: a call with fewer rows then never writes
   // sums where one with more rows keeps its counters
   const size_t ticket_bytes = stream_ticket_bytes(rows_total);
@@ -978,15 +998,10 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   cfg.attrs = attr;
   cfg.numAttrs = env_int("VQ_PDL", 1) ? 1 : 0;
 #ifdef VQ_TUNING
-  if (env_int("VQ_VERBOSE", 0)) fprintf(stderr, "tile launch: grid %d depth %d smem %zu tiles %d S %d steps %d q %d tail %d/%d\n", (int)P, D, smem_bytes, tiles, a.S, a.steps, a.q, a.tail_steps, a.tail_ctas);
+  if (env_int("VQ_VERBOSE", 0)) fprintf(stderr, "tile launch: grid %d depth %d smem %zu tiles %d S %d steps %d q %d share %d+%d\n", (int)P, D, smem_bytes, tiles, a.S, a.steps, a.q, a.share, a.longer);
 #endif
   if (cudaLaunchKernelEx(&cfg, kern, maps, a) != cudaSuccess) return VQ_ERR_CUDA;
   return check_launch();
-}
-
-template <class F>
-vq_status launch_nb(const StreamCall& call, cudaStream_t s) {
-  return call.batch <= 8 ? launch<F, 8>(call, s) : launch<F, 16>(call, s);
 }
 
 }  // namespace
@@ -1049,19 +1064,19 @@ bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
 vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {
   const Geometry& g = call.g;
   if (!tile_covers(g) || call.n_seg < 1 || call.n_seg > kMaxSegments) return VQ_ERR_UNSUPPORTED;
-  if (g.d == 2 && g.b == 4) return launch_nb<Fmt<2, 4, kRow, 1, false>>(call, s);
-  if (g.d == 4) return launch_nb<Fmt<4, 8, kCta, 128, false>>(call, s);
+  if (g.d == 2 && g.b == 4) return launch<Fmt<2, 4, kRow, 1, false>>(call, s);
+  if (g.d == 4) return launch<Fmt<4, 8, kCta, 128, false>>(call, s);
   if (g.Br % kTileRows == 0) {
-    if (g.b == 6) return g.cb_int4 ? launch_nb<Fmt<2, 6, kCta, 128, true>>(call, s) : launch_nb<Fmt<2, 6, kCta, 128, false>>(call, s);
-    return g.cb_int4 ? launch_nb<Fmt<2, 5, kCta, 128, true>>(call, s) : launch_nb<Fmt<2, 5, kCta, 128, false>>(call, s);
+    if (g.b == 6) return g.cb_int4 ? launch<Fmt<2, 6, kCta, 128, true>>(call, s) : launch<Fmt<2, 6, kCta, 128, false>>(call, s);
+    return g.cb_int4 ? launch<Fmt<2, 5, kCta, 128, true>>(call, s) : launch<Fmt<2, 5, kCta, 128, false>>(call, s);
   }
   if (g.Br % 32 == 0) {
-    if (g.b == 6) return g.cb_int4 ? launch_nb<Fmt<2, 6, kWarp, 32, true>>(call, s) : launch_nb<Fmt<2, 6, kWarp, 32, false>>(call, s);
-    return g.cb_int4 ? launch_nb<Fmt<2, 5, kWarp, 32, true>>(call, s) : launch_nb<Fmt<2, 5, kWarp, 32, false>>(call, s);
+    if (g.b == 6) return g.cb_int4 ? launch<Fmt<2, 6, kWarp, 32, true>>(call, s) : launch<Fmt<2, 6, kWarp, 32, false>>(call, s);
+    return g.cb_int4 ? launch<Fmt<2, 5, kWarp, 32, true>>(call, s) : launch<Fmt<2, 5, kWarp, 32, false>>(call, s);
   }
-  if (g.Br == 16) return launch_nb<Fmt<2, 5, kWarp, 16, false>>(call, s);
-  if (g.Br == 8) return launch_nb<Fmt<2, 5, kWarp, 8, false>>(call, s);
-  return launch_nb<Fmt<2, 5, kWarp, 4, false>>(call, s);
+  if (g.Br == 16) return launch<Fmt<2, 5, kWarp, 16, false>>(call, s);
+  if (g.Br == 8) return launch<Fmt<2, 5, kWarp, 8, false>>(call, s);
+  return launch<Fmt<2, 5, kWarp, 4, false>>(call, s);
 }
 
 }  // namespace vq
