@@ -105,8 +105,11 @@ struct Fmt {
   static constexpr int D = D_, B = B_, TK = TK_, BR = BR_;
   static constexpr bool I4 = I4_;
   static constexpr int E = 1 << B;
-  // Columns of a unit: 256 where a row of 128 is no whole number of 16-byte pieces (5 bits) and for row tables, else 128.
-  static constexpr int UC = TK == kRow || (128 * B / (8 * D)) % 16 != 0 ? 256 : 128;
+#ifndef VQ_ROW_UC
+#define VQ_ROW_UC 128
+#endif
+  // Columns of a unit: 128, 256 where a row of 128 is no whole number of 16-byte pieces (5 bits).
+  static constexpr int UC = (TK == kRow && VQ_ROW_UC == 256) || (128 * B / (8 * D)) % 16 != 0 ? 256 : 128;
   static constexpr int RB = UC * B / (8 * D);       // bytes of a row of a unit
   static constexpr int IDX_BYTES = kTileRows * RB;
   static constexpr int STAGES = UC / kStageCols;
@@ -274,9 +277,8 @@ struct Units {
       f.range(a, k, u, end);
     }
   }
-  __device__ __forceinline__ void init(const TileArgs& a, int c, int k) {
-    f.init(a, c);
-    if (!f.valid) return;
+  __device__ __forceinline__ void init(const TileArgs& a, const Walk& first, int k) {
+    f = first;
     f.range(a, k, u, end);
     settle(a, k);
   }
@@ -461,14 +463,15 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   // barriers of a quad: indices and activations of a unit, decoded stages full and consumed, sums ready; then the CTA's
   const uint32_t bars = base + a.bar_off, qb = bars + quad * 112;
   const uint32_t idx_full = qb, x_full = qb + 32, a_full = qb + 64, a_empty = qb + 80, d_full = qb + 96;
-  const uint32_t red_full = bars + 448, red_empty = red_full + 8, tmem_slot = red_full + 16, n_last = tmem_slot + 4, last_tile = n_last + 4;
+  const uint32_t red_full = bars + 448, red_empty = red_full + 8, tmem_slot = red_full + 16, n_last = tmem_slot + 4, last_tile = n_last + 12;
   const uint32_t idx_at = base + a.idx_off + quad * D * F::IDX_BYTES, x_at = base + quad * D * a.x_bytes;
   const bool service = warp >= kDecodeWarps && warp < kResultsWarp;
 
   int tries = kWaitTries;
-  // (service warps) the next unit whose indices are to be requested; columns of the units requested first
-  Units wi;
-  int islot = 0, xu[kMaxDepth] = {};
+  Walk f;
+  f.init(a, c);
+  Units wi;   // (service warps) the next unit whose indices are to be requested
+  int islot = 0, first_x = 0, first_n = 0;   // the units requested first: lane i keeps the i-th
   auto request_indices = [&]() {
     if (elect_one()) {
       const int g = segment_of(a, wi.f.tile);
@@ -478,7 +481,28 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     __syncwarp();
     if (++islot == D) islot = 0;
   };
-  if (service) {
+  auto request_first = [&]() {
+    request_indices();
+    if (lane == first_n) first_x = wi.u;
+    ++first_n;
+    wi.next(a, quad);
+  };
+  // (decoding warps) the current fragment: its tile, next unit of the quad, end, codebook block column; f: the fragment after it
+  Tables<F> tb;
+  const int qt = tid & 127;   // row of the tile
+  int tile = f.tile, u = 0, end = 0, bcol = 0;
+  bool asked = false;         // are the entries of the next block to be used on their way?
+  if (warp < kDecodeWarps) {
+    f.range(a, quad, u, end);
+    f.next(a);
+    bcol = divide(u, a.block_inv) - 1;
+    asked = u < end;
+    if (asked) {
+      const Segment& sg = a.seg[segment_of(a, tile)];
+      tb.open(a, sg, (tile - sg.tile0) * kTileRows, qt);
+      tb.request(a, bcol + 1);
+    }
+  } else if (service) {
     if (elect_one()) {
       for (int i = 0; i < D; ++i) {
         mbar_init(idx_full + 8 * i, 1);
@@ -492,14 +516,8 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       mbar_init_fence();
     }
     __syncwarp();
-    wi.init(a, c, quad);
-#pragma unroll
-    for (int i = 0; i < kMaxDepth; ++i)
-      if (i < D && wi.f.valid) {   // (weights do not depend on the previous kernel)
-        request_indices();
-        xu[i] = wi.u + 1;
-        wi.next(a, quad);
-      }
+    wi.init(a, f, quad);
+    if (wi.f.valid) request_first();   // (weights do not depend on the previous kernel)
   } else if (warp == kResultsWarp) {
     if (lane == 0) {
       mbar_init(red_full, kDecodeWarps);
@@ -530,13 +548,12 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       __syncwarp();
       if (++xslot == D) xslot = 0;
     };
+#pragma unroll 1
+    while (first_n < D && wi.f.valid) request_first();
     pdl_wait();   // the activations belong to the previous kernel of the stream until here
-#pragma unroll
-    for (int i = 0; i < kMaxDepth; ++i)
-      if (xu[i]) request_x(xu[i] - 1);
-    Walk f;
-    f.init(a, c);
-    int u = 0, end = 0, x_next = -1;   // the unit to be multiplied; column of the unit whose activations are to be requested
+#pragma unroll 1
+    for (int i = 0; i < first_n; ++i) request_x(__shfl_sync(0xffffffffu, first_x, i));
+    int x_next = -1;   // (u: the unit to be multiplied) the unit whose activations are to be requested
     int slot = 0, seg = 0, seg_left = 0, st = 0;
     uint32_t ph = 0, fresh = 1;
     for (;; ++st) {
@@ -590,8 +607,6 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   } else if (warp == kResultsWarp) {
     // ---- results: adds the quads' sums of a fragment, stores the outputs or this CTA's share of them --------------
     pdl_wait();   // outputs and workspace belong to earlier kernels of the stream until here
-    Walk f;
-    f.init(a, c);
     const int first_tile = f.tile;   // (of the CTA's piece, if it has one)
     uint32_t ph = 0;
     int listed = 0;
@@ -601,8 +616,14 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       const int row = (f.tile - sg.tile0) * kTileRows + 4 * lane;
       // this CTA's share of a left-over tile: slot 0 if its piece begins inside the tile, else slot 1
       float* part = a.ws_part + (static_cast<long long>(c) * 2 + (f.tile == first_tile ? 0 : 1)) * (kTileRows * a.batch) + 4 * lane;
-      const int first_s = (f.tile - a.tail_tile0) * a.steps;
-      const int shares = complete ? 1 : step_owner(a, first_s + a.steps - 1) - step_owner(a, first_s) + 1;
+      int c_first = 0, shares = 1;   // CTAs that share the tile
+      if (!complete) {
+        const int first_s = (f.tile - a.tail_tile0) * a.steps;
+        c_first = step_owner(a, first_s);
+        shares = step_owner(a, first_s + a.steps - 1) - c_first + 1;
+        // where the first of them keeps its share: in its second slot unless its piece begins with the tile
+        c_first = 2 * c_first + (first_step(a, c_first) == first_s ? 0 : 1);
+      }
       for (int n0 = 0; n0 < a.batch; n0 += red_cols) {
         wait_phase(red_full, ph, tries);
         __syncwarp();
@@ -640,7 +661,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           const int ticket = atomicAdd(a.ws_ticket + f.tile, 1);
           if (ticket == shares - 1) {   // every share of the tile is there: this CTA adds them when it has done its own work
             a.ws_ticket[f.tile] = 0;          // nobody else touches the counter in this call
-            sts32(last_tile + 4 * listed, f.tile);
+            sts128(last_tile + 16 * listed, make_uint4(segment_of(a, f.tile), row - 4 * lane, c_first, shares));
             ++listed;
           }
         }
@@ -654,8 +675,6 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     // ---- decode ----------------------------------------------------------------------------------------------
     // One loop over units; what is not done in every unit stands in one place each (a codebook block, a running sum
     // and a fragment are whole units): the loop has to stay small enough for the instruction cache.
-    const int qt = tid & 127;   // row of the tile
-    Tables<F> tb;
     const uint32_t my_table = tables + (F::TK == kRow ? (warp >> 1) * F::TABLE + (warp & 1) * 128 : F::TK == kWarp ? warp * F::TABLE : quad * F::BUFS * F::TABLE);
     const uint32_t lane_off = F::D == 4 ? (lane & 15) * 8 : lane * 4;
     const uint32_t pat = ((my_table >> 12) & 0xFu) * 0x10101010u;
@@ -667,18 +686,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     int half = 0;
     uint32_t ph_i = 0, ph_red = 1;
 
-    Walk f;        // the fragment after the current one
-    f.init(a, c);
-    int tile = f.tile, u, end;   // the current fragment: next unit of the quad, end
-    f.range(a, quad, u, end);
-    f.next(a);
-    int bcol = divide(u, a.block_inv) - 1, block_left = 0;   // codebook block column, units left in it
-    bool asked = u < end;                             // are the entries of the next block to be used on their way?
-    if (asked) {
-      const Segment& sg = a.seg[segment_of(a, tile)];
-      tb.open(a, sg, (tile - sg.tile0) * kTileRows, qt);
-      tb.request(a, bcol + 1);
-    }
+    int block_left = 0;   // units left in the codebook block
     // The running sum, and one that is complete but not yet read (`pend_*`): it is read a unit or two later, when the tensor
     // core has caught up.
     int st = 0, seg = 0, seg_left = 0, seg_units = 0, fin_at = -1;
@@ -851,20 +859,15 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   uint32_t listed;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(listed) : "r"(n_last) : "memory");
   for (uint32_t i = 0; i < listed; ++i) {
-    uint32_t slab;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(slab) : "r"(last_tile + 4 * i) : "memory");
-    const int tile = static_cast<int>(slab);
-    const int s0 = (tile - a.tail_tile0) * a.steps;
-    const int c_first = step_owner(a, s0), c_last = step_owner(a, s0 + a.steps - 1);
-    const Segment& sg = a.seg[segment_of(a, tile)];
-    const int r = tid & 127, row = (tile - sg.tile0) * kTileRows + r;
-    const int per_cta = 2 * a.batch * kTileRows;
+    const uint4 sum = lds128(last_tile + 16 * i);
+    const Segment& sg = a.seg[sum.x];
+    const int r = tid & 127, row = sum.y + r, part_floats = a.batch * kTileRows;
     for (int n = tid >> 7; n < a.batch && tid < kThreads / 128 * 128; n += kThreads / 128) {
-      // the first CTA's share lies in its second slot unless its piece begins with the tile
-      const float* p = a.ws_part + static_cast<long long>(c_first) * per_cta + n * kTileRows + r;
-      float s = __ldcg(p + (first_step(a, c_first) == s0 ? 0 : a.batch * kTileRows));
+      const float* p = a.ws_part + static_cast<long long>(sum.z) * part_floats + n * kTileRows + r;
+      float s = __ldcg(p);
+      p += ((sum.z & 1) ? 1 : 2) * part_floats;   // the others' shares: in their first slots
 #pragma unroll 4
-      for (int qc = c_first + 1; qc <= c_last; ++qc) s += __ldcg(p += per_cta);
+      for (uint32_t k = 1; k < sum.w; ++k, p += 2 * part_floats) s += __ldcg(p);
       if (row < sg.N) sg.Y[static_cast<long long>(n) * sg.N + row] = __float2half_rn(s);
     }
   }
