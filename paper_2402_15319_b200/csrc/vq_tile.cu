@@ -86,7 +86,7 @@ struct TileArgs {
   unsigned steps_inv, share_inv, share1_inv, block_inv;   // 2^32 / divisor, rounded up, for divide()
   int q;              // whole tiles per CTA
   int tail_tile0;     // the tiles left over: their steps are shared by the CTAs,
-  int share, longer;  // share + 1 each for the first `longer` CTAs, share for the others
+  int sharers, share, longer;  // `sharers` of them, share + 1 each for the first `longer`, share for the others
   int blocks_per_row, Br, Bc, cb_int8;
   int D;              // unit stages of a quad
   int x_bytes, x_row_bytes;    // activations of a unit; bytes of one 64-column group of them
@@ -106,7 +106,7 @@ struct Fmt {
   static constexpr bool I4 = I4_;
   static constexpr int E = 1 << B;
 #ifndef VQ_ROW_UC
-#define VQ_ROW_UC 128
+#define VQ_ROW_UC 256
 #endif
   // Columns of a unit: 128, 256 where a row of 128 is no whole number of 16-byte pieces (5 bits).
   static constexpr int UC = (TK == kRow && VQ_ROW_UC == 256) || (128 * B / (8 * D)) % 16 != 0 ? 256 : 128;
@@ -224,7 +224,7 @@ __device__ __forceinline__ uint32_t nibble_pair(uint32_t byte) {   // two signed
 // x / d for x * d < 2^32 and inv = ceil(2^32 / d)  (d = 1: inv = 0)
 __device__ __forceinline__ int divide(int x, unsigned inv) { return inv ? static_cast<int>(__umulhi(static_cast<unsigned>(x), inv)) : x; }
 // first step of CTA c's piece of the left-over tiles, and the CTA whose piece holds step x
-__device__ __forceinline__ int first_step(const TileArgs& a, int c) { return c * a.share + min(c, a.longer); }
+__device__ __forceinline__ int first_step(const TileArgs& a, int c) { return min(c, a.sharers) * a.share + min(c, a.longer); }
 __device__ __forceinline__ int step_owner(const TileArgs& a, int x) {
   const int n = a.longer * (a.share + 1);
   return x < n ? divide(x, a.share1_inv) : a.longer + divide(x - n, a.share_inv);
@@ -628,6 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         wait_phase(red_full, ph, tries);
         __syncwarp();
         const int cols = min(red_cols, a.batch - n0);
+#pragma unroll 2
         for (int n = 0; n < cols; ++n) {
           float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -862,13 +863,32 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     const uint4 sum = lds128(last_tile + 16 * i);
     const Segment& sg = a.seg[sum.x];
     const int r = tid & 127, row = sum.y + r, part_floats = a.batch * kTileRows;
-    for (int n = tid >> 7; n < a.batch && tid < kThreads / 128 * 128; n += kThreads / 128) {
-      const float* p = a.ws_part + static_cast<long long>(sum.z) * part_floats + n * kTileRows + r;
-      float s = __ldcg(p);
-      p += ((sum.z & 1) ? 1 : 2) * part_floats;   // the others' shares: in their first slots
-#pragma unroll 4
-      for (uint32_t k = 1; k < sum.w; ++k, p += 2 * part_floats) s += __ldcg(p);
-      if (row < sg.N) sg.Y[static_cast<long long>(n) * sg.N + row] = __float2half_rn(s);
+    const float* p = a.ws_part + static_cast<long long>(sum.z) * part_floats + r;
+    const int others = (sum.z & 1 ? -1 : 0) * part_floats;   // (the CTAs behind the first keep their shares in their first slots)
+    constexpr int G = kThreads / 128;
+#pragma unroll 1
+    for (int n = tid >> 7; n < a.batch && tid < G * 128; n += 2 * G) {
+      float s[2] = {};
+#pragma unroll 1
+      for (uint32_t k0 = 0; k0 < sum.w; k0 += 4) {   // (a load takes about 1000 clocks: eight at a time)
+        float v[4][2];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            v[k][i] = 0.f;
+            if (k0 + k < sum.w && n + i * G < a.batch)
+              v[k][i] = __ldcg(p + (2 * (k0 + k)) * part_floats + (k0 + k ? others : 0) + (n + i * G) * kTileRows);
+          }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          s[0] += v[k][0];
+          s[1] += v[k][1];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (row < sg.N && n + i * G < a.batch) sg.Y[static_cast<long long>(n + i * G) * sg.N + row] = __float2half_rn(s[i]);
     }
   }
 }
@@ -956,9 +976,15 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   const int left = static_cast<int>(tiles - a.q * P);
   const long long tail = static_cast<long long>(left) * a.steps;
   a.tail_tile0 = static_cast<int>(a.q * P);
-  if (steps * a.steps >= (1LL << 31) || steps * (tail / P + 1) >= (1LL << 31) || static_cast<long long>(a.S) * a.S >= (1LL << 31)) return VQ_ERR_UNSUPPORTED;   // divide()
-  a.share = static_cast<int>(tail / P);
-  a.longer = static_cast<int>(tail % P);
+  if (steps * a.steps >= (1LL << 31) || steps * (tail + 1) >= (1LL << 31) || static_cast<long long>(a.S) * a.S >= (1LL << 31)) return VQ_ERR_UNSUPPORTED;   // divide()
+  // A tile is shared by eight CTAs at most where every CTA has whole ones.
+  long long Pt = P;
+  const int cap = env_int("VQ_CAP", 8);
+  if (a.q > 0 && Pt > static_cast<long long>(left) * cap) Pt = static_cast<long long>(left) * cap;
+  if (tail > 0 && tail < Pt) Pt = tail;
+  a.sharers = static_cast<int>(Pt);
+  a.share = Pt ? static_cast<int>(tail / Pt) : 0;
+  a.longer = Pt ? static_cast<int>(tail % Pt) : 0;
   auto inverse = [](long long d) { return d > 1 ? static_cast<unsigned>(((1LL << 32) + d - 1) / d) : 0u; };
   a.steps_inv = inverse(a.steps);
   a.share_inv = inverse(a.share);
