@@ -296,6 +296,20 @@ __device__ __forceinline__ int segment_of(const TileArgs& a, int tile) {
   return g;
 }
 
+// outputs of rows row .. row + 3 of one sequence
+__device__ __forceinline__ void store_rows(const Segment& sg, int row, int n, float4 s) {
+  __half* y = sg.Y + static_cast<long long>(n) * sg.N + row;
+  const __half2 lo = __floats2half2_rn(s.x, s.y), hi = __floats2half2_rn(s.z, s.w);
+  if (sg.N % 4 == 0) {   // (the rows then exist together, 8-byte aligned)
+    if (row < sg.N) *reinterpret_cast<uint2*>(y) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+  } else {
+    if (row < sg.N) y[0] = __low2half(lo);
+    if (row + 1 < sg.N) y[1] = __high2half(lo);
+    if (row + 2 < sg.N) y[2] = __low2half(hi);
+    if (row + 3 < sg.N) y[3] = __high2half(hi);
+  }
+}
+
 // ---- look-up tables: request a block's entries (registers), write them as table words --------------------------
 template <class F>
 struct Tables {
@@ -639,16 +653,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           if (!complete) {
             *reinterpret_cast<float4*>(part + (n0 + n) * kTileRows) = s;
           } else {
-            __half* y = sg.Y + static_cast<long long>(n0 + n) * sg.N + row;
-            const __half2 lo = __floats2half2_rn(s.x, s.y), hi = __floats2half2_rn(s.z, s.w);
-            if (sg.N % 4 == 0) {   // (rows 4 l .. 4 l + 3 then exist together, 8-byte aligned)
-              if (row < sg.N) *reinterpret_cast<uint2*>(y) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-            } else {
-              if (row < sg.N) y[0] = __low2half(lo);
-              if (row + 1 < sg.N) y[1] = __high2half(lo);
-              if (row + 2 < sg.N) y[2] = __low2half(hi);
-              if (row + 3 < sg.N) y[3] = __high2half(hi);
-            }
+            store_rows(sg, row, n0 + n, s);
           }
         }
         __syncwarp();
@@ -658,12 +663,36 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       if (!complete) {
         __threadfence();   // this lane's sums are visible to the GPU before the ticket is drawn
         __syncwarp();
+        int ticket = 0;
         if (lane == 0) {
-          const int ticket = atomicAdd(a.ws_ticket + f.tile, 1);
-          if (ticket == shares - 1) {   // every share of the tile is there: this CTA adds them when it has done its own work
-            a.ws_ticket[f.tile] = 0;          // nobody else touches the counter in this call
-            sts128(last_tile + 16 * listed, make_uint4(segment_of(a, f.tile), row - 4 * lane, c_first, shares));
+          ticket = atomicAdd(a.ws_ticket + f.tile, 1);
+          if (ticket == shares - 1) a.ws_ticket[f.tile] = 0;   // nobody else touches the counter in this call
+        }
+        ticket = __shfl_sync(0xffffffffu, ticket, 0);
+        if (ticket == shares - 1) {   // every share of the tile is there
+          if (a.q == 0) {             // this CTA adds them when it has done its own work, by all its threads
+            if (lane == 0) sts128(last_tile + 16 * listed, make_uint4(segment_of(a, f.tile), row - 4 * lane, c_first, shares));
             ++listed;
+          } else {                    // whole tiles are still to come: this warp adds them meanwhile
+            __threadfence();
+            const int part_floats = a.batch * kTileRows;
+            const float* p = a.ws_part + static_cast<long long>(c_first) * part_floats + 4 * lane;
+            const int others = (c_first & 1 ? -1 : 0) * part_floats;   // (behind the first: in their first slots)
+#pragma unroll 1
+            for (int n = 0; n < a.batch; ++n, p += kTileRows) {
+              float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+              for (int k0 = 0; k0 < shares; k0 += 8) {
+                float4 v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                  if (k0 + k < shares) v[k] = __ldcg(reinterpret_cast<const float4*>(p + 2 * (k0 + k) * part_floats + (k0 + k ? others : 0)));
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                  if (k0 + k < shares) s.x += v[k].x, s.y += v[k].y, s.z += v[k].z, s.w += v[k].w;
+              }
+              store_rows(sg, row, n, s);
+            }
           }
         }
       }
@@ -969,6 +998,13 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   const long long steps = static_cast<long long>(tiles) * a.steps;
   long long P = sms < kMaxStreamCtas ? sms : kMaxStreamCtas;
   if (P > steps) P = steps;
+  // As many CTAs for every tile, and so one piece of one tile for each, where that costs at most half a step more than pieces
+  // that end anywhere: a second piece costs its own tables, sums and share of a tile.
+  for (long long k = P / tiles; k >= 1; --k)
+    if (a.steps % k == 0) {
+      if (2 * P * (a.steps / k) <= 2 * steps + P * env_int("VQ_SLACK", 3)) P = tiles * k;
+      break;
+    }
 #ifdef VQ_TUNING
   if (env_int("VQ_TP", 0) && P > env_int("VQ_TP", 0)) P = env_int("VQ_TP", 0);
 #endif
