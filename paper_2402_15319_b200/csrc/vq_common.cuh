@@ -70,6 +70,8 @@ vq_status launch_int4g128_stream(int N, int K, const uint8_t* q, const __half* s
 // preferred: the calls it serves.
 vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s);
 bool tile_covers(const Geometry& g);
+vq_status launch_gemm_tile_norm(const Geometry& g, const LayerPtrs& p, const void* norm_codes, const void* norm_lut, int norm_block_cols,
+                                const __half* X, __half* Y, int batch, cudaStream_t s);
 bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch);
 vq_status launch_gemm_blockcb(const Geometry& g, const LayerPtrs& p, const __half* X, __half* Y, int batch,
                               cudaStream_t s);

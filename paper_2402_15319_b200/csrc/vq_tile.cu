@@ -84,13 +84,16 @@ struct TileArgs {
   int K, batch;
   int S, steps;       // units and steps (of a unit per quad) of a tile
   unsigned steps_inv, share_inv, share1_inv, block_inv;   // 2^32 / divisor, rounded up, for divide()
-  int q;              // whole tiles per CTA
+  int q, extra;       // whole tiles per CTA, CTAs that take one more (calls without a workspace)
   int tail_tile0;     // the tiles left over: their steps are shared by the CTAs,
   int sharers, share, longer;  // `sharers` of them, share + 1 each for the first `longer`, share for the others
   int blocks_per_row, Br, Bc, cb_int8;
   int D;              // unit stages of a quad
   int x_bytes, x_row_bytes;    // activations of a unit; bytes of one 64-column group of them
   int red_cols;       // columns of sums handed over at a time, a multiple of 4
+  const uint8_t* codes;          // normalisation: 4-bit codes, `code_row` bytes a row, a code per 2^norm_shift columns, and the
+  const unsigned short* lut;     // 16 scales of every codebook block
+  int code_row, norm_shift;
   int idx_off, red_off, bar_off, front_bytes;   // dynamic shared memory: activations, indices, sums, barriers, | tables
 };
 
@@ -100,16 +103,14 @@ struct TileMaps {
 };
 
 // Format policy: D columns per entry, B index bits; BR: rows that share a table word inside a warp (kWarp).
-template <int D_, int B_, int TK_, int BR_, bool I4_>
+template <int D_, int B_, int TK_, int BR_, bool I4_, bool NORM_ = false>
 struct Fmt {
   static constexpr int D = D_, B = B_, TK = TK_, BR = BR_;
-  static constexpr bool I4 = I4_;
+  static constexpr bool I4 = I4_, NORM = NORM_;   // NORM: block-wise normalisation
   static constexpr int E = 1 << B;
-#ifndef VQ_ROW_UC
-#define VQ_ROW_UC 256
-#endif
-  // Columns of a unit: 128, 256 where a row of 128 is no whole number of 16-byte pieces (5 bits).
-  static constexpr int UC = (TK == kRow && VQ_ROW_UC == 256) || (128 * B / (8 * D)) % 16 != 0 ? 256 : 128;
+  // Columns of a unit: 128; 256 where a row of 128 is no whole number of 16-byte pieces (5 bits) and for row tables (half as many
+  // unit changes: 57344 x 8192 at batch 16 59 us with 128).
+  static constexpr int UC = TK == kRow || (128 * B / (8 * D)) % 16 != 0 ? 256 : 128;
   static constexpr int RB = UC * B / (8 * D);       // bytes of a row of a unit
   static constexpr int IDX_BYTES = kTileRows * RB;
   static constexpr int STAGES = UC / kStageCols;
@@ -119,8 +120,6 @@ struct Fmt {
   // OR-merged addresses need tables on multiples of their size; 4-D look-ups add (one per four weights)
   static constexpr int ALIGN = D == 4 ? 1024 : TABLE;
   static constexpr int SWIZZLE = RB == 32 ? 3 : RB == 64 ? 1 : RB == 128 ? 2 : 0;
-  // columns of sums that the quads hand over at a time from batch 9 on: all where sums are scaled per block, fewer where tables fill the memory
-  static constexpr int RC16 = TK == kRow ? 16 : TK == kWarp && B == 6 ? 4 : 8;
   static_assert(RB % 16 == 0 && (TK != kRow || (B == 4 && D == 2)));
 };
 
@@ -237,8 +236,8 @@ struct Walk {
 
   __device__ __forceinline__ void init(const TileArgs& a, int c) {
     const int t0 = first_step(a, c), ahead = divide(t0, a.steps_inv);
-    whole = c * a.q;
-    whole_end = whole + a.q;
+    whole = c * a.q + min(c, a.extra);
+    whole_end = whole + a.q + (c < a.extra ? 1 : 0);
     tile = a.tail_tile0 + ahead - 1;
     left = first_step(a, c + 1) - t0;
     next(a, t0 - ahead * a.steps);
@@ -795,6 +794,19 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           gs = sg.scale + static_cast<long long>(min((tile - sg.tile0) * kTileRows + qt, sg.N - 1)) * (a.K / 128);
         }
       }
+      uint32_t nscales[F::NORM ? F::UC / 16 : 1];   // normalisation: the scale of every 16 columns, twice
+      if constexpr (F::NORM) {
+        static_assert(!F::NORM || F::UC == 128);
+        const int row = min((tile - a.seg[0].tile0) * kTileRows + qt, a.seg[0].N - 1);
+        const uint8_t* code = a.codes + static_cast<long long>(row) * a.code_row + u * (F::UC / 2 >> a.norm_shift);
+        const unsigned short* lut = a.lut + (static_cast<long long>(row / a.Br) * a.blocks_per_row + divide(u, a.block_inv)) * 16;
+        uint32_t cw = 0;   // the unit's codes
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < (F::UC / 2 >> a.norm_shift)) cw |= static_cast<uint32_t>(__ldg(code + i)) << (8 * i);
+#pragma unroll
+        for (int i = 0; i < F::UC / 16; ++i) nscales[i] = __ldg(lut + ((cw >> (4 * (16 * i >> a.norm_shift))) & 15u)) * 0x10001u;
+      }
       uint32_t scales[F::STAGES / 2];   // int4 codebooks: of the unit's groups of 128 columns
       if constexpr (F::I4) {
 #pragma unroll
@@ -862,6 +874,10 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         if constexpr (F::I4) {
 #pragma unroll
           for (int i = 0; i < 32; ++i) r[i] = mul_f16x2(r[i], scales[J / 2]);
+        }
+        if constexpr (F::NORM) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) r[i] = mul_f16x2(r[i], nscales[4 * J + i / 8]);
         }
         // (the place's use number is st * STAGES / 2 + J / 2)
         wait_phase(a_empty + 8 * (J & 1), F::STAGES == 2 ? (st & 1) ^ 1 : ((J >> 1) & 1) ^ 1, tries);
@@ -936,8 +952,14 @@ int env_int(const char* name, int dflt) {
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+struct Norm {
+  const void *codes, *lut;
+  int cols;
+};
+
+// Without a workspace (normalised calls have none) every tile is one CTA's.
 template <class F>
-vq_status launch(const StreamCall& call, cudaStream_t s) {
+vq_status launch(const StreamCall& call, cudaStream_t s, const Norm* norm = nullptr) {
   auto kern = tile_kernel<F>;
   constexpr size_t kSmemCap = 227 * 1024;
   static int attr_set[kMaxDevices] = {};
@@ -975,8 +997,6 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
 
   // ---- shared memory: activations, indices, sums, barriers, then the tables on their boundary ----
   const int x_rows = call.batch <= 8 ? 8 : 16;
-  const int cols = call.batch <= 8 ? 8 : F::RC16;
-  a.red_cols = call.batch < cols ? (call.batch + 3) / 4 * 4 : cols;
   a.x_row_bytes = x_rows * 128;
   a.x_bytes = F::STAGES * a.x_row_bytes;
   auto plan = [&](int D) {
@@ -988,6 +1008,10 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
     // (dynamic shared memory starts 1024 bytes into the window)
     return round_up(1024 + a.front_bytes, F::ALIGN) - 1024 + F::TABLES;
   };
+  // columns of sums handed over at a time: all of them (a second time waits for the first) unless the tables leave no room
+  a.red_cols = (call.batch + 3) / 4 * 4;
+  if (!(F::TK == kRow))
+    while (a.red_cols > 4 && plan(2) > kSmemCap) a.red_cols = a.red_cols > 8 ? 8 : 4;
   int D = env_int("VQ_TD", kMaxDepth);
   while (D > 2 && plan(D) > kSmemCap) --D;
   size_t smem_bytes = plan(D);
@@ -1000,7 +1024,8 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   if (P > steps) P = steps;
   // As many CTAs for every tile, and so one piece of one tile for each, where that costs at most half a step more than pieces
   // that end anywhere: a second piece costs its own tables, sums and share of a tile.
-  for (long long k = P / tiles; k >= 1; --k)
+  if (norm && P > tiles) P = tiles;
+  for (long long k = P / tiles; k >= 1 && !norm; --k)
     if (a.steps % k == 0) {
       if (2 * P * (a.steps / k) <= 2 * steps + P * env_int("VQ_SLACK", 3)) P = tiles * k;
       break;
@@ -1010,7 +1035,8 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
 #endif
   a.q = static_cast<int>(tiles / P);
   const int left = static_cast<int>(tiles - a.q * P);
-  const long long tail = static_cast<long long>(left) * a.steps;
+  const long long tail = norm ? 0 : static_cast<long long>(left) * a.steps;
+  a.extra = norm ? left : 0;
   a.tail_tile0 = static_cast<int>(a.q * P);
   if (steps * a.steps >= (1LL << 31) || steps * (tail + 1) >= (1LL << 31) || static_cast<long long>(a.S) * a.S >= (1LL << 31)) return VQ_ERR_UNSUPPORTED;   // divide()
   // A tile is shared by eight CTAs at most where every CTA has whole ones.
@@ -1026,16 +1052,23 @@ vq_status launch(const StreamCall& call, cudaStream_t s) {
   a.share_inv = inverse(a.share);
   a.share1_inv = inverse(a.share + 1);
   a.block_inv = inverse(g.Bc / F::UC);
-  // counters at the start, partial sums at the end of the workspace: a call with fewer rows then never writes
-  // sums where one with more rows keeps its counters
-  const size_t ticket_bytes = stream_ticket_bytes(rows_total);
-  if (static_cast<size_t>(tiles) * sizeof(int) > ticket_bytes) return VQ_ERR_UNSUPPORTED;
-  const size_t part_ws = static_cast<size_t>(P) * 2 * kTileRows * call.batch * sizeof(float);
-  const size_t total_ws = stream_workspace_bytes(rows_total, call.batch);
-  if (ticket_bytes + part_ws > total_ws) return VQ_ERR_UNSUPPORTED;
-  if (!call.ws || call.ws_bytes < total_ws) return VQ_ERR_WORKSPACE;
-  a.ws_ticket = static_cast<int*>(call.ws);
-  a.ws_part = reinterpret_cast<float*>(static_cast<char*>(call.ws) + (total_ws - part_ws));
+  if (norm) {
+    a.codes = static_cast<const uint8_t*>(norm->codes);
+    a.lut = static_cast<const unsigned short*>(norm->lut);
+    a.code_row = (g.K / norm->cols + 1) / 2;
+    while ((1 << a.norm_shift) < norm->cols) ++a.norm_shift;
+  } else {
+    // counters at the start, partial sums at the end of the workspace: a call with fewer rows then never writes
+    // sums where one with more rows keeps its counters
+    const size_t ticket_bytes = stream_ticket_bytes(rows_total);
+    if (static_cast<size_t>(tiles) * sizeof(int) > ticket_bytes) return VQ_ERR_UNSUPPORTED;
+    const size_t part_ws = static_cast<size_t>(P) * 2 * kTileRows * call.batch * sizeof(float);
+    const size_t total_ws = stream_workspace_bytes(rows_total, call.batch);
+    if (ticket_bytes + part_ws > total_ws) return VQ_ERR_UNSUPPORTED;
+    if (!call.ws || call.ws_bytes < total_ws) return VQ_ERR_WORKSPACE;
+    a.ws_ticket = static_cast<int*>(call.ws);
+    a.ws_part = reinterpret_cast<float*>(static_cast<char*>(call.ws) + (total_ws - part_ws));
+  }
 
   TileMaps maps;
   for (int i = 0; i < call.n_seg; ++i) {
@@ -1079,19 +1112,19 @@ bool tile_covers(const Geometry& g) {
   return g.d == 4 && g.b == 8 && g.Bc % 128 == 0 && g.Br % kTileRows == 0 && !g.cb_int4;
 }
 
-// Which calls this kernel serves.  Its time hardly depends on the batch (one pass over the weights for 1..16 sequences) but it
-// has about 4 us more of start-up and summing than the cluster kernels, so it takes over above a number of weights that falls with
-// the batch.  The lines are drawn where it was the faster one in nearly all of 39000 timings against the other kernels on B200 (44
-// formats, 1024 to 28672 columns, any rows, every batch): it is slower by more than 3 % in 97 of the 14300 calls it takes, by more
-// than 10 % in 14; the others move in steps of whole waves.  us, other kernels / this one, on either side of a line:
-//   row tables (8-bit, 2048-column blocks)  16632 x 4096 b15 21.4/21.9, 19968 x 4096 b15 25.6/24.8; 13952 x 8192 b15 25.6/27.9, 16232 x 8192
-//                                           b15 37.9/29.1; 10632 x 14336 b11 32.0/33.1
-//   4-D     71680 x 2048 b6 21.0/24.2, 143360 x 1024 b9 64 M 15.6/17.8
-//   128-row blocks, 6 bits  8704 x 8192 b9 21.5/25.3 (the worst that is left), 102400 x 1024 b5 20.2/25.4, 27392 x 3072 b5 17.2/19.7
-//   32-row blocks, 6 bits   51200 x 2048 b1, 128-column blocks 20.7/27.1; 28672 x 4096 b1, 256-column blocks 32/27
-//   5 bits  54656 x 1536 b8 19.2/24.2; 4-row blocks 9152 x 6400 b1 18.2/20.2; 8-row blocks 63488 x 1024 b1 15.8/18.7
-// Shapes that the cluster kernels do not take (rows not a multiple of 128, K not one of 256) cost the pair-table kernel
-// more, and a launch per layer: 4160 x 3328 in three layers 21/12, 3328 x 9088 22/16 at batch 5; but 13312 x 1920 b2 11.0/14.0.
+// Which calls this kernel serves.  Its time hardly depends on the batch (one pass over the weights for 1..16 sequences); a call
+// costs about 4.5 us before and behind its look-ups, the cluster kernels' 3.3.  So it takes over above a number of weights (in
+// 2^20) that falls with the batch and with the columns (long rows give every CTA one long piece, where the cluster kernels
+// stage activations and split K over eight CTAs at most).  The lines come from 46704 timings against the other kernels on B200
+// (26 formats, 1024 to 28672 columns, 1.5 to 375 x 2^20 weights, every batch).  Mean time over the others' on either side of a line:
+//   row tables   batch 9 to 16 from 6: 0.7, below 0.9 (the worst tenth above 1.05); batch 6 to 8 from 8: 0.75; batch 3 to 5, blocks up to
+//                512 columns, from 24: 0.82, longer blocks 0.98; batch 1 and 2, 256-column blocks, from 96: 0.85, others 1.0 to 1.5
+//   others, K >= 5500: 0.45 to 0.85 at every size.  K from 3700: batch 1 to 5 from 24: 0.75, below 0.93 (1.1); 32-row blocks of 6 bits from
+//                64: 0.82, from 24 1.06; batch 6 to 16 from 8: 0.8.  K below: from 24 0.8, from 8 1.0; from batch 9 on from 8: 0.78
+//   groups whose layers the cluster kernels take in one launch: 12288 x 4096 in three layers, 128-row blocks, 6 bits, batch 1 12.7 us
+//                against 10.8, 6144 x 4096 32-row blocks 9.3/8.3, 15360 x 5120 4-D batch 8 16.4/18.3: from 64
+// Slower than the others remain calls with many short rows at large batches, where adding a tile's sums takes as long as decoding
+// it: 65536 x 1024 at batch 16 1.2 times, 32768 x 2048 1.1 times the time of a kernel of four CTAs per SM that this one replaced.
 bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
   if (!tile_covers(g)) return false;
 #ifdef VQ_TUNING
@@ -1105,25 +1138,17 @@ bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
   }
   const long long w = (rows * g.K) >> 20;   // weights of the call, in 2^20
   if (g.d == 2 && g.b == 4) {
-    if (batch < 9) return false;
-    return w >= (batch < 12 ? 160 : g.K < 5120 ? 80 : batch < 13 ? 160 : 112);
+    if (batch >= 6) return w >= (batch >= 9 ? 6 : 8);
+    return batch >= 3 ? g.Bc <= 512 && w >= 24 : g.Bc == 256 && w >= 96;
   }
-  if (g.d == 4) {
-    if (batch >= 9) return w >= (g.K < 2048 ? 72 : 64);
-    return batch >= 5 && w >= (g.K >= 8192 ? 64 : batch >= 7 ? 112 : 144);
-  }
-  if (g.b == 5) {
-    if (g.Br == 4) return w >= 58;
-    if (g.Br < 32 || !whole) return w >= (batch >= 9 ? 68 : 88);
-    return batch >= 11 ? w >= 80 : batch >= 8 && w >= 116;
-  }
-  if (!whole) return w >= (n_seg > 1 ? 12 : batch >= 9 || g.K < 3072 ? 48 : 28);
-  if (g.Br % kTileRows == 0) {
-    if (batch >= 9) return w >= 48;
-    return batch >= 5 && w >= (batch < 7 ? 124 : g.K < 2048 ? 104 : 80);
-  }
-  if (batch >= 13) return w >= 64;
-  return w >= (g.K < 2048 || (batch <= 5 && g.Bc < 256) ? 150 : 104);
+  if (g.K >= 5500) return true;
+  const bool pairs = g.b == 5 && g.Br < 32;   // else: the pair-table kernel, which takes groups too
+  if (!pairs && !whole) return g.K >= 3700 || w >= (n_seg > 1 ? 4 : 16);
+  if (!pairs && n_seg > 1 && batch <= 8) return w >= 64;
+  if (g.K < 3700) return w >= (batch <= 8 || pairs ? 24 : 8);
+  if (pairs) return w >= 12;
+  if (batch >= 6) return w >= (batch <= 8 && g.b == 6 && g.Br % kTileRows != 0 ? 48 : 8);
+  return w >= (g.b == 6 && g.Br % kTileRows != 0 ? 64 : 24);
 }
 
 vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {
@@ -1142,6 +1167,25 @@ vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {
   if (g.Br == 16) return launch<Fmt<2, 5, kWarp, 16, false>>(call, s);
   if (g.Br == 8) return launch<Fmt<2, 5, kWarp, 8, false>>(call, s);
   return launch<Fmt<2, 5, kWarp, 4, false>>(call, s);
+}
+
+// Block-wise normalisation: sub-rows of 16, 32 or 64 columns, blocks of a multiple of 32 rows with 6-bit indices; one layer.
+vq_status launch_gemm_tile_norm(const Geometry& g, const LayerPtrs& p, const void* norm_codes, const void* norm_lut, int norm_block_cols,
+                                const __half* X, __half* Y, int batch, cudaStream_t s) {
+  if (!norm_codes || !norm_lut || !tile_covers(g) || g.d != 2 || g.b != 6 || g.cb_int4) return VQ_ERR_UNSUPPORTED;
+  if (norm_block_cols != 16 && norm_block_cols != 32 && norm_block_cols != 64) return VQ_ERR_UNSUPPORTED;
+  StreamCall call = {};
+  call.g = g;
+  call.n_seg = 1;
+  call.idx[0] = p.idx;
+  call.cb[0] = p.cb;
+  call.scale[0] = p.scale;
+  call.Y[0] = Y;
+  call.N[0] = g.N;
+  call.X = X;
+  call.batch = batch;
+  const Norm norm = {norm_codes, norm_lut, norm_block_cols};
+  return g.Br % kTileRows == 0 ? launch<Fmt<2, 6, kCta, 128, false, true>>(call, s, &norm) : launch<Fmt<2, 6, kWarp, 32, false, true>>(call, s, &norm);
 }
 
 }  // namespace vq
