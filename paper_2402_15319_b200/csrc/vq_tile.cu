@@ -722,6 +722,19 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
     bool open_sum = false, first_sum = true, more = true, pend_last = false, pend_zero = false;
     float pend_scale = 1.f, block_scale = 1.f;
     const __half* gs = nullptr;   // int4 codebooks: the scales of the thread's row
+    const uint8_t* codes = nullptr;          // normalisation: the codes of the thread's row,
+    const unsigned short* lut = nullptr;     // the scales of its blocks,
+    uint32_t code_word = 0;                  // and the codes of the next unit, requested a unit ahead
+    auto request_codes = [&](int unit) {
+      if constexpr (F::NORM) {
+        static_assert(!F::NORM || F::UC == 128);
+        const uint8_t* p = codes + unit * (F::UC / 2 >> a.norm_shift);
+        code_word = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i < (F::UC / 2 >> a.norm_shift)) code_word |= static_cast<uint32_t>(__ldg(p + i)) << (8 * i);
+      }
+    };
 
 #pragma unroll 1
     for (;;) {
@@ -793,19 +806,19 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           const Segment& sg = a.seg[segment_of(a, tile)];
           gs = sg.scale + static_cast<long long>(min((tile - sg.tile0) * kTileRows + qt, sg.N - 1)) * (a.K / 128);
         }
+        if constexpr (F::NORM) {
+          const int row = min((tile - a.seg[0].tile0) * kTileRows + qt, a.seg[0].N - 1);
+          codes = a.codes + static_cast<long long>(row) * a.code_row;
+          lut = a.lut + static_cast<long long>(row / a.Br) * a.blocks_per_row * 16;
+          request_codes(u);
+        }
       }
       uint32_t nscales[F::NORM ? F::UC / 16 : 1];   // normalisation: the scale of every 16 columns, twice
       if constexpr (F::NORM) {
-        static_assert(!F::NORM || F::UC == 128);
-        const int row = min((tile - a.seg[0].tile0) * kTileRows + qt, a.seg[0].N - 1);
-        const uint8_t* code = a.codes + static_cast<long long>(row) * a.code_row + u * (F::UC / 2 >> a.norm_shift);
-        const unsigned short* lut = a.lut + (static_cast<long long>(row / a.Br) * a.blocks_per_row + divide(u, a.block_inv)) * 16;
-        uint32_t cw = 0;   // the unit's codes
+        const unsigned short* l = lut + divide(u, a.block_inv) * 16;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (i < (F::UC / 2 >> a.norm_shift)) cw |= static_cast<uint32_t>(__ldg(code + i)) << (8 * i);
-#pragma unroll
-        for (int i = 0; i < F::UC / 16; ++i) nscales[i] = __ldg(lut + ((cw >> (4 * (16 * i >> a.norm_shift))) & 15u)) * 0x10001u;
+        for (int i = 0; i < F::UC / 16; ++i) nscales[i] = __ldg(l + ((code_word >> (4 * (16 * i >> a.norm_shift))) & 15u)) * 0x10001u;
+        if (seg_left > 1) request_codes(u + 1);
       }
       uint32_t scales[F::STAGES / 2];   // int4 codebooks: of the unit's groups of 128 columns
       if constexpr (F::I4) {
@@ -1174,6 +1187,13 @@ vq_status launch_gemm_tile_norm(const Geometry& g, const LayerPtrs& p, const voi
                                 const __half* X, __half* Y, int batch, cudaStream_t s) {
   if (!norm_codes || !norm_lut || !tile_covers(g) || g.d != 2 || g.b != 6 || g.cb_int4) return VQ_ERR_UNSUPPORTED;
   if (norm_block_cols != 16 && norm_block_cols != 32 && norm_block_cols != 64) return VQ_ERR_UNSUPPORTED;
+  // A tile is one CTA's whole: worth it where the tiles fill the SMs.  0.1 ns, fitted to both kernels' times: a round of tiles against
+  // the pair-table kernel's weights (sub-rows of 32, batch 1: 14336 x 4096 18.0 us against 23.6, 11008 x 4096 17.0/19.3, 8192 x 1024
+  // 4.0/7.7; 4096 x 4096 14.5/9.6, 19200 x 2048 15.2/17.5, which this leaves to the other; of 16, batch 4: 11008 x 4096 22.2/21.5).
+  int sms = 0;
+  if (device_sms(&sms) != VQ_OK) return VQ_ERR_CUDA;
+  const long long rounds = ((g.N + kTileRows - 1) / kTileRows + sms - 1) / sms, w = (static_cast<long long>(g.N) * g.K) >> 20;
+  if (35000 + rounds * g.K * (norm_block_cols == 16 ? 47 : 35) > 50000 + 3100 * w) return VQ_ERR_UNSUPPORTED;
   StreamCall call = {};
   call.g = g;
   call.n_seg = 1;

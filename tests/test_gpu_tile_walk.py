@@ -1,0 +1,94 @@
+"""The tcgen05 kernel's walk: pieces of tiles that meet in the workspace, whole tiles beside them, units that do not divide among
+the four groups of decoding warps; row tables below batch 9; block-wise normalisation."""
+import numpy as np
+import pytest
+
+import vq_synth
+from oracle import vq_oracle as orc
+from tests.helpers import DeviceLayer, assert_outputs_close, draw, guarded, assert_guards_intact, kernels_launched, oracle_fmt
+
+vq = pytest.importorskip("paper_2402_15319_b200")
+pytestmark = pytest.mark.gpu
+
+
+def _spec(name, N, K, d, b, Br, Bc, cb):
+    return vq_synth.LayerSpec(name, N=N, K=K, d=d, b=b, Br=Br, Bc=Bc, int8=cb)
+
+
+def _rows(N):
+    edge = [r for t in (0, 128, N // 128 * 128, N) for r in range(t - 12, t + 12) if 0 <= r < N]
+    return np.unique(np.concatenate([edge, np.random.default_rng(5).integers(0, N, 64)])).astype(np.int32)
+
+
+@pytest.mark.parametrize("spec,batches", [
+    # one CTA per tile, several pieces a tile of equal length, pieces that cross tiles (148 CTAs)
+    (_spec("equal_pieces", 4096, 4096, 2, 6, 128, 128, False), (1, 9)),
+    (_spec("crossing", 5120, 5120, 4, 8, 256, 512, False), (8, 16)),
+    (_spec("crossing_i4", 3328, 9088, 2, 6, 32, 128, 2), (5, 13)),
+    # 1, 2, 3, 5 units: some groups of warps have none
+    (_spec("units1", 256, 128, 2, 6, 128, 128, True), (1, 16)),
+    (_spec("units3", 384, 384, 2, 6, 32, 128, False), (4, 12)),
+    (_spec("units5", 200, 1280, 2, 5, 4, 256, True), (3, 9)),
+    # whole tiles and a left-over tile shared by eight CTAs, by one
+    (_spec("whole_and_shared", 149 * 128, 2048, 2, 6, 128, 128, False), (2, 16)),
+    (_spec("whole_only", 296 * 128, 512, 2, 4, 1, 512, True), (11,)),
+], ids=lambda v: v.name if hasattr(v, "name") else None)
+def test_pieces(spec, batches):
+    L = draw(spec, 91)
+    dev = DeviceLayer(spec, L)
+    rows = _rows(spec.N)
+    for batch in batches:
+        X = vq_synth.make_x(spec, 92, batch)
+        Y, A = orc.gemm(oracle_fmt(spec), L.idx, L.cb, L.scale, X, rows=rows, threads=8)
+        first = dev.gemm(X, vq.VQ_IMPL_TILE)
+        assert_outputs_close(first[:, rows], Y, A, f"{spec.name} batch {batch}")
+        for _ in range(3):
+            assert np.array_equal(dev.gemm(X, vq.VQ_IMPL_TILE).view(np.uint16), first.view(np.uint16))
+    assert vq.vq_device_wait_failures() == 0
+
+
+@pytest.mark.parametrize("cb,bc", [(True, 2048), (False, 1024)])
+def test_row_tables_at_batch_8(cb, bc):
+    import torch
+    spec = _spec("rows", 57344, 4096, 2, 4, 1, bc, cb)
+    L = draw(spec, 93)
+    dev = DeviceLayer(spec, L)
+    X = vq_synth.make_x(spec, 94, 8)
+    dX, Y = torch.from_numpy(X).cuda(), torch.empty((8, spec.N), dtype=torch.float16, device="cuda")
+    names = kernels_launched(lambda: vq.vq_gemm_small_batch(dev.fmt, dev.idx, dev.cb, dev.scale, dX, Y, 8, dev.ws))
+    assert len(names) == 1 and "tile_kernel" in names[0], names
+    rows = _rows(spec.N)
+    ref, A = orc.gemm(oracle_fmt(spec), L.idx, L.cb, L.scale, X, rows=rows, threads=8)
+    assert_outputs_close(dev.gemm(X)[:, rows], ref, A, spec.name)
+    assert vq.vq_device_wait_failures() == 0
+
+
+@pytest.mark.parametrize("spec", [
+    _spec("warp_i8", 13344, 4096, 2, 6, 32, 256, True),
+    _spec("warp_fp16_odd", 19072, 3328, 2, 6, 64, 128, False),
+    _spec("cta_fp16", 14336, 4096, 2, 6, 128, 128, False),
+    _spec("two_tiles_a_cta", 22016, 2048, 2, 6, 256, 256, True),
+], ids=lambda v: v.name)
+@pytest.mark.parametrize("cols", [16, 32, 64])
+def test_normalised(spec, cols):
+    import torch
+    L = draw(spec, 95)
+    dev = DeviceLayer(spec, L)
+    codes, lut = vq_synth.make_norm(spec, cols, seed=96)
+    dc, dl = torch.from_numpy(codes).cuda(), torch.from_numpy(lut).cuda()
+    for batch in (1, 8, 9, 16):
+        X = vq_synth.make_x(spec, 97, batch)
+        dX = torch.from_numpy(X).cuda()
+        dY, raw = guarded((batch, spec.N), torch.float16, "cuda")
+        torch.cuda.synchronize()
+        vq.vq_gemm_small_batch_normalized(dev.fmt, dev.idx, dev.cb, dev.scale, dc, dl, cols, dX, dY, batch)
+        torch.cuda.synchronize()
+        assert_guards_intact(raw, spec.name)
+        if batch in (1, 9):
+            W, _ = orc.normalized_decode(oracle_fmt(spec), L.idx, L.cb, L.scale, codes, lut, cols)
+            rows = _rows(spec.N)
+            Wr = W[rows].astype(np.float64)
+            ref, A = X.astype(np.float64) @ Wr.T, np.abs(X.astype(np.float64)) @ np.abs(Wr).T
+            assert_outputs_close(dY.cpu().numpy()[:, rows], ref, A, f"{spec.name} {cols} batch {batch}")
+        assert np.isfinite(dY.float().cpu().numpy()).all()
+    assert vq.vq_device_wait_failures() == 0
