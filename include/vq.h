@@ -104,8 +104,8 @@ typedef enum {
   VQ_IMPL_STREAM = 3,   /* the persistent tuned kernel only (the one AUTO picks for large per-row 4-bit
                            layers and for groups at small batch); VQ_ERR_UNSUPPORTED if it does not cover
                            the format */
-  VQ_IMPL_TILE = 4      /* the tcgen05 kernel only (the one AUTO and TUNED pick for large layers and
-                           batches); VQ_ERR_UNSUPPORTED if it does not cover the format and batch */
+  VQ_IMPL_TILE = 4      /* the tcgen05 kernel only (the one AUTO and TUNED pick for most calls of its
+                           formats); VQ_ERR_UNSUPPORTED if it does not cover the format and batch */
 } vq_impl;
 
 /* Caller-filled description of one VQ-compressed matrix (paper Sec. 2.1 notation in comments). */

@@ -1117,7 +1117,7 @@ vq_status launch(const StreamCall& call, cudaStream_t s, const Norm* norm = null
 
 }  // namespace
 
-// Codebook blocks that are whole units of columns (so K is one too).  (Row tables: from batch 9 on only, see launch_gemm_tile.)
+// Codebook blocks that are whole units of columns (so K is one too).
 bool tile_covers(const Geometry& g) {
   if (g.d == 2 && g.b == 4) return !g.cb_int4 && g.Bc % 256 == 0;
   if (g.d == 2 && g.b == 5) return g.Bc % 256 == 0 && (g.Br % 32 == 0 || (!g.cb_int4 && (g.Br == 4 || g.Br == 8 || g.Br == 16)));
@@ -1135,7 +1135,7 @@ bool tile_covers(const Geometry& g) {
 //   others, K >= 5500: 0.45 to 0.85 at every size.  K from 3700: batch 1 to 5 from 24: 0.75, below 0.93 (1.1); 32-row blocks of 6 bits from
 //                64: 0.82, from 24 1.06; batch 6 to 16 from 8: 0.8.  K below: from 24 0.8, from 8 1.0; from batch 9 on from 8: 0.78
 //   groups whose layers the cluster kernels take in one launch: 12288 x 4096 in three layers, 128-row blocks, 6 bits, batch 1 12.7 us
-//                against 10.8, 6144 x 4096 32-row blocks 9.3/8.3, 15360 x 5120 4-D batch 8 16.4/18.3: from 64
+//                against 10.8, 6144 x 4096 32-row blocks 9.3/8.3; 18176 x 3328 4-bit codebooks batch 5 15.7/19.1, 15360 x 5120 4-D batch 8 16.4/18.3: from 54
 // Slower than the others remain calls with many short rows at large batches, where adding a tile's sums takes as long as decoding
 // it: 65536 x 1024 at batch 16 1.2 times, 32768 x 2048 1.1 times the time of a kernel of four CTAs per SM that this one replaced.
 bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
@@ -1157,7 +1157,7 @@ bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
   if (g.K >= 5500) return true;
   const bool pairs = g.b == 5 && g.Br < 32;   // else: the pair-table kernel, which takes groups too
   if (!pairs && !whole) return g.K >= 3700 || w >= (n_seg > 1 ? 4 : 16);
-  if (!pairs && n_seg > 1 && batch <= 8) return w >= 64;
+  if (!pairs && n_seg > 1 && batch <= 8) return w >= 54;
   if (g.K < 3700) return w >= (batch <= 8 || pairs ? 24 : 8);
   if (pairs) return w >= 12;
   if (batch >= 6) return w >= (batch <= 8 && g.b == 6 && g.Br % kTileRows != 0 ? 48 : 8);
