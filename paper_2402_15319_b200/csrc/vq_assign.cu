@@ -18,6 +18,9 @@
 // (for large or one-dimensional codebooks the two best) and the best score outside.  If that one is further from the best than
 // both forms' rounding errors can account for (the gap, below), the winner lies in the group or groups kept and the exact
 // sequence runs over their centroids; else over all of them.
+// Weights belong to columns: where a thread ranks the same vector of four rows of a block together, the part of the score that holds
+// no x is computed once for the four, and so are the ratios r_t.  11008 x 4096, 64 2-D entries, weighted: 378 us with four
+// neighbouring vectors of one row, 326 with four rows, 312 with the four vectors' exact sequences side by side.
 #include "vq_common.cuh"
 
 namespace vq {
@@ -187,8 +190,173 @@ __device__ __forceinline__ void load_pair(uint64_t (&c)[D], const unsigned char*
   }
 }
 
-// TOP2: the two best groups are kept, with the group's number in the low bits of its score; else the best group only.
-template <int D, bool HD, bool TOP2>
+// Indices of the winners of V vectors of one block, given to emit(vector, index).  TOP2: the two best groups are kept, with the group's number in the low bits
+// of its score; else the best group only.  COL: the vectors lie in the same columns, so that they share their weights (dw[0]) and with
+// them the part of the score that the vector does not enter, sum_t r_t c_t^2: d fused steps a vector and pair are left of 2 d - 1.
+template <int D, bool HD, bool TOP2, bool COL, int V, class Emit>
+__device__ __forceinline__ void pick(const float (&x)[V][D], const float (&dw)[COL ? 1 : V][D], const unsigned char* tab, float c_max, int groups, Emit emit) {
+  constexpr int GB = group_bytes<D>();
+  const uint64_t minus1 = pack2(-1.f, -1.f);
+  constexpr int W = COL ? 1 : V;
+  [[maybe_unused]] int bi[V];
+  // ---- rank the groups ----
+  uint64_t ca[V][D], cr[W][D];   // (-2 r_t x_t) and r_t, twice each
+  float best[V], second[V], third[V], xx[V];
+  int gi[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    float sq = 0.f;
+    if constexpr (!HD) {
+#pragma unroll
+      for (int t = 0; t < D; ++t) {
+        const float at = -2.f * x[v][t];
+        ca[v][t] = pack2(at, at);
+        sq += x[v][t] * x[v][t];
+      }
+      // infinity or NaN among the values: NaN, which makes the exact sequence run over all centroids.  (Values are multiples
+      // of 2^-24 below 2^23, so that nothing else overflows or underflows.)
+      xx[v] = sq + c_max < 1e30f ? sq : __int_as_float(0x7fc00000);
+    } else {
+      const float (&dv)[D] = dw[COL ? 0 : v];
+      float m = 0.f, base = dv[0], far = 0.f;
+      bool usable = true;
+      if (base == 0.f) {   // a first weight of zero counts as 2^-40 of the largest, and the gap takes in what that adds
+#pragma unroll
+        for (int t = 1; t < D; ++t) base = fmaxf(base, dv[t] * 0x1p-40f);
+        far = (fabsf(x[v][0]) + c_max) * (fabsf(x[v][0]) + c_max);
+      }
+#pragma unroll
+      for (int t = 0; t < D; ++t) {
+        const float rt = t > 0 ? __fdiv_rn(dv[t], base) : 1.f;
+        const float at = -2.f * rt * x[v][t], reach = fabsf(x[v][t]) + c_max;
+        ca[v][t] = pack2(at, at);
+        if (!COL || v == 0) cr[COL ? 0 : v][t] = pack2(rt, rt);
+        m += rt * reach * reach;
+        sq += rt * x[v][t] * x[v][t];
+        usable = usable && dv[t] >= 0.f;
+      }
+      // in range, so that no term overflows or underflows to where the bounds above do not hold; what single terms lose to
+      // underflow is less than the gap that 1e-30 over the weights' base adds
+      const float dm = base * m;
+      usable = usable && base > 0.f && m > 1e-30f && m < 1e30f && dm > 1e-30f && dm < 1e30f;
+      sq += 1e-30f + __fdividef(1e-30f, base) + far * (2.f / kGapBase);
+      xx[v] = usable ? sq : __int_as_float(0x7fc00000);
+    }
+    best[v] = second[v] = third[v] = __int_as_float(0x7f800000);
+    gi[v] = 0;
+  }
+  for (int g = 0; g < groups; ++g) {
+    float gm[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) gm[v] = __int_as_float(0x7f7fffff);   // (a group of NaN: finite with any number in its low bits)
+#pragma unroll
+    for (int p = 0; p < kGroup / 2; ++p) {
+      uint64_t c[D], q[D];
+      load_pair<D>(c, tab + g * GB + p * (D * 8));
+#pragma unroll
+      for (int t = 0; t < D; ++t) q[t] = mul2(c[t], c[t]);
+      if constexpr (!HD) {
+#pragma unroll
+        for (int t = 1; t < D; ++t) q[0] = add2(q[0], q[t]);
+      } else if constexpr (COL) {
+#pragma unroll
+        for (int t = 1; t < D; ++t) q[0] = fma2(cr[0][t], q[t], q[0]);
+      }
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        uint64_t sc = fma2(ca[v][0], c[0], q[0]);
+#pragma unroll
+        for (int t = 1; t < D; ++t) {
+          if constexpr (HD && !COL) sc = fma2(cr[v][t], q[t], sc);
+          sc = fma2(ca[v][t], c[t], sc);
+        }
+        float lo, hi;
+        unpack2(sc, lo, hi);
+        gm[v] = fminf(fminf(gm[v], lo), hi);
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      float k = gm[v];
+      if constexpr (TOP2) {
+        k = __int_as_float((__float_as_int(k) & ~(groups - 1)) | g);
+        third[v] = fminf(third[v], fmaxf(second[v], k));
+      } else {
+        gi[v] = k < best[v] ? g : gi[v];
+      }
+      second[v] = fminf(second[v], fmaxf(best[v], k));
+      best[v] = fminf(best[v], k);
+    }
+  }
+
+  // ---- the exact sequence over the groups that can hold the winner, in order ----
+  // pair p of group g for vector v
+  auto compare = [&](int v, int g, int p, float& bd, int& b) {
+    uint64_t c[D];
+    load_pair<D>(c, tab + g * GB + p * (D * 8));
+    float lo = 0.f, hi = 0.f;
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+      const uint64_t diff = fma2(c[t], minus1, pack2(x[v][t], x[v][t]));   // x - c, rounded once
+      uint64_t term = mul2(diff, diff);
+      const float w = HD ? dw[COL ? 0 : v][t] : 0.f;
+      if constexpr (HD) term = mul2(pack2(w, w), term);
+      float tl, th;
+      unpack2(term, tl, th);
+      // (scalar: with a packed sum the product and the sum came out as one rounding)
+      lo = t == 0 ? tl : __fadd_rn(lo, tl);
+      hi = t == 0 ? th : __fadd_rn(hi, th);
+    }
+    if (lo < bd) {
+      bd = lo;
+      b = g * kGroup + 2 * p;
+    }
+    if (hi < bd) {
+      bd = hi;
+      b = g * kGroup + 2 * p + 1;
+    }
+  };
+  const float inf = __int_as_float(0x7f800000);
+  if constexpr (!TOP2 && COL) {
+    // the best groups of all vectors together: one vector's chain of comparisons alone leaves most issue slots empty
+    float bd[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      bd[v] = inf;
+      bi[v] = 0;
+    }
+#pragma unroll
+    for (int p = 0; p < kGroup / 2; ++p)
+#pragma unroll
+      for (int v = 0; v < V; ++v) compare(v, gi[v], p, bd[v], bi[v]);
+  }
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const float limit = best[v] + (kGapBase + (TOP2 ? kGapGroup * groups : 0.f)) * (xx[v] + fmaxf(best[v] + xx[v], 0.f));
+    int g1 = gi[v], g2 = 0, count = second[v] > limit ? 1 : groups;
+    if constexpr (TOP2) {
+      g1 = __float_as_int(best[v]) & (groups - 1);
+      g2 = __float_as_int(second[v]) & (groups - 1);
+      count = second[v] > limit ? 1 : third[v] > limit ? 2 : groups;
+    }
+    if (!TOP2 && COL && count == 1) {
+      emit(v, bi[v]);
+      continue;
+    }
+    float bd = inf;
+    int b = 0;
+#pragma unroll 1
+    for (int i = 0; i < count; ++i) {
+      const int g = count == 1 ? g1 : !TOP2 || count == groups ? i : i == 0 ? min(g1, g2) : max(g1, g2);
+#pragma unroll
+      for (int p = 0; p < kGroup / 2; ++p) compare(v, g, p, bd, b);
+    }
+    emit(v, b);
+  }
+}
+
+// COL: blocks of a multiple of 4 rows; a thread takes the same vector of four rows at a time.
+template <int D, bool HD, bool TOP2, bool COL = false>
 __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_kernel(const AssignArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int GB = group_bytes<D>();
@@ -271,7 +439,50 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
   if (grp >= a.groups) return;
   const int col = grp * 8 * D;              // first column of the thread's 8 vectors
   const int lbc = (col - col0) >> a.bc_shift;   // 0 when the block is wider than the segment
-  const uint64_t minus1 = pack2(-1.f, -1.f);
+
+  if constexpr (COL) {
+    static_assert(kRows == 4 * kWarps);
+    const int r = 4 * warp;   // the warp's rows: of one block
+    if (row0 + r >= a.N) return;
+    const int tb = (r / a.rows_per_br) * a.bc_per_seg + lbc;
+    const unsigned char* tab = smem + tb * table_bytes;
+    const float c_max = __int_as_float(cmax[tb]);
+    unsigned long long bits[4] = {};
+#pragma unroll 1
+    for (int v = 0; v < 8; ++v) {
+      float x[4][D], dw[1][D];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {   // (rows of a block exist together: N is a multiple of the block rows)
+        const __half* src = a.W + static_cast<long long>(row0 + r + i) * a.K + col + v * D;
+        uint32_t wds[D / 2];
+        if constexpr (D == 2) {
+          wds[0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+        } else {
+          const uint2 raw = __ldg(reinterpret_cast<const uint2*>(src));
+          wds[0] = raw.x;
+          wds[D / 2 - 1] = raw.y;
+        }
+#pragma unroll
+        for (int t = 0; t < D; ++t) {
+          const __half_raw hr = {static_cast<unsigned short>((wds[t >> 1] >> (16 * (t & 1))) & 0xffff)};
+          x[i][t] = __half2float(__half(hr));
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < D; ++t) dw[0][t] = __ldg(a.hdiag + col + v * D + t);
+      pick<D, HD, TOP2, true, 4>(x, dw, tab, c_max, groups,
+                                 [&](int i, int index) { bits[i] |= static_cast<unsigned long long>(index) << (v * a.b); });
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int n = row0 + r + i;
+      uint8_t* dst = a.idx + n * a.stride + static_cast<long long>(grp) * a.b;
+      for (int k = 0; k < a.b; ++k) dst[k] = static_cast<uint8_t>(bits[i] >> (8 * k));
+      if (grp == a.groups - 1)   // padding up to the row stride
+        for (long long k = a.used_bytes; k < a.stride; ++k) a.idx[n * a.stride + k] = 0;
+    }
+    return;
+  }
 
   for (int r = warp; r < kRows; r += kWarps) {
     const int n = row0 + r;
@@ -304,141 +515,8 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
           for (int t = 0; t < D; ++t) dw[v][t] = __ldg(a.hdiag + col + (v0 + v) * D + t);
       }
 
-      // ---- rank the groups ----
-      uint64_t ca[V][D], cr[V][D];   // (-2 r_t x_t) and r_t, twice each
-      float best[V], second[V], third[V], xx[V];
-      int gi[V];
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        float sq = 0.f;
-        if constexpr (!HD) {
-#pragma unroll
-          for (int t = 0; t < D; ++t) {
-            const float at = -2.f * x[v][t];
-            ca[v][t] = pack2(at, at);
-            sq += x[v][t] * x[v][t];
-          }
-          // infinity or NaN among the values: NaN, which makes the exact sequence run over all centroids.  (Values are multiples
-          // of 2^-24 below 2^23, so that nothing else overflows or underflows.)
-          xx[v] = sq + c_max < 1e30f ? sq : __int_as_float(0x7fc00000);
-        } else {
-          float m = 0.f, base = dw[v][0], far = 0.f;
-          bool usable = true;
-          if (base == 0.f) {   // a first weight of zero counts as 2^-40 of the largest, and the gap takes in what that adds
-#pragma unroll
-            for (int t = 1; t < D; ++t) base = fmaxf(base, dw[v][t] * 0x1p-40f);
-            far = (fabsf(x[v][0]) + c_max) * (fabsf(x[v][0]) + c_max);
-          }
-#pragma unroll
-          for (int t = 0; t < D; ++t) {
-            const float rt = t > 0 ? __fdiv_rn(dw[v][t], base) : 1.f;
-            const float at = -2.f * rt * x[v][t], reach = fabsf(x[v][t]) + c_max;
-            ca[v][t] = pack2(at, at);
-            cr[v][t] = pack2(rt, rt);
-            m += rt * reach * reach;
-            sq += rt * x[v][t] * x[v][t];
-            usable = usable && dw[v][t] >= 0.f;
-          }
-          // in range, so that no term overflows or underflows to where the bounds above do not hold; what single terms lose to
-          // underflow is less than the gap that 1e-30 over the weights' base adds
-          const float dm = base * m;
-          usable = usable && base > 0.f && m > 1e-30f && m < 1e30f && dm > 1e-30f && dm < 1e30f;
-          sq += 1e-30f + __fdividef(1e-30f, base) + far * (2.f / kGapBase);
-          xx[v] = usable ? sq : __int_as_float(0x7fc00000);
-        }
-        best[v] = second[v] = third[v] = __int_as_float(0x7f800000);
-        gi[v] = 0;
-      }
-      for (int g = 0; g < groups; ++g) {
-        float gm[V];
-#pragma unroll
-        for (int v = 0; v < V; ++v) gm[v] = __int_as_float(0x7f7fffff);   // (a group of NaN: finite with any number in its low bits)
-#pragma unroll
-        for (int p = 0; p < kGroup / 2; ++p) {
-          uint64_t c[D], q[D];
-          load_pair<D>(c, tab + g * GB + p * (D * 8));
-#pragma unroll
-          for (int t = 0; t < D; ++t) q[t] = mul2(c[t], c[t]);
-          if constexpr (!HD) {
-#pragma unroll
-            for (int t = 1; t < D; ++t) q[0] = add2(q[0], q[t]);
-          }
-#pragma unroll
-          for (int v = 0; v < V; ++v) {
-            uint64_t sc = fma2(ca[v][0], c[0], q[0]);
-#pragma unroll
-            for (int t = 1; t < D; ++t) {
-              if constexpr (HD) sc = fma2(cr[v][t], q[t], sc);
-              sc = fma2(ca[v][t], c[t], sc);
-            }
-            float lo, hi;
-            unpack2(sc, lo, hi);
-            gm[v] = fminf(fminf(gm[v], lo), hi);
-          }
-        }
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          float k = gm[v];
-          if constexpr (TOP2) {
-            k = __int_as_float((__float_as_int(k) & ~(groups - 1)) | g);
-            third[v] = fminf(third[v], fmaxf(second[v], k));
-          } else {
-            gi[v] = k < best[v] ? g : gi[v];
-          }
-          second[v] = fminf(second[v], fmaxf(best[v], k));
-          best[v] = fminf(best[v], k);
-        }
-      }
-
-      // ---- the exact sequence over the groups that can hold the winner, in order ----
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        const float limit = best[v] + (kGapBase + (TOP2 ? kGapGroup * groups : 0.f)) * (xx[v] + fmaxf(best[v] + xx[v], 0.f));
-        int g1 = gi[v], g2 = 0, count = second[v] > limit ? 1 : groups;
-        if constexpr (TOP2) {
-          g1 = __float_as_int(best[v]) & (groups - 1);
-          g2 = __float_as_int(second[v]) & (groups - 1);
-          count = second[v] > limit ? 1 : third[v] > limit ? 2 : groups;
-        }
-        uint64_t x2[D], d2[D];
-#pragma unroll
-        for (int t = 0; t < D; ++t) {
-          x2[t] = pack2(x[v][t], x[v][t]);
-          if constexpr (HD) d2[t] = pack2(dw[v][t], dw[v][t]);
-        }
-        float bd = __int_as_float(0x7f800000);   // +inf
-        int bi = 0;
-#pragma unroll 1
-        for (int i = 0; i < count; ++i) {
-          const int g = count == 1 ? g1 : !TOP2 || count == groups ? i : i == 0 ? min(g1, g2) : max(g1, g2);
-#pragma unroll
-          for (int p = 0; p < kGroup / 2; ++p) {
-            uint64_t c[D];
-            load_pair<D>(c, tab + g * GB + p * (D * 8));
-            float lo = 0.f, hi = 0.f;
-#pragma unroll
-            for (int t = 0; t < D; ++t) {
-              const uint64_t diff = fma2(c[t], minus1, x2[t]);   // x - c, rounded once
-              uint64_t term = mul2(diff, diff);
-              if constexpr (HD) term = mul2(d2[t], term);
-              float tl, th;
-              unpack2(term, tl, th);
-              // (scalar: with a packed sum the product and the sum came out as one rounding)
-              lo = t == 0 ? tl : __fadd_rn(lo, tl);
-              hi = t == 0 ? th : __fadd_rn(hi, th);
-            }
-            if (lo < bd) {
-              bd = lo;
-              bi = g * kGroup + 2 * p;
-            }
-            if (hi < bd) {
-              bd = hi;
-              bi = g * kGroup + 2 * p + 1;
-            }
-          }
-        }
-        bits |= static_cast<unsigned long long>(bi) << ((v0 + v) * a.b);
-      }
+      pick<D, HD, TOP2, false, V>(x, dw, tab, c_max, groups,
+                                  [&](int v, int index) { bits |= static_cast<unsigned long long>(index) << ((v0 + v) * a.b); });
     }
     uint8_t* dst = a.idx + n * a.stride + static_cast<long long>(grp) * a.b;
     for (int i = 0; i < a.b; ++i) dst[i] = static_cast<uint8_t>(bits >> (8 * i));
@@ -483,7 +561,7 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
   const size_t smem = static_cast<size_t>(a.br_per_tile) * a.bc_per_seg * g.entries * g.d * sizeof(float);
   if (smem > 96 * 1024) return VQ_ERR_UNSUPPORTED;
   const dim3 grid((a.groups + 31) / 32, (g.N + kRows - 1) / kRows, 1);
-  static int attr_set[kMaxDevices][13] = {};
+  static int attr_set[kMaxDevices][17] = {};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return VQ_ERR_CUDA;
   auto launch = [&](auto kern, int slot, size_t smem) {
@@ -508,6 +586,12 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
   if (two && smem2 <= 96 * 1024) {
     const bool top2 = g.entries >= 128;
     if (g.d == 1) return hdiag ? launch(assign_two_pass_kernel<1, true, true>, 3, smem2) : launch(assign_two_pass_kernel<1, false, true>, 4, smem2);
+    // The same columns of four rows share their weights (one row at a time / four, 4096 x 4096, us: 32 2-D entries 106/87, 64 2-D 144/120,
+    // 256 2-D 413/352, 64 4-D 183/131, 256 4-D 463/359); blocks of one or two rows do not hold four rows.
+    if (hdiag && g.Br % 4 == 0 && g.d != 1) {
+      if (g.d == 2) return top2 ? launch(assign_two_pass_kernel<2, true, true, true>, 13, smem2) : launch(assign_two_pass_kernel<2, true, false, true>, 14, smem2);
+      return top2 ? launch(assign_two_pass_kernel<4, true, true, true>, 15, smem2) : launch(assign_two_pass_kernel<4, true, false, true>, 16, smem2);
+    }
     if (g.d == 2 && top2) return hdiag ? launch(assign_two_pass_kernel<2, true, true>, 5, smem2) : launch(assign_two_pass_kernel<2, false, true>, 6, smem2);
     if (g.d == 2) return hdiag ? launch(assign_two_pass_kernel<2, true, false>, 7, smem2) : launch(assign_two_pass_kernel<2, false, false>, 8, smem2);
     if (top2) return hdiag ? launch(assign_two_pass_kernel<4, true, true>, 9, smem2) : launch(assign_two_pass_kernel<4, false, true>, 10, smem2);
