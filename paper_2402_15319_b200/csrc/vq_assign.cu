@@ -317,7 +317,7 @@ __device__ __forceinline__ void pick(const float (&x)[V][D], const float (&dw)[C
     }
   };
   const float inf = __int_as_float(0x7f800000);
-  if constexpr (!TOP2 && COL) {
+  if constexpr (!TOP2) {
     // the best groups of all vectors together: one vector's chain of comparisons alone leaves most issue slots empty
     float bd[V];
 #pragma unroll
@@ -339,7 +339,7 @@ __device__ __forceinline__ void pick(const float (&x)[V][D], const float (&dw)[C
       g2 = __float_as_int(second[v]) & (groups - 1);
       count = second[v] > limit ? 1 : third[v] > limit ? 2 : groups;
     }
-    if (!TOP2 && COL && count == 1) {
+    if (!TOP2 && count == 1) {
       emit(v, bi[v]);
       continue;
     }
