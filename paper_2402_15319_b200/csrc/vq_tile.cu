@@ -19,12 +19,12 @@
 // contiguous pieces, one per CTA, walked first, so that shared tiles are summed while everyone still computes whole
 // ones.  (With four CTAs of one quad each per SM a tile was shared by four times as many CTAs, whose sums met in the workspace.)
 //
-// Roles (672 threads).  Warps 0..15 decode, four to a quad: thread = weight row = lane of tensor memory.  A thread reads its
+// Roles (672 threads with row tables, else 768).  Warps 0..15 decode, four to a quad: thread = weight row = lane of tensor memory.  A thread reads its
 // row's indices of a unit from the stage the copy engine filled, looks up 32 pairs (64 columns) and stores them as
 // 32 columns of tensor memory, of which the quad has two such stages.  Warps 16..19 serve a quad each: they request its index and
 // activation boxes by TMA (index boxes run ahead of the programmatic-dependency wait, activations come after it) and issue its
 // products (one elected lane, warp-uniform control flow: with a divergent branch in place of elect.sync an issue took
-// five times as long).  Warp 20 owns the tensor memory, adds the quads' sums and stores outputs or shares of them.
+// five times as long).  Warp 20 owns the tensor memory; it, or warps 20..23, add the quads' sums and store outputs or shares of them.
 //
 // Tables.  One 32-bit word per entry and lane, bank = lane: no conflicts whatever the indices.  Three kinds:
 //   row  : 16 entries of the lane's own row; two warps' tables alternate (256-byte entry pitch), so that the index byte
@@ -35,10 +35,15 @@
 // scale; the other tables hold fp16(scale * c), the value vq_decode_weights writes.  4-bit codebooks multiply
 // the looked-up pair by the scale of the row and its group of 128 columns, the same value again.
 //
-// Sums.  Each quad accumulates into its own columns of tensor memory and hands its sums over through shared memory, where the
-// results warp adds them in quad order.  A tile whose steps all belong to one CTA is rounded to fp16 and stored.  A shared
+// Sums.  Each quad accumulates into its own columns of tensor memory, of which it has two sets.  Four results warps (thread = weight
+// row) read a fragment's sums there, add them in quad order and give the columns back, so that the decoding warps never touch a sum.  With row
+// tables, whose sums are scaled block by block, the decoding warps scale and add them in shared memory and one results warp adds
+// the quads'.  (So did every format once: in pieces of 4 or 8 columns where tables leave no room for 16, the decoding warps
+// waiting in between, and one warp adding eight shares of a tile a column at a time.  Batch 16: 131072 x 1024, 6 bits, 32-row
+// blocks 47.9 -> 31.0 us, 19712 x 5120, 128-row blocks 33.5 -> 22.7, 4-D 33.0 -> 20.9; four CTAs of one quad per SM, this kernel's
+// predecessor, 32.8, 26.5, 23.8.)  A tile whose steps all belong to one CTA is rounded to fp16 and stored.  A shared
 // tile's parts go to the workspace; the CTA that draws the tile's last ticket adds them in CTA order when it has done its own
-// work (results do not depend on timing) and resets the counter.
+// work, or beside its whole tiles (results do not depend on timing), and resets the counter.
 //
 // Every wait on a barrier is bounded; a wait that runs out increments a device counter, the role stops waiting for anything
 // else and still arrives on every barrier it owes, so that the kernel ends.
@@ -58,7 +63,7 @@ using namespace dev;
 constexpr int kTileRows = 128;
 constexpr int kStageCols = 64;        // columns a thread decodes between two hand-overs to the tensor core
 constexpr int kQuads = 4;             // groups of four decoding warps
-constexpr int kDecodeWarps = 4 * kQuads, kResultsWarp = kDecodeWarps + kQuads, kThreads = 32 * (kResultsWarp + 1);
+constexpr int kDecodeWarps = 4 * kQuads, kResultsWarp = kDecodeWarps + kQuads;   // (the first of the results warps)
 constexpr int kAStages = 2;           // decoded stages of a quad in tensor memory, 32 columns each
 constexpr int kTmemCols = 512;        // per quad 2 x 16 accumulator columns, then per quad 2 x 32 weight columns
 constexpr int kAOff = 32 * kQuads;
@@ -124,6 +129,10 @@ struct Fmt {
   static constexpr int TABLES = TK == kRow ? kDecodeWarps / 2 * TABLE : TK == kWarp ? kDecodeWarps * TABLE : kQuads * BUFS * TABLE;
   // OR-merged addresses need tables on multiples of their size; 4-D look-ups add (one per four weights)
   static constexpr int ALIGN = D == 4 ? 1024 : TABLE;
+  // Results warps: four read the accumulators themselves; for row tables, whose sums are scaled per block, the decoding warps read
+  // them and one warp adds the quads'.
+  static constexpr int RW = TK == kRow ? 1 : 4;
+  static constexpr int THREADS = 32 * (kResultsWarp + RW);
   static constexpr int SWIZZLE = RB == 32 ? 3 : RB == 64 ? 1 : RB == 128 ? 2 : 0;
   static_assert(RB % 16 == 0 && (TK != kRow || (B == 4 && D == 2)));
 };
@@ -149,6 +158,7 @@ __device__ __forceinline__ void wait_phase(uint32_t bar, uint32_t parity, int& t
       break;
     }
 }
+__device__ __forceinline__ void results_barrier() { asm volatile("bar.sync 5, 128;" ::: "memory"); }
 __device__ __forceinline__ void quad_barrier(int quad) { asm volatile("bar.sync %0, 128;" ::"r"(1 + quad) : "memory"); }
 __device__ __forceinline__ void tma_box_3d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, uint32_t bar) {
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
@@ -187,18 +197,25 @@ __device__ __forceinline__ void tc_store32(uint32_t addr, const uint32_t (&r)[32
       : "memory");
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tc_load4(uint32_t addr, float (&v)[4]) {   // four accumulator columns of the thread's row
-  uint32_t r[4];
+// four accumulator columns of the thread's row, to be used behind tc_load_wait()
+__device__ __forceinline__ void tc_load4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void tc_load_wait(uint32_t (&r)[N][4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    asm volatile("" : "+r"(r[i]));   // used behind the wait only
-    v[i] = __uint_as_float(r[i]);
-  }
+  for (int k = 0; k < N; ++k)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) asm volatile("" : "+r"(r[k][i]));   // used behind the wait only
 }
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t lds32_now(uint32_t addr) {   // (not moved across barriers)
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
 }
 __device__ __forceinline__ float lds32f(uint32_t addr) {
   float v;
@@ -458,7 +475,7 @@ __device__ __forceinline__ void gather(uint32_t (&r)[32], const uint32_t (&w)[F:
 }
 
 template <class F>
-__global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant__ TileMaps maps, const TileArgs a) {
+__global__ void __launch_bounds__(F::THREADS, 1) tile_kernel(const __grid_constant__ TileMaps maps, const TileArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -478,10 +495,11 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   const bool by_block = kExact && a.cb_int8;
   const int block_units = a.Bc / F::UC;
   const int quad = warp < kDecodeWarps ? warp >> 2 : warp & 3;
-  // barriers of a quad: indices and activations of a unit, decoded stages full and consumed, sums ready; then the CTA's
-  const uint32_t bars = base + a.bar_off, qb = bars + quad * 112;
-  const uint32_t idx_full = qb, x_full = qb + 32, a_full = qb + 64, a_empty = qb + 80, d_full = qb + 96;
-  const uint32_t red_full = bars + 448, red_empty = red_full + 8, tmem_slot = red_full + 16, n_last = tmem_slot + 4, last_tile = n_last + 12;
+  // barriers of a quad: indices and activations of a unit, decoded stages full and consumed, sums ready and read; then the CTA's
+  constexpr int kQuadBars = 128;
+  const uint32_t bars = base + a.bar_off, qb = bars + quad * kQuadBars;
+  const uint32_t idx_full = qb, x_full = qb + 32, a_full = qb + 64, a_empty = qb + 80, d_full = qb + 96, d_empty = qb + 112;
+  const uint32_t red_full = bars + kQuads * kQuadBars, red_empty = red_full + 8, tmem_slot = red_full + 16, n_last = tmem_slot + 4, ticket_word = n_last + 4, last_tile = n_last + 12;
   const uint32_t idx_at = base + a.idx_off + quad * D * F::IDX_BYTES, x_at = base + quad * D * a.x_bytes;
   const bool service = warp >= kDecodeWarps && warp < kResultsWarp;
 
@@ -530,6 +548,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         mbar_init(a_full + 8 * i, 4);
         mbar_init(a_empty + 8 * i, 1);
         mbar_init(d_full + 8 * i, 1);
+        mbar_init(d_empty + 8 * i, F::RW);
       }
       mbar_init_fence();
     }
@@ -552,8 +571,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   // The next kernel's CTAs may come as soon as this one's leave: a CTA of this kernel fills an SM, so that they take no slot
   // beside it, and their indices arrive while the last sums of this call are added.
   if (tid == 0) pdl_launch_dependents();
-  uint32_t tmem;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(tmem_slot) : "memory");
+  const uint32_t tmem = lds32_now(tmem_slot);
 
   if (service) {
     // ---- service: a quad's copies and products ---------------------------------------------------------------
@@ -579,7 +597,10 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         for (; f.valid && u == end; f.next(a)) f.range(a, quad, u, end);
         if (u == end) break;
       }
-      if (seg_left == 0) seg_left = (by_block ? min(end, (divide(u, a.block_inv) + 1) * block_units) : end) - u;
+      if (seg_left == 0) {
+        seg_left = (by_block ? min(end, (divide(u, a.block_inv) + 1) * block_units) : end) - u;
+        if (F::RW > 1) wait_phase(d_empty + 8 * (seg & 1), ((seg >> 1) & 1) ^ 1, tries);   // the sum but one before is read
+      }
       wait_phase(x_full + 8 * slot, ph, tries);
 #pragma unroll
       for (int j = 0; j < F::STAGES; ++j) {
@@ -622,8 +643,109 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
       ++u;
     }
     if (tries == 0) __nanosleep(1000000);   // gave up: let this CTA's own copies land before its shared memory goes away
-  } else if (warp == kResultsWarp) {
-    // ---- results: adds the quads' sums of a fragment, stores the outputs or this CTA's share of them --------------
+  } else if (warp >= kResultsWarp && F::RW > 1) {
+    // ---- results: four warps add the quads' accumulators of a fragment (thread = row), store the outputs or this CTA's share --------
+    pdl_wait();   // outputs and workspace belong to earlier kernels of the stream until here
+    const int first_tile = f.tile;   // (of the CTA's piece, if it has one)
+    const int r = tid & 127, part_floats = a.batch * kTileRows;
+    const uint32_t lane_at = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    uint32_t segs = 0;   // per quad, a byte: its sums so far
+    int listed = 0;
+#pragma unroll 1
+    for (; f.valid; f.next(a)) {
+      const Segment& sg = a.seg[segment_of(a, f.tile)];
+      const int row = (f.tile - sg.tile0) * kTileRows + r, units = min(kQuads * f.s1, a.S) - kQuads * f.s0;
+      const bool complete = f.complete(a);
+      uint32_t has = 0;   // quads that have units of the fragment: a one in the byte
+#pragma unroll
+      for (int k = 0; k < kQuads; ++k)
+        if (units * k / kQuads < units * (k + 1) / kQuads) has |= 1u << (8 * k);
+#pragma unroll 1
+      for (int k = 0; k < kQuads; ++k)
+        if ((has >> (8 * k)) & 1) wait_phase(bars + k * kQuadBars + 96 + 8 * ((segs >> (8 * k)) & 1), (segs >> (8 * k + 1)) & 1, tries);
+      __syncwarp();
+      tc_fence_after();
+      // this CTA's share of a left-over tile: slot 0 if its piece begins inside the tile, else slot 1
+      float* part = a.ws_part + static_cast<long long>(c * 2 + (f.tile == first_tile ? 0 : 1)) * part_floats + r;
+      __half* y = sg.Y + row;
+#pragma unroll 1
+      for (int n0 = 0; n0 < a.batch; n0 += 4) {
+        uint32_t v[kQuads][4];
+#pragma unroll
+        for (int k = 0; k < kQuads; ++k) tc_load4(lane_at + k * 32 + ((segs >> (8 * k)) & 1) * 16 + n0, v[k]);
+        tc_load_wait(v);
+        float s[4] = {};
+#pragma unroll
+        for (int k = 0; k < kQuads; ++k)
+          if ((has >> (8 * k)) & 1)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[i] += __uint_as_float(v[k][i]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (n0 + i < a.batch) {
+            if (!complete) part[(n0 + i) * kTileRows] = s[i];
+            else if (row < sg.N) y[static_cast<long long>(n0 + i) * sg.N] = __float2half_rn(s[i]);
+          }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane < kQuads && ((has >> (8 * lane)) & 1)) mbar_arrive(bars + lane * kQuadBars + 112 + 8 * ((segs >> (8 * lane)) & 1));
+      segs = (segs + has) & 0x03030303u;
+      if (!complete) {
+        const int first_s = (f.tile - a.tail_tile0) * a.steps, owner = step_owner(a, first_s);
+        const int shares = step_owner(a, first_s + a.steps - 1) - owner + 1;   // CTAs that share the tile
+        // where the first of them keeps its share: in its second slot unless its piece begins with the tile
+        const int c_first = 2 * owner + (first_step(a, owner) == first_s ? 0 : 1);
+        __threadfence();   // this thread's sums are visible to the GPU before the ticket is drawn
+        results_barrier();
+        if (tid == 32 * kResultsWarp) {
+          const int ticket = atomicAdd(a.ws_ticket + f.tile, 1);
+          if (ticket == shares - 1) a.ws_ticket[f.tile] = 0;   // nobody else touches the counter in this call
+          sts32(ticket_word, ticket == shares - 1);
+        }
+        results_barrier();
+        if (lds32_now(ticket_word)) {   // every share of the tile is there
+          if (a.q == 0) {           // this CTA adds them when it has done its own work, by all its threads
+            if (tid == 32 * kResultsWarp) sts128(last_tile + 16 * listed, make_uint4(segment_of(a, f.tile), row - r, c_first, shares));
+            ++listed;
+          } else {                  // whole tiles are still to come: these warps add them meanwhile
+            __threadfence();
+            const float* p = a.ws_part + static_cast<long long>(c_first) * part_floats + r;
+            const int others = (c_first & 1 ? -1 : 0) * part_floats;   // (behind the first: in their first slots)
+#pragma unroll 1
+            for (int n0 = 0; n0 < a.batch; n0 += 2) {
+              float s[2] = {};
+#pragma unroll 1
+              for (int k0 = 0; k0 < shares; k0 += 8) {   // (a load takes about 1000 clocks: sixteen at a time)
+                float v[8][2];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+#pragma unroll
+                  for (int i = 0; i < 2; ++i) {
+                    v[k][i] = 0.f;
+                    if (k0 + k < shares && n0 + i < a.batch)
+                      v[k][i] = __ldcg(p + (2 * (k0 + k)) * part_floats + (k0 + k ? others : 0) + (n0 + i) * kTileRows);
+                  }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                  s[0] += v[k][0];
+                  s[1] += v[k][1];
+                }
+              }
+#pragma unroll
+              for (int i = 0; i < 2; ++i)
+                if (row < sg.N && n0 + i < a.batch) y[static_cast<long long>(n0 + i) * sg.N] = __float2half_rn(s[i]);
+            }
+          }
+        }
+      }
+    }
+    if (tid == 32 * kResultsWarp && listed) {
+      sts32(n_last, listed);
+      __threadfence();   // the tickets before the shares are read
+    }
+  } else if (warp >= kResultsWarp) {
+    // ---- results, row tables: one warp adds the quads' sums of a fragment, stores the outputs or this CTA's share of them --------
     pdl_wait();   // outputs and workspace belong to earlier kernels of the stream until here
     const int first_tile = f.tile;   // (of the CTA's piece, if it has one)
     uint32_t ph = 0;
@@ -642,28 +764,25 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         // where the first of them keeps its share: in its second slot unless its piece begins with the tile
         c_first = 2 * c_first + (first_step(a, c_first) == first_s ? 0 : 1);
       }
-      for (int n0 = 0; n0 < a.batch; n0 += red_cols) {
-        wait_phase(red_full, ph, tries);
-        __syncwarp();
-        const int cols = min(red_cols, a.batch - n0);
+      wait_phase(red_full, ph, tries);
+      __syncwarp();
 #pragma unroll 2
-        for (int n = 0; n < cols; ++n) {
-          float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int n = 0; n < a.batch; ++n) {
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-          for (int k = 0; k < kQuads; ++k) {
-            const uint4 v = lds128(base + a.red_off + ((k * red_cols + n) * kTileRows + 4 * lane) * 4);
-            s.x += __uint_as_float(v.x); s.y += __uint_as_float(v.y); s.z += __uint_as_float(v.z); s.w += __uint_as_float(v.w);
-          }
-          if (!complete) {
-            *reinterpret_cast<float4*>(part + (n0 + n) * kTileRows) = s;
-          } else {
-            store_rows(sg, row, n0 + n, s);
-          }
+        for (int k = 0; k < kQuads; ++k) {
+          const uint4 v = lds128(base + a.red_off + ((k * red_cols + n) * kTileRows + 4 * lane) * 4);
+          s.x += __uint_as_float(v.x); s.y += __uint_as_float(v.y); s.z += __uint_as_float(v.z); s.w += __uint_as_float(v.w);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(red_empty);
-        ph ^= 1u;
+        if (!complete) {
+          *reinterpret_cast<float4*>(part + n * kTileRows) = s;
+        } else {
+          store_rows(sg, row, n, s);
+        }
       }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(red_empty);
+      ph ^= 1u;
       if (!complete) {
         __threadfence();   // this lane's sums are visible to the GPU before the ticket is drawn
         __syncwarp();
@@ -743,7 +862,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
 
 #pragma unroll 1
     for (;;) {
-      if (st == fin_at) {
+      if (F::RW == 1 && st == fin_at) {
         // ---- read a finished sum ----
         fin_at = -1;
         const int buf = (seg - 1) & 1;
@@ -753,30 +872,24 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
           tc_fence_after();
         }
         // (columns from the batch on are not used by anyone)
+        if (first_sum) wait_phase(red_empty, ph_red, tries);
+        __syncwarp();
 #pragma unroll 1
-        for (int n0 = 0; n0 < a.batch; n0 += red_cols) {
-          if (first_sum) wait_phase(red_empty, ph_red, tries);
-          __syncwarp();
-#pragma unroll 1
-          for (int n = 0; n < red_cols; n += 4) {
-            float v[4];
-            tc_load4(tmem_d + buf * 16 + n0 + n, v);
+        for (int n = 0; n < red_cols; n += 4) {
+          uint32_t v[1][4];
+          tc_load4(tmem_d + buf * 16 + n, v[0]);
+          tc_load_wait(v);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint32_t at = red_at + (n + i) * kTileRows * 4;
-              float s = pend_zero ? 0.f : v[i];
-              if (kExact) {
-                const float before = lds32f(at);
-                s = fmaf(pend_scale, s, first_sum ? 0.f : before);
-              }
-              sts32f(at, s);
-            }
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t at = red_at + (n + i) * kTileRows * 4;
+            const float before = lds32f(at);
+            sts32f(at, fmaf(pend_scale, pend_zero ? 0.f : __uint_as_float(v[0][i]), first_sum ? 0.f : before));
           }
-          if (pend_last) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(red_full);
-            ph_red ^= 1u;
-          }
+        }
+        if (pend_last) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(red_full);
+          ph_red ^= 1u;
         }
         tc_fence_before();
         first_sum = pend_last;
@@ -786,13 +899,16 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         // ---- a sum ends (all but the first time), the next one begins ----
         if (open_sum) {
           open_sum = false;
-          pend_zero = seg_units == 0;
-          pend_scale = block_scale;
           pend_last = u == end;
-          if (!pend_zero) ++seg;
-          fin_at = st;
+          if (F::RW == 1) {
+            pend_zero = seg_units == 0;
+            pend_scale = block_scale;
+            if (!pend_zero) ++seg;
+            fin_at = st;
+          }
           if (pend_last) {   // to the next fragment
             if (!f.valid) {
+              if (F::RW > 1) break;
               more = false;
               continue;
             }
@@ -806,7 +922,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
         open_sum = true;
         seg_units = seg_left = (by_block ? min(end, (bcol + 2) * block_units) : end) - u;
         if (seg_left == 0) continue;   // nothing of the fragment is this quad's
-        if (fin_at >= 0) fin_at = st + min(F::STAGES == 2 ? 2 : 1, seg_left);
+        if (F::RW == 1 && fin_at >= 0) fin_at = st + min(F::STAGES == 2 ? 2 : 1, seg_left);
         if constexpr (F::I4) {
           const Segment& sg = a.seg[segment_of(a, tile)];
           gs = sg.scale + static_cast<long long>(min((tile - sg.tile0) * kTileRows + qt, sg.N - 1)) * (a.K / 128);
@@ -920,15 +1036,14 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const __grid_constant
   tc_fence_after();
   if (warp == kResultsWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols));
   // ---- the shared tiles whose last share came from this CTA: every share is added, in CTA order ----
-  uint32_t listed;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(listed) : "r"(n_last) : "memory");
+  const uint32_t listed = lds32_now(n_last);
   for (uint32_t i = 0; i < listed; ++i) {
     const uint4 sum = lds128(last_tile + 16 * i);
     const Segment& sg = a.seg[sum.x];
     const int r = tid & 127, row = sum.y + r, part_floats = a.batch * kTileRows;
     const float* p = a.ws_part + static_cast<long long>(sum.z) * part_floats + r;
     const int others = (sum.z & 1 ? -1 : 0) * part_floats;   // (the CTAs behind the first keep their shares in their first slots)
-    constexpr int G = kThreads / 128;
+    constexpr int G = F::THREADS / 128;
 #pragma unroll 1
     for (int n = tid >> 7; n < a.batch && tid < G * 128; n += 2 * G) {
       float s[2] = {};
@@ -1026,10 +1141,8 @@ vq_status launch(const StreamCall& call, cudaStream_t s, const Norm* norm = null
     // (dynamic shared memory starts 1024 bytes into the window)
     return round_up(1024 + a.front_bytes, F::ALIGN) - 1024 + F::TABLES;
   };
-  // columns of sums handed over at a time: all of them (a second time waits for the first) unless the tables leave no room
-  a.red_cols = (call.batch + 3) / 4 * 4;
-  if (!(F::TK == kRow))
-    while (a.red_cols > 4 && plan(2) > kSmemCap) a.red_cols = a.red_cols > 8 ? 8 : 4;
+  // row tables: columns of sums handed over in shared memory
+  a.red_cols = F::RW == 1 ? (call.batch + 3) / 4 * 4 : 0;
   int D = env_int("VQ_TD", kMaxDepth);
   while (D > 2 && plan(D) > kSmemCap) --D;
   size_t smem_bytes = plan(D);
@@ -1105,7 +1218,7 @@ vq_status launch(const StreamCall& call, cudaStream_t s, const Norm* norm = null
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(P), 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.blockDim = dim3(F::THREADS, 1, 1);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

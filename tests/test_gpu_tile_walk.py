@@ -47,6 +47,30 @@ def test_pieces(spec, batches):
     assert vq.vq_device_wait_failures() == 0
 
 
+@pytest.mark.parametrize("spec,batches", [
+    # sums of many short tiles, read while the next ones are multiplied: 1, 2, 3 and 4 units a tile (quads without any), 3 or 4 tiles a CTA
+    (_spec("units1", 444 * 128 - 32, 128, 2, 6, 32, 128, 2), (1, 16)),
+    (_spec("units2", 500 * 128, 256, 2, 6, 128, 128, True), (7, 16)),
+    (_spec("units3", 450 * 128 - 96, 384, 2, 6, 32, 128, False), (4, 13)),
+    (_spec("units4_4d", 444 * 128, 512, 4, 8, 128, 128, False), (9, 16)),
+    (_spec("units2_5b", 592 * 128 - 4, 512, 2, 5, 4, 256, True), (5, 12)),
+    # a tile and a quarter per CTA: pieces that cross left-over tiles, whose shares are added beside the whole ones
+    (_spec("crossing_beside", 185 * 128, 2816, 2, 6, 128, 128, True), (3, 16)),
+    (_spec("crossing_beside_w", 185 * 128 - 64, 2816, 2, 6, 32, 256, False), (1, 10)),
+], ids=lambda v: v.name if hasattr(v, "name") else None)
+def test_sums_of_every_tile(spec, batches):
+    L = draw(spec, 98)
+    dev = DeviceLayer(spec, L)
+    for batch in batches:
+        X = vq_synth.make_x(spec, 99, batch)
+        Y, A = orc.gemm(oracle_fmt(spec), L.idx, L.cb, L.scale, X, threads=8)
+        first = dev.gemm(X, vq.VQ_IMPL_TILE)
+        assert_outputs_close(first, Y, A, f"{spec.name} batch {batch}")
+        for _ in range(3):
+            assert np.array_equal(dev.gemm(X, vq.VQ_IMPL_TILE).view(np.uint16), first.view(np.uint16))
+    assert vq.vq_device_wait_failures() == 0
+
+
 @pytest.mark.parametrize("cb,bc", [(True, 2048), (False, 1024)])
 def test_row_tables_at_batch_8(cb, bc):
     import torch
