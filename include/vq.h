@@ -305,7 +305,7 @@ vq_status vq_assign_indices(const vq_format* fmt, const void* d_W, const void* d
  *   w[n][k] = value decoded as without normalisation * d_norm_lut[blk(n, k)][code(n, k / norm_block_cols)].
  * vq_decode_weights_normalized writes binary16(w), the exact product rounded once; vq_gemm_small_batch_normalized
  * computes Y[m][n] = sum_k w[n][k] X[m][k] (fp32 accumulation, one rounding), batch 1..16.  Every valid
- * format is taken; no workspace, plain stream-order launches: everything these two calls read (weights, codes,
+ * format is taken; no workspace; stream order alone is enough: everything these two calls read (weights, codes,
  * tables, activations) may be written by work in front of them on the same stream.  With fp16 or int8 codebooks
  * the product runs in the tcgen05 kernel (2-D 6-bit indices, blocks of a multiple of 32 rows and of 128 columns,
  * norm_block_cols 16, 32 or 64, layers of enough rows to fill the GPU with tiles of 128) or in the tuned pair-table

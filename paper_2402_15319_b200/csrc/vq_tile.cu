@@ -172,6 +172,23 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
   return p != 0;
 }
+// Weights, codes and scale tables: complete before the call, so read-only for the kernel, or (ORDERED: normalised calls) perhaps written
+// by the kernel in front, so read behind griddepcontrol.wait only and not through the read-only path.  (volatile: not moved across the wait)
+template <int BYTES, bool ORDERED>
+__device__ __forceinline__ uint32_t load_weight(const void* p) {
+  static_assert(BYTES == 1 || BYTES == 2 || BYTES == 4);
+  if constexpr (!ORDERED) {
+    if constexpr (BYTES == 1) return __ldg(static_cast<const uint8_t*>(p));
+    else if constexpr (BYTES == 2) return __ldg(static_cast<const unsigned short*>(p));
+    else return __ldg(static_cast<const uint32_t*>(p));
+  } else {
+    uint32_t v;
+    if constexpr (BYTES == 1) asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
+    else if constexpr (BYTES == 2) asm volatile("ld.global.u16 %0, [%1];" : "=r"(v) : "l"(p));
+    else asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+  }
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
@@ -370,17 +387,19 @@ struct Tables {
       load<VALS / 2>(p);
     } else if (a.cb_int8) {
       load<VALS>(p);
-      sc = __ldg(ssrc + bcol);
+      sc = load_weight<2, F::NORM>(ssrc + bcol);
     } else {
       load<VALS * 2>(p);
     }
   }
   template <int BYTES>
   __device__ __forceinline__ void load(const uint8_t* p) {
-    if constexpr (BYTES == 1) raw[0] = __ldg(p);
-    else if constexpr (BYTES == 2) raw[0] = __ldg(reinterpret_cast<const unsigned short*>(p));
-    else if constexpr (BYTES == 4) raw[0] = __ldg(reinterpret_cast<const uint32_t*>(p));
-    else if constexpr (BYTES == 8) {
+    static_assert(!F::NORM || BYTES <= 8);
+    if constexpr (BYTES <= 4) raw[0] = load_weight<BYTES, F::NORM>(p);
+    else if constexpr (F::NORM) {
+      raw[0] = load_weight<4, true>(p);
+      raw[RAW - 1] = load_weight<4, true>(p + 4);
+    } else if constexpr (BYTES == 8) {
       const uint2 v = ldg64_nc(p);
       raw[0] = v.x; raw[1] = v.y;
     } else {
@@ -528,7 +547,9 @@ __global__ void __launch_bounds__(F::THREADS, 1) tile_kernel(const __grid_consta
   const int qt = tid & 127;   // row of the tile
   int tile = f.tile, u = 0, end = 0, bcol = 0;
   bool asked = false;         // are the entries of the next block to be used on their way?
+  // A normalised call reads nothing, weights, codes and scale tables included, before all in front of it on the stream is complete.
   if (warp < kDecodeWarps) {
+    if (F::NORM) pdl_wait();
     f.range(a, quad, u, end);
     f.next(a);
     bcol = divide(u, a.block_inv) - 1;
@@ -553,8 +574,9 @@ __global__ void __launch_bounds__(F::THREADS, 1) tile_kernel(const __grid_consta
       mbar_init_fence();
     }
     __syncwarp();
+    if (F::NORM) pdl_wait();
     wi.init(a, f, quad);
-    if (wi.f.valid) request_first();   // (weights do not depend on the previous kernel)
+    if (wi.f.valid) request_first();   // (weights do not depend on the previous kernel, but for normalised calls)
   } else if (warp == kResultsWarp) {
     if (lane == 0) {
       mbar_init(red_full, kDecodeWarps);
@@ -856,7 +878,7 @@ __global__ void __launch_bounds__(F::THREADS, 1) tile_kernel(const __grid_consta
         code_word = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (i < (F::UC / 2 >> a.norm_shift)) code_word |= static_cast<uint32_t>(__ldg(p + i)) << (8 * i);
+          if (i < (F::UC / 2 >> a.norm_shift)) code_word |= load_weight<1, true>(p + i) << (8 * i);
       }
     };
 
@@ -938,7 +960,7 @@ __global__ void __launch_bounds__(F::THREADS, 1) tile_kernel(const __grid_consta
       if constexpr (F::NORM) {
         const unsigned short* l = lut + divide(u, a.block_inv) * 16;
 #pragma unroll
-        for (int i = 0; i < F::UC / 16; ++i) nscales[i] = __ldg(l + ((code_word >> (4 * (16 * i >> a.norm_shift))) & 15u)) * 0x10001u;
+        for (int i = 0; i < F::UC / 16; ++i) nscales[i] = load_weight<2, true>(l + ((code_word >> (4 * (16 * i >> a.norm_shift))) & 15u)) * 0x10001u;
         if (seg_left > 1) request_codes(u + 1);
       }
       uint32_t scales[F::STAGES / 2];   // int4 codebooks: of the unit's groups of 128 columns
@@ -1225,10 +1247,7 @@ vq_status launch(const StreamCall& call, cudaStream_t s, const Norm* norm = null
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  // A normalised call is a plain launch: its entry point promises that whatever the stream holds in front of it is complete, for codes,
-  // scale tables and weights too, which the decoding warps read without waiting, through the read-only path.  (With programmatic
-  // launch and griddepcontrol.wait in every reading warp 14336 x 4096 takes 18.9 us back to back, plainly 19.3, before 17.3.)
-  cfg.numAttrs = !norm && env_int("VQ_PDL", 1) ? 1 : 0;
+  cfg.numAttrs = env_int("VQ_PDL", 1) ? 1 : 0;
 #ifdef VQ_TUNING
   if (env_int("VQ_VERBOSE", 0)) fprintf(stderr, "tile launch: grid %d depth %d smem %zu tiles %d S %d steps %d q %d share %d+%d\n", (int)P, D, smem_bytes, tiles, a.S, a.steps, a.q, a.share, a.longer);
 #endif

@@ -1,4 +1,4 @@
-"""The normalised product is a plain launch on its stream: codes, scale table and indices may be written by kernels directly in front of
+"""The normalised product is ordered by its stream alone: codes, scale table and indices may be written by kernels directly in front of
 it, the scale table even by a product call that lets its successor start early."""
 import numpy as np
 import pytest
