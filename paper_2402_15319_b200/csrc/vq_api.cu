@@ -218,7 +218,8 @@ static int group_family(const Geometry& g, int) {
 int vq_grouped_kernel_launches(const vq_format* fmt, int n_members, int batch) {
   Geometry g;
   if (make_geometry(fmt, &g) != VQ_OK || n_members < 1 || n_members > VQ_MAX_GROUP || batch < 1 || batch > 16) return 0;
-  if (n_members > 1 && tile_preferred(g, &g.N, 1, batch)) return 1;   // (g.N: the members' rows together)
+  const int rows[VQ_MAX_GROUP] = {g.N};   // the members' rows together
+  if (n_members > 1 && tile_preferred(g, rows, n_members, batch)) return 1;
   if (n_members > 1 && blockcb_covers(g) && group_family(g, batch) == 2) return 1;
   if (n_members > 1 && group_family(g, batch) == 3) return 1;
   return (n_members > 1 && group_family(g, batch) == 1 && stream_covers(g)) ? 1 : n_members;

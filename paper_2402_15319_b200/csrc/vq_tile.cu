@@ -1265,43 +1265,85 @@ bool tile_covers(const Geometry& g) {
   return g.d == 4 && g.b == 8 && g.Bc % 128 == 0 && g.Br % kTileRows == 0 && !g.cb_int4;
 }
 
-// Which calls this kernel serves.  Its time hardly depends on the batch (one pass over the weights for 1..16 sequences); a call
-// costs about 4.5 us before and behind its look-ups, the cluster kernels' 3.3.  So it takes over above a number of weights (in
-// 2^20) that falls with the batch and with the columns (long rows give every CTA one long piece, where the cluster kernels
-// stage activations and split K over eight CTAs at most).  The lines come from 46704 timings against the other kernels on B200
-// (26 formats, 1024 to 28672 columns, 1.5 to 375 x 2^20 weights, every batch).  Mean time over the others' on either side of a line:
-//   row tables   batch 9 to 16 from 6: 0.7, below 0.9 (the worst tenth above 1.05); batch 6 to 8 from 8: 0.75; batch 3 to 5, blocks up to
-//                512 columns, from 24: 0.82, longer blocks 0.98; batch 1 and 2, 256-column blocks, from 96: 0.85, others 1.0 to 1.5
-//   others, K >= 5500: 0.45 to 0.85 at every size.  K from 3700: batch 1 to 5 from 24: 0.75, below 0.93 (1.1); 32-row blocks of 6 bits from
-//                64: 0.82, from 24 1.06; batch 6 to 16 from 8: 0.8.  K below: from 24 0.8, from 8 1.0; from batch 9 on from 8: 0.78
-//   groups whose layers the cluster kernels take in one launch: 12288 x 4096 in three layers, 128-row blocks, 6 bits, batch 1 12.7 us
-//                against 10.8, 6144 x 4096 32-row blocks 9.3/8.3; 18176 x 3328 4-bit codebooks batch 5 15.7/19.1, 15360 x 5120 4-D batch 8 16.4/18.3: from 54
-// Slower than the others remain calls with many short rows at large batches, where adding a tile's sums takes as long as decoding
-// it: 65536 x 1024 at batch 16 1.2 times, 32768 x 2048 1.1 times the time of a kernel of four CTAs per SM that this one replaced.
+// Which calls this kernel serves.  Its time hardly depends on the batch (one pass over the weights for 1..16 sequences), but a call
+// costs about 4.5 us before and behind its look-ups, the cluster kernels' 3.3.  So it takes over above a number of weights (in 2^20,
+// "line") that falls with the batch and with the columns: long rows give a CTA one long piece, where the cluster kernels stage
+// activations and split K over eight CTAs at most.  One layer and a group of as many rows are planned alike, so they share their lines; the
+// persistent kernel, which takes row tables of 8192 rows or of a group, is another rival than the cluster kernels and has lines of its own.
+// The lines are drawn from 108394 calls (24 formats, 1024 to 28672 columns, 1.5 to 320 x 2^20 weights, one layer or three, batches 1 to 16),
+// each timed here, in every other kernel, and in the library before this kernel had one CTA per SM: where nearly no call is more
+// than 3 % slower than it was then, not where the mean is lower.  820 of them are (0.8 %; of calls that one kernel serves on both sides
+// 1.4 % differ as much); together they take 0.70 of the time of then.  Both sides' times (us, others / here):
+//   128-row blocks, 6 bits  4096 x 4096 b1 5.8/6.7, b8 8.4/7.1; 12288 x 4096 b1 10.9/12.4, b8 13.6/13.1; 19712 x 5120 b16 53/22.7
+//   32-row blocks, 6 bits   6144 x 4096 b1 7.7/9.0, b16 15.0/9.8; 32768 x 1024 b1 10.9/8.8, b16 12.5/13.9
+//   4-D                     49152 x 1024 b3 10.9/11.5; 19712 x 5120 b3 25.9/15.3, b8 34.2/16.3
+//   row tables, 2048-column blocks, against the persistent kernel  8192 x 4096 b6 8.5/9.5; 8192 x 8192 b1 10.2/13.0, b9 16.5/13.9;
+//                           24576 x 8192 b1 26.4/26.5, b6 30.3/27.8, b9 38.6/28.3
+// Left: 4-D and 5 bits with 1024 to 1536 columns and 64 x 2^20 weights or more, up to 1.15 times the time of then at batch 16, in
+// every kernel there is now.
+constexpr unsigned char kNever = 255;
+constexpr int kLineCols[5] = {1500, 2600, 3700, 4800, 5500};        // columns: below the first, the second, ..., from the last on
+constexpr int kRowLineCols[5] = {1500, 2600, 4800, 5500, 10000};
+struct Lines { unsigned char at[4][6]; };      // batch 1-2, 3-5, 6-8, 9-16
+struct RowLines { unsigned char at[6][6]; };   // batch 1-2, 3-5, 6-7, 8, 9-10, 11-16
+// against the cluster kernels: blocks of 128 k rows and 6 bits, of 32 and 64 rows and 6 bits (each: 16- and 8-bit, 4-bit codebooks), 5 bits, 4-D
+constexpr Lines kTall6 = {{{128, 28, 32, 56, 64, 3}, {128, 24, 32, 56, 3, 3}, {32, 5, 20, 5, 0, 0}, {}}};
+constexpr Lines kTall6Int4 = {{{80, 24, 0, 28, 0, 0}, {56, 24, 0, 28, 0, 0}, {0, 3, 0, 0, 0, 0}, {}}};
+constexpr Lines kWarp6 = {{{80, 28, 32, 56, 0, 0}, {80, 24, 0, 28, 0, 0}, {56, 3, 0, 0, 0, 0}, {0, 0, 0, 3, 0, 0}}};
+constexpr Lines kWarp6Int4 = {{{kNever, 56, 32, 56, 64, 0}, {128, 56, 32, 56, 0, 0}, {56, 3, 0, 28, 0, 0}, {}}};
+constexpr Lines k5 = {{{12, 20, 28, 36, 3, 0}, {3, 20, 5, 5, 0, 0}, {3, 3, 3, 3, 0, 0}, {0, 3, 0, 0, 0, 0}}};
+constexpr Lines k5Int4 = {{{3, 20, 3, 36, 0, 0}, {0, 3, 3, 3, 0, 0}, {0, 3, 0, 0, 0, 0}, {0, 3, 0, 0, 0, 0}}};
+constexpr Lines k4D = {{{80, 24, 0, 0, 0, 0}, {80, 12, 0, 0, 0, 0}, {3, 3, 0, 0, 0, 0}, {}}};
+// against the pair-table kernel: blocks of 4, of 8 and 16 rows; rows or columns that the cluster kernels do not take, 5 bits and 6
+constexpr Lines kSmall4 = {{{}, {12, 0, 0, 0, 0, 0}, {12, 3, 0, 0, 0, 0}, {3, 5, 3, 0, 0, 0}}};
+constexpr Lines kSmall = {{{0, 24, 24, 20, 0, 0}, {12, 24, 24, 20, 0, 0}, {12, 24, 24, 20, 0, 0}, {12, 12, 8, 8, 0, 0}}};
+constexpr Lines kRagged5 = {{{12, 24, 20, 3, 0, 0}, {12, 24, 20, 3, 0, 0}, {12, 24, 20, 3, 0, 0}, {3, 5, 8, 3, 0, 0}}};
+constexpr Lines kRagged6 = {{{12, 12, 0, 0, 0, 0}, {12, 0, 0, 0, 0, 0}, {8, 0, 0, 0, 0, 0}, {3, 0, 0, 0, 0, 0}}};
+// row tables, blocks of 256, of up to 960 and of more columns: against the cluster kernels, against the persistent kernel
+constexpr RowLines kRows[3][2] = {
+    {{{{kNever, kNever, kNever, 24, 48, 56}, {0, 3, 20, 0, 5, 5}, {0, 3, 0, 0, 0, 0}, {}, {kNever, 0, 5, 0, 0, 0}, {}}},
+     {{{kNever, 56, 0, 0, 0, 0}, {}, {}, {}, {}, {}}}},
+    {{{{kNever, kNever, kNever, kNever, kNever, 80}, {0, kNever, 20, 24, 48, 8}, {0, 3, 20, 0, 3, 0}, {0, 3, 0, 0, 0, 0}, {0, 5, 3, 5, 0, 0}, {}}},
+     {{{kNever, kNever, kNever, kNever, kNever, kNever}, {kNever, kNever, kNever, 32, kNever, kNever}, {3, 56, 40, 0, 80, kNever},
+       {3, 20, 24, 0, 48, 160}, {0, 20, 28, 0, 0, 0}, {0, 5, 0, 0, 0, 0}}}},
+    {{{{kNever, kNever, kNever, kNever, 56, 80}, {0, kNever, 20, 24, 48, 24}, {0, 5, 5, 0, 3, 0}, {0, 3, 0, 0, 0, 0}, {0, 5, 5, 5, 5, 0},
+       {0, 5, 0, 0, 0, 0}}},
+     {{{kNever, kNever, kNever, kNever, kNever, kNever}, {kNever, kNever, kNever, kNever, kNever, kNever}, {5, 20, 40, 0, 80, kNever},
+       {0, 20, 24, 0, 56, 160}, {0, 56, 0, 0, 0, 0}, {0, 12, 0, 0, 0, 0}}}},
+};
+
 bool tile_preferred(const Geometry& g, const int* N, int n_seg, int batch) {
   if (!tile_covers(g)) return false;
 #ifdef VQ_TUNING
   if (env_int("VQ_TILE", -1) >= 0) return env_int("VQ_TILE", 0) != 0;
 #endif
   long long rows = 0;
-  bool whole = g.K % 256 == 0;
+  bool whole = blockcb_covers(g);   // do the cluster kernels take the call?
   for (int i = 0; i < n_seg; ++i) {
     rows += N[i];
     whole = whole && N[i] % kTileRows == 0;
   }
   const long long w = (rows * g.K) >> 20;   // weights of the call, in 2^20
+  auto column = [&](const int (&limits)[5]) {
+    int k = 0;
+    while (k < 5 && g.K >= limits[k]) ++k;
+    return k;
+  };
+  int line;
   if (g.d == 2 && g.b == 4) {
-    if (batch >= 6) return w >= (batch >= 9 ? 6 : 8);
-    return batch >= 3 ? g.Bc <= 512 && w >= 24 : g.Bc == 256 && w >= 96;
+    const RowLines& l = kRows[g.Bc < 512 ? 0 : g.Bc < 1024 ? 1 : 2][n_seg > 1 || rows >= 8192];
+    line = l.at[batch <= 2 ? 0 : batch <= 5 ? 1 : batch <= 7 ? 2 : batch == 8 ? 3 : batch <= 10 ? 4 : 5][column(kRowLineCols)];
+  } else {
+    const bool pairs = g.b == 5 && g.Br < 32;
+    if (!pairs && !whole && (g.d == 4 || g.cb_int4)) return true;   // (0.2 to 0.8 of the pair-table kernel's time at every size)
+    const Lines& l = pairs ? (g.Br == 4 ? kSmall4 : kSmall)
+                   : !whole ? (g.b == 5 ? kRagged5 : kRagged6)
+                   : g.d == 4 ? k4D
+                   : g.b == 5 ? (g.cb_int4 ? k5Int4 : k5)
+                   : g.Br % kTileRows == 0 ? (g.cb_int4 ? kTall6Int4 : kTall6) : (g.cb_int4 ? kWarp6Int4 : kWarp6);
+    line = l.at[batch <= 2 ? 0 : batch <= 5 ? 1 : batch <= 8 ? 2 : 3][column(kLineCols)];
   }
-  if (g.K >= 5500) return true;
-  const bool pairs = g.b == 5 && g.Br < 32;   // else: the pair-table kernel, which takes groups too
-  if (!pairs && !whole) return g.K >= 3700 || w >= (n_seg > 1 ? 4 : 16);
-  if (!pairs && n_seg > 1 && batch <= 8) return w >= 54;
-  if (g.K < 3700) return w >= (batch <= 8 || pairs ? 24 : 8);
-  if (pairs) return w >= 12;
-  if (batch >= 6) return w >= (batch <= 8 && g.b == 6 && g.Br % kTileRows != 0 ? 48 : 8);
-  return w >= (g.b == 6 && g.Br % kTileRows != 0 ? 64 : 24);
+  return line != kNever && w >= line;
 }
 
 vq_status launch_gemm_tile(const StreamCall& call, cudaStream_t s) {
