@@ -1369,13 +1369,16 @@ vq_status launch_gemm_tile_norm(const Geometry& g, const LayerPtrs& p, const voi
                                 const __half* X, __half* Y, int batch, cudaStream_t s) {
   if (!norm_codes || !norm_lut || !tile_covers(g) || g.d != 2 || g.b != 6 || g.cb_int4) return VQ_ERR_UNSUPPORTED;
   if (norm_block_cols != 16 && norm_block_cols != 32 && norm_block_cols != 64) return VQ_ERR_UNSUPPORTED;
-  // A tile is one CTA's whole: worth it where the tiles fill the SMs.  0.1 ns, fitted to both kernels' times: a round of tiles against
-  // the pair-table kernel's weights (sub-rows of 32, batch 1: 14336 x 4096 18.0 us against 23.6, 11008 x 4096 17.0/19.3, 8192 x 1024
-  // 4.0/7.7; 4096 x 4096 14.5/9.6, 19200 x 2048 15.2/17.5, which this leaves to the other; of 16, batch 4: 11008 x 4096 22.2/21.5).
+  // A tile is one CTA's whole: worth it where the tiles fill the SMs.  Both kernels' times in us, fitted to 20160 calls (six formats, 256 to
+  // 14336 columns, 480 to 57344 rows, batches 1 to 16), with a twentieth to spare: of the 8571 calls taken 109 are more than 3 % slower than
+  // in the pair-table kernel.  Sub-rows of 32, batch 1, 8-bit codebooks of 32 x 256 (pair-table kernel / here): 11008 x 4096 18.9/18.8,
+  // 14336 x 4096 24.2/19.4, 37888 x 4096 59.0/34.7, 14336 x 11008 61.3/44.3; 24576 x 1024 11.6/11.8 is left to the other.
   int sms = 0;
   if (device_sms(&sms) != VQ_OK) return VQ_ERR_CUDA;
-  const long long rounds = ((g.N + kTileRows - 1) / kTileRows + sms - 1) / sms, w = (static_cast<long long>(g.N) * g.K) >> 20;
-  if (35000 + rounds * g.K * (norm_block_cols == 16 ? 47 : 35) > 50000 + 3100 * w) return VQ_ERR_UNSUPPORTED;
+  const double rounds = ((g.N + kTileRows - 1) / kTileRows + sms - 1) / sms, cols = g.K / 1000., w = static_cast<double>(g.N) * g.K / (1 << 20);
+  const double here = 2.75 + 0.06 * batch + rounds * (1.55 + (norm_block_cols == 16 ? 4.7 : 3.9) * cols);
+  const double pairs = batch <= 8 ? 4.45 + 0.335 * w + 0.88 * cols : 4.85 + 0.41 * w + 0.88 * cols;
+  if (1.05 * here > pairs) return VQ_ERR_UNSUPPORTED;
   StreamCall call = {};
   call.g = g;
   call.n_seg = 1;

@@ -116,3 +116,47 @@ def test_normalised(spec, cols):
             assert_outputs_close(dY.cpu().numpy()[:, rows], ref, A, f"{spec.name} {cols} batch {batch}")
         assert np.isfinite(dY.float().cpu().numpy()).all()
     assert vq.vq_device_wait_failures() == 0
+
+
+def _normalised_rows(spec, L, codes, lut, cols, r0, n):
+    """Rows r0 .. r0 + n - 1 of the normalised weights, in binary64 (whole codebook blocks)."""
+    part = vq_synth.LayerSpec("part", N=n, K=spec.K, d=spec.d, b=spec.b, Br=spec.Br, Bc=spec.Bc, int8=spec.int8)
+    across = spec.K // spec.Bc
+    blocks = slice(r0 // spec.Br * across, (r0 + n) // spec.Br * across)
+    W, _ = orc.normalized_decode(oracle_fmt(part), L.idx[r0:r0 + n], L.cb.reshape(spec.n_blocks, -1)[blocks],
+                                 None if L.scale is None else L.scale[blocks], codes[r0:r0 + n], lut[blocks], cols)
+    return W.astype(np.float64)
+
+
+@pytest.mark.parametrize("spec,kernel", [
+    (_spec("warp_i8", 16384, 4096, 2, 6, 32, 256, True), "tile_kernel"),
+    (_spec("warp_fp16_odd", 18880, 3456, 2, 6, 32, 128, False), "tile_kernel"),
+    (_spec("warp64_fp16_7_units", 18944, 896, 2, 6, 64, 128, False), "tile_kernel"),
+    (_spec("cta_fp16", 16384, 4096, 2, 6, 128, 128, False), "tile_kernel"),
+    (_spec("two_tiles_a_cta", 37888, 2048, 2, 6, 256, 256, True), "tile_kernel"),
+    (_spec("one_tile_too_many", 19072, 3328, 2, 6, 64, 128, False), "warptab_kernel"),   # 149 tiles on 148 SMs
+], ids=lambda v: v.name if hasattr(v, "name") else v)
+@pytest.mark.parametrize("cols", [16, 32, 64])
+def test_normalised_in_the_kernel_it_claims(spec, kernel, cols):
+    import torch
+    L = draw(spec, 95)
+    dev = DeviceLayer(spec, L)
+    codes, lut = vq_synth.make_norm(spec, cols, seed=96)
+    dc, dl = torch.from_numpy(codes).cuda(), torch.from_numpy(lut).cuda()
+    parts = [(r0, _normalised_rows(spec, L, codes, lut, cols, r0, 512)) for r0 in (0, (spec.N - 512) // 2 // 256 * 256, spec.N - 512)]
+    for batch in (1, 8, 9, 16):
+        X = vq_synth.make_x(spec, 97, batch)
+        dX = torch.from_numpy(X).cuda()
+        dY, raw = guarded((batch, spec.N), torch.float16, "cuda")
+        torch.cuda.synchronize()
+        call = lambda: vq.vq_gemm_small_batch_normalized(dev.fmt, dev.idx, dev.cb, dev.scale, dc, dl, cols, dX, dY, batch)  # noqa: E731
+        names = kernels_launched(call)
+        assert len(names) == 1 and kernel in names[0], names
+        call()
+        torch.cuda.synchronize()
+        assert_guards_intact(raw, spec.name)
+        Y, X64 = dY.cpu().numpy(), X.astype(np.float64)
+        assert np.isfinite(Y.astype(np.float32)).all()
+        for r0, W in parts:
+            assert_outputs_close(Y[:, r0:r0 + 512], X64 @ W.T, np.abs(X64) @ np.abs(W).T, f"{spec.name} {cols} batch {batch} rows from {r0}")
+    assert vq.vq_device_wait_failures() == 0
