@@ -4,8 +4,9 @@
 // format the decode path reads.
 //
 // A CTA takes a tile of 32 rows x 256*d columns; its codebooks go to shared memory as binary32
-// (int8 entries times their block scale, exact).  A thread owns 8 consecutive vectors of a row
-// (one group of 8 indices = b whole bytes of the stream) and writes its b bytes.
+// (int8 entries times their block scale, exact).  A thread owns 8 consecutive vectors of each of its four
+// rows (a group of 8 indices = b whole bytes of the stream) and writes their b bytes; the rows are adjacent where
+// the weighted search ranks the same vector of the four together, else 8 apart.
 //
 // The decision is taken in binary32 with every operation rounded separately (no fused
 // multiply-add), terms added left to right, lowest index among equal distances: the same
@@ -481,47 +482,46 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
       if (grp == a.groups - 1)   // padding up to the row stride
         for (long long k = a.used_bytes; k < a.stride; ++k) a.idx[n * a.stride + k] = 0;
     }
-    return;
-  }
-
-  for (int r = warp; r < kRows; r += kWarps) {
-    const int n = row0 + r;
-    if (n >= a.N) break;
-    const int tb = (r / a.rows_per_br) * a.bc_per_seg + lbc;
-    const unsigned char* tab = smem + tb * table_bytes;
-    const float c_max = __int_as_float(cmax[tb]);
-    unsigned long long bits = 0;
-#pragma unroll
-    for (int v0 = 0; v0 < 8; v0 += V) {
-      float x[V][D], dw[V][D];
-      {
-        const uint4* src = reinterpret_cast<const uint4*>(a.W + static_cast<long long>(n) * a.K + col + v0 * D);
-#pragma unroll
-        for (int q = 0; q < V * D / 8; ++q) {   // V*D halves
-          const uint4 raw = __ldg(src + q);
-          const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-          for (int h = 0; h < 8; ++h) {
-            const int e = q * 8 + h;
-            const __half_raw hr = {static_cast<unsigned short>((wds[h >> 1] >> (16 * (h & 1))) & 0xffff)};
-            x[e / D][e % D] = __half2float(__half(hr));
+  } else {
+    for (int r = warp; r < kRows; r += kWarps) {
+      const int n = row0 + r;
+      if (n >= a.N) break;
+      const int tb = (r / a.rows_per_br) * a.bc_per_seg + lbc;
+      const unsigned char* tab = smem + tb * table_bytes;
+      const float c_max = __int_as_float(cmax[tb]);
+      unsigned long long bits = 0;
+  #pragma unroll
+      for (int v0 = 0; v0 < 8; v0 += V) {
+        float x[V][D], dw[V][D];
+        {
+          const uint4* src = reinterpret_cast<const uint4*>(a.W + static_cast<long long>(n) * a.K + col + v0 * D);
+  #pragma unroll
+          for (int q = 0; q < V * D / 8; ++q) {   // V*D halves
+            const uint4 raw = __ldg(src + q);
+            const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
+  #pragma unroll
+            for (int h = 0; h < 8; ++h) {
+              const int e = q * 8 + h;
+              const __half_raw hr = {static_cast<unsigned short>((wds[h >> 1] >> (16 * (h & 1))) & 0xffff)};
+              x[e / D][e % D] = __half2float(__half(hr));
+            }
           }
         }
-      }
-      if constexpr (HD) {
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-#pragma unroll
-          for (int t = 0; t < D; ++t) dw[v][t] = __ldg(a.hdiag + col + (v0 + v) * D + t);
-      }
+        if constexpr (HD) {
+  #pragma unroll
+          for (int v = 0; v < V; ++v)
+  #pragma unroll
+            for (int t = 0; t < D; ++t) dw[v][t] = __ldg(a.hdiag + col + (v0 + v) * D + t);
+        }
 
-      pick<D, HD, TOP2, false, V>(x, dw, tab, c_max, groups,
-                                  [&](int v, int index) { bits |= static_cast<unsigned long long>(index) << ((v0 + v) * a.b); });
+        pick<D, HD, TOP2, false, V>(x, dw, tab, c_max, groups,
+                                    [&](int v, int index) { bits |= static_cast<unsigned long long>(index) << ((v0 + v) * a.b); });
+      }
+      uint8_t* dst = a.idx + n * a.stride + static_cast<long long>(grp) * a.b;
+      for (int i = 0; i < a.b; ++i) dst[i] = static_cast<uint8_t>(bits >> (8 * i));
+      if (grp == a.groups - 1)   // padding up to the row stride
+        for (long long i = a.used_bytes; i < a.stride; ++i) a.idx[n * a.stride + i] = 0;
     }
-    uint8_t* dst = a.idx + n * a.stride + static_cast<long long>(grp) * a.b;
-    for (int i = 0; i < a.b; ++i) dst[i] = static_cast<uint8_t>(bits >> (8 * i));
-    if (grp == a.groups - 1)   // padding up to the row stride
-      for (long long i = a.used_bytes; i < a.stride; ++i) a.idx[n * a.stride + i] = 0;
   }
 }
 
@@ -588,7 +588,7 @@ vq_status launch_assign(const Geometry& g, const LayerPtrs& p, const __half* W, 
     if (g.d == 1) return hdiag ? launch(assign_two_pass_kernel<1, true, true>, 3, smem2) : launch(assign_two_pass_kernel<1, false, true>, 4, smem2);
     // The same columns of four rows share their weights (one row at a time / four, 4096 x 4096, us: 32 2-D entries 106/87, 64 2-D 144/120,
     // 256 2-D 413/352, 64 4-D 183/131, 256 4-D 463/359); blocks of one or two rows do not hold four rows.
-    if (hdiag && g.Br % 4 == 0 && g.d != 1) {
+    if (hdiag && g.Br % 4 == 0) {
       if (g.d == 2) return top2 ? launch(assign_two_pass_kernel<2, true, true, true>, 13, smem2) : launch(assign_two_pass_kernel<2, true, false, true>, 14, smem2);
       return top2 ? launch(assign_two_pass_kernel<4, true, true, true>, 15, smem2) : launch(assign_two_pass_kernel<4, true, false, true>, 16, smem2);
     }

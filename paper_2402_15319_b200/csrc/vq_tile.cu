@@ -164,9 +164,6 @@ __device__ __forceinline__ void tma_box_3d(uint32_t dst, const CUtensorMap* tm, 
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                ::"r"(dst), "l"(tm), "r"(c0), "r"(c1), "r"(c2), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* tm) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
-}
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
@@ -525,7 +522,7 @@ __global__ void __launch_bounds__(F::THREADS, 1) tile_kernel(const __grid_consta
   int tries = kWaitTries;
   Walk f;
   f.init(a, c);
-  Units wi;   // (service warps) the next unit whose indices are to be requested
+  Units wi = {};   // (service warps) the next unit whose indices are to be requested
   int islot = 0, first_x = 0, first_n = 0;   // the units requested first: lane i keeps the i-th
   auto request_indices = [&]() {
     if (elect_one()) {
