@@ -490,16 +490,16 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
       const unsigned char* tab = smem + tb * table_bytes;
       const float c_max = __int_as_float(cmax[tb]);
       unsigned long long bits = 0;
-  #pragma unroll
+#pragma unroll
       for (int v0 = 0; v0 < 8; v0 += V) {
         float x[V][D], dw[V][D];
         {
           const uint4* src = reinterpret_cast<const uint4*>(a.W + static_cast<long long>(n) * a.K + col + v0 * D);
-  #pragma unroll
+#pragma unroll
           for (int q = 0; q < V * D / 8; ++q) {   // V*D halves
             const uint4 raw = __ldg(src + q);
             const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
-  #pragma unroll
+#pragma unroll
             for (int h = 0; h < 8; ++h) {
               const int e = q * 8 + h;
               const __half_raw hr = {static_cast<unsigned short>((wds[h >> 1] >> (16 * (h & 1))) & 0xffff)};
@@ -508,9 +508,9 @@ __global__ void __launch_bounds__(32 * kWarps, D == 4 ? 2 : 3) assign_two_pass_k
           }
         }
         if constexpr (HD) {
-  #pragma unroll
+#pragma unroll
           for (int v = 0; v < V; ++v)
-  #pragma unroll
+#pragma unroll
             for (int t = 0; t < D; ++t) dw[v][t] = __ldg(a.hdiag + col + (v0 + v) * D + t);
         }
 
