@@ -76,10 +76,11 @@ typedef enum {
  *   d_cb    : per block 2^index_bits * vq_dim signed 4-bit integers (-8..7), two per byte, value
  *             v = entry * vq_dim + t in nibble v mod 2 (low nibble first) of byte v / 2;
  *   d_scale : binary16 [N][K/128]; w[n][k] = scale[n][k/128] * c.  K % 128 == 0.
- * vq_decode_weights decodes it with its tile kernel; the skinny GEMM runs in the tuned shared-codebook
- * kernels for 2-D formats with 5- or 6-bit indices (blocks of 32, 64 or a multiple of 128 rows and a
- * multiple of 128 columns, K a multiple of 256), for large layers and batches of 5- or 6-bit formats with
- * blocks of a multiple of 32 rows in the tcgen05 kernel, and in the pair-table kernel for the block shapes
+ * vq_decode_weights decodes it with its tile kernel; the skinny GEMM runs, for 2-D formats with 5- or 6-bit
+ * indices and blocks of a multiple of 32 rows and of 128 (5 bits: 256) columns, in the tcgen05 kernel (from 5500 columns on at
+ * nearly every size, below that from a number of weights on that falls with the batch, and always where the
+ * next ones do not take the call), in the tuned shared-codebook kernels (blocks of 32, 64 or a multiple of 128 rows,
+ * K a multiple of 256), and in the pair-table kernel for the block shapes
  * that one takes (see vq_impl); in all of them a looked-up pair is fp16(scale * c), the value
  * vq_decode_weights writes; other formats of this codebook type run in the format-generic kernel (VQ_IMPL_TUNED returns
  * VQ_ERR_UNSUPPORTED for them); vq_assign_indices does not take it. */
@@ -105,7 +106,8 @@ typedef enum {
                            layers and for groups at small batch); VQ_ERR_UNSUPPORTED if it does not cover
                            the format */
   VQ_IMPL_TILE = 4      /* the tcgen05 kernel only (the one AUTO and TUNED pick for most calls of its
-                           formats); VQ_ERR_UNSUPPORTED if it does not cover the format and batch */
+                           formats); VQ_ERR_UNSUPPORTED if it does not cover the format, and for 2-D 4-bit
+                           indices below batch 9, where only AUTO and TUNED pick it */
 } vq_impl;
 
 /* Caller-filled description of one VQ-compressed matrix (paper Sec. 2.1 notation in comments). */

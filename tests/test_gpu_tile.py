@@ -139,7 +139,7 @@ def test_tile_kernel_edges(kind):
 @pytest.mark.parametrize("rows", [75776, 75776 + 256, 2 * 75776 + 1280])
 @pytest.mark.parametrize("kind", ["row_fp16", "row4_i8", "cta6_i8", "cta_4d_fp16", "warp6_i4", "warp5_8"])
 def test_tile_kernel_whole_tiles(kind, rows):
-    """More tiles than CTAs (592 on 148 SMs): whole tiles per CTA, without tiles left over and with some (an output layer)."""
+    """More tiles than CTAs (one per SM, 148): whole tiles per CTA, without tiles left over and with some (an output layer)."""
     d, b, Br, Bc, cb = KINDS[kind]
     rows = rows // Br * Br
     _forced(_spec(kind, rows, Bc * (1 if rows < 80000 else 2), d, b, Br, Bc, cb), (11,), 67)
