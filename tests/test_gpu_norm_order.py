@@ -1,5 +1,5 @@
 """The normalised product is ordered by its stream alone: codes, scale table and indices may be written by kernels directly in front of
-it, the scale table even by a product call that lets its successor start early."""
+it, the scale table even by a product call that lets its successor start early; captured in a graph too."""
 import numpy as np
 import pytest
 
@@ -61,6 +61,16 @@ def test_reads_what_the_stream_wrote_before_it(N, K, Br, Bc, cols, kernel):
     torch.cuda.synchronize()
     for i, Y in enumerate(Ys):
         assert torch.equal(Y.view(torch.int16), want[i % V].view(torch.int16)), f"launch {i}"
+    graph = torch.cuda.CUDAGraph()   # the same row of calls captured
+    with torch.cuda.graph(graph):
+        for i, Y in enumerate(Ys):
+            step(i % V, i // V % 3, Y)
+    for replay in range(3):
+        Ys.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        for i, Y in enumerate(Ys):
+            assert torch.equal(Y.view(torch.int16), want[i % V].view(torch.int16)), f"captured launch {i}, replay {replay}"
 
     rows = np.unique(np.concatenate([np.arange(8), np.random.default_rng(7).integers(0, N, 56), np.arange(N - 8, N)])).astype(np.int32)
     for v in range(V):
